@@ -132,6 +132,7 @@ struct dg_domain {
   dg::DevBuf<float> shares32;
   dg::DevBuf<int> orient_map;   // [48][nS]: canonical subdomain row -> (actual slot, point)
   dg::DevBuf<int> orient_inv;   // [48][7][N^3]: (actual slot, point) -> canonical row or -1
+  dg::DevBuf<int4> orient_aff;  // [48][7]: the same as an affine map, row = x + y i + z j + w k
   // puncture
   dg::DevBuf<double> alpha, beta, lin64;
   dg::DevBuf<float> lin32;

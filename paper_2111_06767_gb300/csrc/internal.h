@@ -142,6 +142,10 @@ struct OpGeom {
   T Jf[3];       // face Jacobian of faces normal to d: product of the tangential h/2
   T sigma[3];    // penalty C N^2 / h_d (Eq. penalty, equal neighbours)
   T lift[3];     // 1 / (w_0 h_d): L = M^-1 ML at a face node is 2 lift[d]
+  // constants of the direction-by-direction apply (dir_apply.cuh), rounded once from double
+  T f2[3];       // J (2 / h_d)^2 / 2
+  T lam;         // 1 / (2 w_0)
+  T pen;         // 2 Jf_d (sigma_d - lift_d) / (J w_0 (2 / h_d)^2) = (C N^2 - 1 / w_0) / w_0, the same for every d
   int neumann;   // bit f: box face f (= 2 d + side) is homogeneous Neumann, else Dirichlet
 };
 
@@ -159,7 +163,7 @@ struct SubdomainOut {
   int ov = 0;                    // N_overlap
   const int* col_of_elem = nullptr;
   const int* orient = nullptr;   // orientation index per element
-  const int* inv = nullptr;      // [48][7][N^3] canonical row or -1
+  const int4* aff = nullptr;     // [48][7]: canonical row of point (i, j, k) = x + y i + z j + w k
 };
 
 // Everything one DG apply reads and writes (rS != nullptr: write into the subdomain vectors).
@@ -177,18 +181,18 @@ struct ApplyArgs {
   int ld, ov;
   const int* col_of_elem;
   const int* orient;
-  const int* inv;
+  const int4* aff;
+  // direction-by-direction kernel: brick of (1 << bsx) x (1 << bsy) x bz elements, bricks along x and y
+  int bsx, bsy, bz, nbx, nby;
 };
 
 // out = A u (+ diag * u)  or, with b != nullptr, out = b - (A u + diag * u). variant: launch shape
-// (0 chosen by grid size, 1..3 few / middle / many elements per CTA; FP32 only: 4 the N = 4
-// slice-per-thread kernel, 5 and 6 the block-of-lines kernel, 7 the N = 4 element-per-thread kernel,
-// whose bounded staging wait raises *err if it gives up; a variant that cannot serve the call runs
-// as 0).
+// (0 chosen by grid size, 1..3 few / middle / many elements per CTA, 4 the three directions side by
+// side, 7 the FP32 N = 4 element-per-thread kernel, whose bounded staging wait raises *err if it
+// gives up; a variant that cannot serve the call runs as 0).
 template <typename T>
 void launch_apply(int N, const OpGeom<T>& g, const T* D, const T* w, const T* u, const T* diag, const T* b, T* out,
                   cudaStream_t s, const SubdomainOut* so = nullptr, int variant = 0, int* err = nullptr);
-constexpr int kApplyVariants = 3;
 
 // Build explicit subdomain matrices A_S for a set of classes (column-major == row-major by symmetry).
 template <typename T>
@@ -222,6 +226,8 @@ struct CoarseArgs {
   const int* elem_of_col;    // gather of the first step when u = 0
   const int* map;
   const float* shares;       // scatter weights
+  const int* inv;            // [48][7][N^3]: canonical row of a point
+  int n_bricks;              // bricks of the residual (set by the launcher)
   float* duS;
   const float* invm;         // class inverses [class][ld][ld] (unit width)
   float alpha;               // 1 / h_x

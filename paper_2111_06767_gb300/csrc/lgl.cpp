@@ -117,7 +117,12 @@ OpGeom<T> make_geom(const int n[3], const double h[3], int N, double penalty, co
     g.Jf[d] = (T)jf;
     g.sigma[d] = (T)(penalty * (double)N * (double)N / h[d]);
     g.lift[d] = (T)(1.0 / (t.w[0] * h[d]));
+    g.f2[d] = (T)(0.5 * (h[0] * h[1] * h[2] / 8.0) * (2.0 / h[d]) * (2.0 / h[d]));
   }
+  g.lam = (T)(0.5 / t.w[0]);
+  // the penalty term is the largest of the operator and is multiplied by the rounded w_0 at the end:
+  // divided by that value, so that its weight is exact
+  g.pen = (T)((penalty * (double)N * (double)N - 1.0 / t.w[0]) / (double)(T)t.w[0]);
   return g;
 }
 

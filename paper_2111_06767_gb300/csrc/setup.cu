@@ -321,8 +321,25 @@ void build_orientation_tables(dg_domain* dom) {
         inv[((size_t)o * 7 + slot) * N3 + p] = q;
       }
     }
+  // per orientation and slot the row is affine in (i, j, k) over the points the slot covers
+  std::vector<int4> aff(48 * 7);
+  for (int os = 0; os < 48 * 7; ++os) {
+    const int* row = &inv[(size_t)os * N3];
+    int p0 = 0;
+    while (row[p0] < 0) ++p0;
+    const int step[3] = {1, N, N2};
+    const int c0[3] = {p0 % N, (p0 / N) % N, p0 / N2};
+    int s[3];
+    for (int d = 0; d < 3; ++d)  // a slot one layer deep has no second point along its normal
+      s[d] = c0[d] + 1 < N && row[p0 + step[d]] >= 0 ? row[p0 + step[d]] - row[p0] : 0;
+    aff[os] = make_int4(row[p0] - s[0] * c0[0] - s[1] * c0[1] - s[2] * c0[2], s[0], s[1], s[2]);
+    for (int p = 0; p < N3; ++p)
+      DG_REQUIRE(row[p] < 0 || row[p] == aff[os].x + s[0] * (p % N) + s[1] * ((p / N) % N) + s[2] * (p / N2),
+                 "subdomain rows are not affine in the point indices");
+  }
   upload(dom->orient_map, map, dom->stream);
   upload(dom->orient_inv, inv, dom->stream);
+  upload(dom->orient_aff, aff, dom->stream);
 }
 
 // Schwarz weight shares of every point for the 64 patterns of existing face neighbours.
@@ -713,7 +730,7 @@ size_t domain_device_bytes(const dg_domain* dom) {
              dom->lin64.bytes() + dom->lin32.bytes() + dom->V.bytes() + dom->Zb.bytes() + dom->w.bytes() +
              dom->r.bytes() + dom->du.bytes() + dom->ut.bytes() + dom->rt.bytes() + dom->tmp.bytes() +
              dom->partial.bytes() + dom->dots.bytes() + dom->vin32.bytes() + dom->shares64.bytes() +
-             dom->shares32.bytes() + dom->orient_map.bytes() + dom->orient_inv.bytes() + dom->vin64.bytes() +
+             dom->shares32.bytes() + dom->orient_map.bytes() + dom->orient_inv.bytes() + dom->orient_aff.bytes() + dom->vin64.bytes() +
              dom->vout64.bytes() + dom->err_flag.bytes();
   for (const auto& L : dom->levels) {
     const auto& sw = L.sw;

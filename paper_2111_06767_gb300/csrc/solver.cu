@@ -27,16 +27,9 @@ template <typename T>
 int apply_variant(dg_domain* dom, Level& L, bool fused, const std::function<void(int)>& run, cudaStream_t s) {
   int& v = L.apply_variant[sizeof(T) == 4][fused];
   if (v < 0) {
-    // launch shapes of the line kernel; the plane kernel for plain FP32 applies at N = 4
-    std::vector<int> cand{0, 1, 2, 3};
-    if (!fused && dom->N == 4 && sizeof(T) == 4) {  // the slice kernel and the element kernel
-      cand.push_back(4);
-      cand.push_back(7);
-    }
-    if (dom->N >= 4 && sizeof(T) == 4) {  // the block-of-lines kernel, two launch shapes
-      cand.push_back(5);
-      cand.push_back(6);
-    }
+    // the direction kernel's launch shapes, and at N = 4 the element kernel for plain FP32 applies
+    std::vector<int> cand{0, 1, 2, 3, 4};
+    if (!fused && dom->N == 4 && sizeof(T) == 4) cand.push_back(7);
     // DG_APPLY_VARIANT=v pins one candidate (tests of each launch shape)
     static const int forced = [] {
       const char* e = std::getenv("DG_APPLY_VARIANT");
@@ -314,7 +307,8 @@ void schwarz_smooth(dg_domain* dom, int level, const T* b, T* u, int iterations,
       CoarseArgs a{};
       const float* diag = (level == 0 && dom->lin_set && dom->lin32.get()) ? dom->lin32.get() : nullptr;
       a.ap = ApplyArgs<float>{L.g32, dom->D32.get(), dom->w32.get(), u, diag, b, nullptr, L.E, W.rS.get(), sw.ld,
-                              dom->desc.overlap, sw.col_of_elem.get(), sw.xform_of_elem.get(), dom->orient_inv.get()};
+                              dom->desc.overlap, sw.col_of_elem.get(), sw.xform_of_elem.get(), dom->orient_aff.get()};
+      a.inv = dom->orient_inv.get();
       a.sg = sw.geom;
       a.elem_of_col = sw.elem_of_col.get();
       a.map = dom->orient_map.get();
@@ -343,7 +337,7 @@ void schwarz_smooth(dg_domain* dom, int level, const T* b, T* u, int iterations,
   so.ov = dom->desc.overlap;
   so.col_of_elem = sw.col_of_elem.get();
   so.orient = sw.xform_of_elem.get();
-  so.inv = dom->orient_inv.get();
+  so.aff = dom->orient_aff.get();
   for (int it = 0; it < iterations; ++it) {
     const double sz = sizeof(T), vec = (double)L.E * sw.nS * sz;
     const int ld = sw.ld;
