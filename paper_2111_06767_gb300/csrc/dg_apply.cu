@@ -19,9 +19,6 @@
 // Kernels: apply_dir_kernel and apply_par_kernel (dir_apply.cuh) for every order, precision and
 // output; apply_elem4_kernel for the plain FP32 apply at N = 4; coarse_smooth_kernel, which runs
 // the apply inside a fused smoother.
-#include <cuda.h>
-#include <cudaTypedefs.h>
-
 #include <algorithm>
 #include <mutex>
 #include <set>
@@ -33,6 +30,7 @@
 #include "lines.cuh"
 #include "pdl.cuh"
 #include "schwarz_dev.cuh"
+#include "tcgen05.cuh"
 
 namespace dg {
 
@@ -110,26 +108,6 @@ struct E4Shape {
   static_assert(BX <= 254 && BY <= 254 && BZ <= 254, "TMA boxes are at most 256 elements per dimension");
 };
 
-constexpr uint32_t kE4WaitPolls = 1u << 20;  // polls before the staging wait gives up
-
-__device__ __forceinline__ uint32_t e4_smem(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
-__device__ __forceinline__ bool e4_wait(uint32_t bar, int* err) {
-  for (uint32_t it = 0; it < kE4WaitPolls; ++it) {
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred P1;\n\t"
-        "mbarrier.try_wait.parity.shared::cta.b64 P1, [%1], 0;\n\t"
-        "selp.u32 %0, 1, 0, P1;\n\t}"
-        : "=r"(ok)
-        : "r"(bar)
-        : "memory");
-    if (ok) return true;
-  }
-  if (err) atomicExch(err, 1);
-  return false;
-}
-
 __device__ __forceinline__ void ld4p(const float* p, float2 (&r)[2]) {
   const float4 v = *reinterpret_cast<const float4*>(p);
   r[0] = make_float2(v.x, v.y);
@@ -193,8 +171,8 @@ __global__ void __launch_bounds__(BX* BY* BZ, E4Shape<BX, BY, BZ>::PER_SM)
   extern __shared__ __align__(128) unsigned char e4_raw[];
   // 128-byte aligned for TMA; offset from the shared array itself, so that the compiler keeps
   // every access in the shared window (LDS/STS rather than generic loads)
-  float* sm = reinterpret_cast<float*>(e4_raw + ((128u - (e4_smem(e4_raw) & 127u)) & 127u));
-  const uint32_t bar = e4_smem(sm + S::IN_WORDS);
+  float* sm = reinterpret_cast<float*>(e4_raw + ((128u - (smem_u32(e4_raw) & 127u)) & 127u));
+  const uint32_t bar = smem_u32(sm + S::IN_WORDS);
   const OpGeom<float>& g = A.g;
   const int tid = threadIdx.x;
   const int tx = tid % BX, ty = (tid / BX) % BY, tz = tid / (BX * BY);
@@ -215,12 +193,12 @@ __global__ void __launch_bounds__(BX* BY* BZ, E4Shape<BX, BY, BZ>::PER_SM)
                  : "memory");
     asm volatile(
         "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, "
-        "%5}], [%6];" ::"r"(e4_smem(sm)),
+        "%5}], [%6];" ::"r"(smem_u32(sm)),
         "l"(&mu), "r"(0), "r"(x0 - 1), "r"(y0 - 1), "r"(z0 - 1), "r"(bar)
         : "memory");
   }
-  if (!__syncthreads_and(e4_wait(bar, err))) {
-    if (tid == 0) e4_wait(bar, err);  // let the copy land (bounded) before the CTA leaves
+  if (!__syncthreads_and(mbar_wait(bar, 0, err))) {
+    if (tid == 0) mbar_wait(bar, 0, err);  // let the copy land (bounded) before the CTA leaves
     __syncthreads();
     return;
   }
@@ -455,7 +433,7 @@ __global__ void __launch_bounds__(BX* BY* BZ, E4Shape<BX, BY, BZ>::PER_SM)
   __syncthreads();
   if (tid == 0) {
     asm volatile("cp.async.bulk.tensor.4d.global.shared::cta.tile.bulk_group [%0, {%1, %2, %3, %4}], [%5];" ::"l"(&mo),
-                 "r"(0), "r"(x0), "r"(y0), "r"(z0), "r"(e4_smem(sm))
+                 "r"(0), "r"(x0), "r"(y0), "r"(z0), "r"(smem_u32(sm))
                  : "memory");
     asm volatile("cp.async.bulk.commit_group;" ::: "memory");
     asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
@@ -465,23 +443,8 @@ __global__ void __launch_bounds__(BX* BY* BZ, E4Shape<BX, BY, BZ>::PER_SM)
 // Tensor maps of the element-per-thread apply: u (or the result) as a 4-D tensor [nz][ny][nx][64]
 // read or written in boxes of (BX, BY, BZ) elements of 68 words (the 4 words past an element are
 // outside the tensor: zeros on loads, not written on stores). No swizzle.
-PFN_cuTensorMapEncodeTiled_v12000 e4_encode_fn() {
-  static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
-  static std::once_flag once;
-  std::call_once(once, [] {
-    void* p = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) == cudaSuccess &&
-        q == cudaDriverEntryPointSuccess)
-      fn = (PFN_cuTensorMapEncodeTiled_v12000)p;
-    else
-      (void)cudaGetLastError();
-  });
-  return fn;
-}
-
 bool e4_map(CUtensorMap* m, const float* base, int nx, int ny, int nz, int bx, int by, int bz) {
-  auto fn = e4_encode_fn();
+  auto fn = tensor_map_encoder();
   if (!fn) return false;
   const cuuint64_t dims[4] = {64, (cuuint64_t)nx, (cuuint64_t)ny, (cuuint64_t)nz};
   const cuuint64_t strides[3] = {256, 256ull * nx, 256ull * nx * ny};
@@ -863,6 +826,14 @@ void launch_apply(int N, const OpGeom<T>& g, const T* D, const T* w, const T* u,
     default: fail(DG_ERR_INVALID_ARG, "unsupported N");
   }
   DG_LAUNCHED(1);
+}
+
+int apply_bricks(int N, int variant, int E) {
+  constexpr int m[] = {DirEpb<2>::m, DirEpb<3>::m, DirEpb<4>::m, DirEpb<5>::m, DirEpb<6>::m, DirEpb<7>::m,
+                       DirEpb<8>::m, DirEpb<9>::m, DirEpb<10>::m};
+  constexpr int l[] = {DirEpb<2>::l, DirEpb<3>::l, DirEpb<4>::l, DirEpb<5>::l, DirEpb<6>::l, DirEpb<7>::l,
+                       DirEpb<8>::l, DirEpb<9>::l, DirEpb<10>::l};
+  return E / (variant == 2 ? m : l)[N - 2];
 }
 
 template void launch_apply<double>(int, const OpGeom<double>&, const double*, const double*, const double*,

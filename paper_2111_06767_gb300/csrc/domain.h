@@ -43,6 +43,15 @@ struct SchwarzLevel {
   int n_tiles_tc128 = 0;
   DevBuf<int4> tiles_tc256;        // tensor-core GEMM tiles: 128 rows x 256 columns (one read of a
   int n_tiles_tc256 = 0;           //   128-row slab of the inverse per class of at most 256 columns)
+  // FP64 domains on the tensor cores: digit slices of the scaled inverses [class][8][ld][ld] with their
+  // row and equilibration exponents [class][ld], tiles of 128 rows x 16..48 columns, K chunks of 64, and the slices of r_S
+  bool f64_tc = false;
+  DevBuf<uint16_t> inv_digits, x_digits;
+  DevBuf<int> inv_row_exp, inv_hexp, x_exp;
+  F64Maps f64_maps;
+  DevBuf<int4> tiles_f64;
+  int n_tiles_f64 = 0;
+  DevBuf<int> kchunks64;
   DevBuf<int4> units;              // fused coarse smoother GEMM units: 16 rows x all columns of a class
   int n_units = 0;
   DevBuf<unsigned> bar;            // fused coarse smoother barrier state
@@ -76,6 +85,7 @@ struct Level {
   int apply_variant[2][2] = {{-1, -1}, {-1, -1}};
   int gemm_split = -1;
   int simt_split[2] = {-1, -1};
+  int f64_split = -1;
 };
 
 // Event-based per-phase timing of launches (dg_profile_*).

@@ -1,6 +1,7 @@
 // Internal declarations of the GB300 DG elliptic library (not part of the C ABI).
 #pragma once
 
+#include <cuda.h>
 #include <cuda_runtime.h>
 
 #include <cstdint>
@@ -190,6 +191,7 @@ struct ApplyArgs {
 // (0 chosen by grid size, 1..3 few / middle / many elements per CTA, 4 the three directions side by
 // side, 7 the FP32 N = 4 element-per-thread kernel, whose bounded staging wait raises *err if it
 // gives up; a variant that cannot serve the call runs as 0).
+int apply_bricks(int N, int variant, int E);  // full bricks of E elements in shape 2 or 3
 template <typename T>
 void launch_apply(int N, const OpGeom<T>& g, const T* D, const T* w, const T* u, const T* diag, const T* b, T* out,
                   cudaStream_t s, const SubdomainOut* so = nullptr, int variant = 0, int* err = nullptr);
@@ -253,6 +255,24 @@ void launch_class_gemm_tc(const float* inv, int n_classes, const float* X, float
                           cudaStream_t s, int split = 0, int bn = 64);
 // Splits the tensor-core GEMM accepts for this shape (each CTA keeps >= 4 K chunks).
 std::vector<int> tc_gemm_splits(int ld);
+
+// FP64 class GEMM on the tensor cores from digit slices (f64_gemm.cu): the digits of alpha times the
+// inverses [class][8][ld][ld] (BF16), their row exponents and equilibration exponents [class][ld]; the
+// digits [8][column][ld] and exponents of the columns of X.
+void launch_f64_inverse_digits(const double* inv, double alpha, int n_classes, int ld, int* hexp, uint16_t* dst,
+                               int* row_exp, cudaStream_t s);
+void launch_f64_column_digits(const double* X, int n_cols, int ld, const int* hexp, const int* class_of_col,
+                              uint16_t* dst, int* col_exp, cudaStream_t s);
+// Tensor maps of a level's digit buffers, encoded once with them: the inverses' (128 x 64 boxes of one
+// digit) and the columns' (16, 32 and 48 columns of every digit).
+struct F64Maps {
+  CUtensorMap a, x[3];
+};
+void make_f64_maps(F64Maps& m, const uint16_t* inv, int n_classes, const uint16_t* X, int n_cols, int ld);
+// Tiles: 128 rows x 16 (width code + 1) columns; d_kchunks as above for chunks of 64, (ld + 63) / 64 + 1
+// ints per class; split as above.
+void launch_f64_gemm(const F64Maps& maps, const int* inv_exp, const int* x_exp, double* Y, int ld,
+                     const int4* d_tiles, int n_tiles, const int* d_kchunks, int* err, cudaStream_t s, int split = 0);
 
 // Launch-shape autotuning: the first time a kernel shape (key) is seen in the process, time each
 // candidate (run(c) launches it once on stream s) and keep the fastest; later calls return the

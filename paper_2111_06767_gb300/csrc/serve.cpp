@@ -299,6 +299,10 @@ dg_status elliptic_serve_submit(dg_server* srv, const dg_request* req, uint64_t*
   Job* job = new (std::nothrow) Job();
   if (!job) return DG_ERR_OOM;
   job->req = *req;
+  // FP64 domains of the pool keep the CUDA-core product: requests are admitted, and idle domains kept,
+  // by footprint, and the tensor-core product's digit slices take twice the bytes of the inverses
+  if (d.precision == DG_PRECISION_FP64 && d.subdomain_gemm == DG_GEMM_DEFAULT)
+    job->req.domain.subdomain_gemm = DG_GEMM_SIMT;
   job->bytes = bytes;
   if (d.problem == DG_PROBLEM_POISSON) {
     const size_t ndof = (size_t)d.n[0] * d.n[1] * d.n[2] * d.N * d.N * d.N;

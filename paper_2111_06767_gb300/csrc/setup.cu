@@ -226,15 +226,15 @@ void classify_schwarz(dg_domain* dom, Level& L) {
     sw.alg_vec += m * n;
     sw.alg_mac += m * n * n;
   }
-  for (int bk : {16, 32}) {
-    const int per = sw.ld / bk + 1, nck = dom->curved ? 0 : nc;  // curved levels use no class GEMM
+  for (int bk : {16, 32, 64}) {
+    const int nk = (sw.ld + bk - 1) / bk, per = nk + 1, nck = dom->curved ? 0 : nc;  // curved levels use no class GEMM
     std::vector<int> kc((size_t)nck * per, 0);
     for (int c = 0; c < nck; ++c) {
       int* k = &kc[(size_t)c * per];
-      for (int q = 0; q < sw.ld / bk; ++q)
+      for (int q = 0; q < nk; ++q)
         if (present(c, q * bk, (q + 1) * bk)) k[1 + k[0]++] = q;
     }
-    upload(bk == 16 ? sw.kchunks16 : sw.kchunks32, kc, s);
+    upload(bk == 16 ? sw.kchunks16 : (bk == 32 ? sw.kchunks32 : sw.kchunks64), kc, s);
   }
   auto tile = [&](int c, int r0, int rows, int c0, int wcode) {
     const int zero = present(c, r0, std::min(r0 + rows, sw.ld)) ? 0 : 1;
@@ -252,6 +252,15 @@ void classify_schwarz(dg_domain* dom, Level& L) {
       }
   sw.n_tiles = (int)tiles.size();
   upload(sw.tiles, tiles, s);
+  // FP64 tensor-core tiles: a class's columns in equal parts of at most 48, rounded up to 16
+  std::vector<int4> tiles_f64;
+  for (int c = 0; c < (dom->curved || dom->mixed ? 0 : nc); ++c) {
+    const int parts = (sw.class_count[c] + 47) / 48, w = ((sw.class_count[c] + parts - 1) / parts + 15) / 16 * 16;
+    for (int r0 = 0; r0 < sw.ld; r0 += 128)
+      for (int c0 = 0; c0 < sw.class_count[c]; c0 += w) tiles_f64.push_back(tile(c, r0, 128, c0, w / 16 - 1));
+  }
+  sw.n_tiles_f64 = (int)tiles_f64.size();
+  upload(sw.tiles_f64, tiles_f64, s);
   std::vector<int4> tiles_tc;
   for (int c = 0; c < (dom->curved ? 0 : nc); ++c)
     for (int r0 = 0; r0 < sw.ld; r0 += 128)
@@ -716,8 +725,39 @@ void ensure_schwarz(dg_domain* dom, int level) {
     }
     DG_CUDA(cudaStreamSynchronize(s));
   }
-  if (dom->mixed) alloc_work(L.w32, L, s);
-  else alloc_work(L.w64, L, s);
+  if (dom->mixed) {
+    alloc_work(L.w32, L, s);
+  } else {
+    alloc_work(L.w64, L, s);
+    // Tensor cores except where one or two small subdomains leave the CUDA-core product shorter than
+    // the slicing and the longer kernel (three steps: 1 element at N = 4 61 against 76 us, 2 elements 70
+    // against 76, 1 element at N = 5 78 against 79; 1 at N = 6 83 against 83, at N = 8 126 against 107),
+    // or where the digits (twice the bytes of the inverses) would take more than 8 GiB.
+    sw.f64_tc = dom->desc.subdomain_gemm == DG_GEMM_DEFAULT && tc_gemm_available() && (int64_t)L.E * ld > 512 &&
+                (size_t)16 * nc * ld * ld <= ((size_t)8 << 30);
+    if (sw.f64_tc) {
+      try {
+        sw.inv_digits.alloc((size_t)8 * nc * ld * ld);
+        sw.inv_row_exp.alloc((size_t)nc * ld);
+        sw.inv_hexp.alloc((size_t)nc * ld);
+        sw.x_digits.alloc((size_t)8 * L.E * ld);
+        sw.x_exp.alloc(L.E);
+      } catch (const Error& err) {
+        if (err.status != DG_ERR_OOM) throw;
+        sw.f64_tc = false;  // what fits without the digits still runs, on the CUDA cores
+      }
+      if (sw.f64_tc) {
+        launch_f64_inverse_digits(sw.inv64.get(), sw.inv_scale, nc, ld, sw.inv_hexp.get(), sw.inv_digits.get(),
+                                  sw.inv_row_exp.get(), s);
+        make_f64_maps(sw.f64_maps, sw.inv_digits.get(), nc, sw.x_digits.get(), L.E, ld);
+        DG_CUDA(cudaStreamSynchronize(s));
+        sw.inv64.release();
+      } else {
+        for (auto* p : {&sw.inv_digits, &sw.x_digits}) p->release();
+        for (auto* p : {&sw.inv_row_exp, &sw.inv_hexp, &sw.x_exp}) p->release();
+      }
+    }
+  }
   DG_CUDA(cudaStreamSynchronize(s));
   sw.built = true;
   dom->bytes = domain_device_bytes(dom);
@@ -740,7 +780,8 @@ size_t domain_device_bytes(const dg_domain* dom) {
          sw.inv64.bytes() +
          sw.inv32.bytes() + sw.inv16.bytes() + sw.inv16_scale.bytes() + sw.tiles.bytes() + sw.tiles_tc.bytes() +
          sw.tiles_tc128.bytes() + sw.tiles_tc256.bytes() +
-         sw.units.bytes() + sw.bar.bytes();
+         sw.units.bytes() + sw.bar.bytes() + sw.inv_digits.bytes() + sw.inv_row_exp.bytes() + sw.x_digits.bytes() +
+         sw.x_exp.bytes() + sw.inv_hexp.bytes() + sw.tiles_f64.bytes();
     for (auto* p : {&L.w64.b, &L.w64.u, &L.w64.r, &L.w64.rS, &L.w64.duS, &L.w64.gV, &L.w64.gZ, &L.w64.gW, &L.w64.gD,
                     &L.w64.gH, &L.w64.linA, &L.w64.linv})
       b += p->bytes();

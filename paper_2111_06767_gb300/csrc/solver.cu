@@ -28,7 +28,11 @@ int apply_variant(dg_domain* dom, Level& L, bool fused, const std::function<void
   int& v = L.apply_variant[sizeof(T) == 4][fused];
   if (v < 0) {
     // the direction kernel's launch shapes, and at N = 4 the element kernel for plain FP32 applies
-    std::vector<int> cand{0, 1, 2, 3, 4};
+    // (shapes 2 and 3 only where their bricks can fill half the SMs; the tuner's few short launches
+    // are too noisy to be trusted with shapes that leave the GPU idle)
+    std::vector<int> cand{0, 1, 4};
+    for (int v : {2, 3})
+      if (apply_bricks(dom->N, v, L.E) >= 76) cand.push_back(v);
     if (!fused && dom->N == 4 && sizeof(T) == 4) cand.push_back(7);
     // DG_APPLY_VARIANT=v pins one candidate (tests of each launch shape)
     static const int forced = [] {
@@ -227,6 +231,29 @@ void class_gemm<double>(dg_domain* dom, Level& L, const double* X, double* Y, cu
     launch_lin_gemv<double>(sw.inv64.get(), X, sw.nS, sw.ld, L.E, Y, s);
     return;
   }
+  if (sw.f64_tc) {
+    launch_f64_column_digits(X, L.E, sw.ld, sw.inv_hexp.get(), sw.class_of_col.get(), sw.x_digits.get(),
+                             sw.x_exp.get(), s);
+    auto run = [&](int split) {
+      launch_f64_gemm(sw.f64_maps, sw.inv_row_exp.get(), sw.x_exp.get(), Y, sw.ld, sw.tiles_f64.get(),
+                      sw.n_tiles_f64, sw.kchunks64.get(), dom->err_flag.get(), s, split);
+    };
+    if (L.f64_split < 0) {  // the K split, tuned per level on first use
+      std::vector<int> cand{0, 1};
+      for (int sp = 2; sp <= 8; sp *= 2)
+        if ((sw.ld + 63) / 64 >= sp) cand.push_back(sp);
+      const int pick = autotune({5, sw.n_classes, sw.ld, sw.n_tiles_f64, L.E}, cand, run, s);
+      cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+      DG_CUDA(cudaStreamIsCapturing(s, &cap));
+      if (cap != cudaStreamCaptureStatusNone) {
+        run(pick);
+        return;
+      }
+      L.f64_split = pick;
+    }
+    run(L.f64_split);
+    return;
+  }
   simt_class_gemm<double>(L, sw.inv64.get(), X, Y, sw.inv_scale, s);
 }
 template <>
@@ -295,7 +322,7 @@ void schwarz_smooth(dg_domain* dom, int level, const T* b, T* u, int iterations,
   Level& L = dom->levels[level];
   LevelWork<T>& W = work<T>(L);
   SchwarzLevel& sw = L.sw;
-  DG_REQUIRE((inverses<T>(sw) != nullptr || (sizeof(T) == 4 && sw.inv16.get())) && shares<T>(dom) != nullptr,
+  DG_REQUIRE((inverses<T>(sw) != nullptr || (sizeof(T) == 4 && sw.inv16.get()) || (sizeof(T) == 8 && sw.f64_tc)) && shares<T>(dom) != nullptr,
              "Schwarz data of this precision are not built for this domain");
   if (iterations <= 0) return;
   const bool linearized_level = linearized_smoother<T>(dom, level);
