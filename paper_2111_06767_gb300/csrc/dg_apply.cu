@@ -581,8 +581,7 @@ void launch_apply_n(const OpGeom<T>& g, const T* D, const T* w, const T* u, cons
   DG_REQUIRE(!(((uintptr_t)u | (uintptr_t)diag | (uintptr_t)b | (uintptr_t)out | (uintptr_t)so.rS) & a),
              "DG apply vectors must be aligned to " + std::to_string(a + 1) + " bytes");
   using DE = DirEpb<N>;
-  const ApplyArgs<T> A{g, D, w, u, diag, b, out, E, static_cast<T*>(so.rS), so.ld, so.ov, so.col_of_elem, so.orient,
-                       so.aff};
+  const ApplyArgs<T> A{g, D, w, u, diag, b, out, E, static_cast<T*>(so.rS), so.ld, so.ov, so.rec};
   if constexpr (N == 4 && std::is_same<T, float>::value) {
     if (variant == 7 && !so.rS && launch_elem4<8, 4, 4>(A, err, s)) return;
   }
@@ -698,14 +697,15 @@ __global__ void __launch_bounds__(EPB* N* N) coarse_smooth_kernel(const CoarseAr
   // a wait of an earlier launch gave up and the host has not read the flag yet: skip the work
   // (its inputs are incomplete) instead of waiting again
   if (*reinterpret_cast<volatile int*>(a.err) != 0) return;
+  constexpr int N3 = N * N * N;
   extern __shared__ __align__(16) float coarse_smem[];
   const unsigned G = gridDim.x + (unsigned)a.stall;
   const int E = a.ap.E;
   const int nblk = a.n_bricks;
   for (int it = 0; it < a.iterations; ++it) {
     if (it == 0 && a.u_zero) {
-      for (int col = blockIdx.x; col < E; col += gridDim.x)
-        gather_column<float, false>(a.sg, a.ap.b, a.elem_of_col, a.ap.orient, a.map, a.ap.rS, col);
+      for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < E * N3; t += gridDim.x * blockDim.x)
+        gather_point<N, float>(a.sg, a.ap.rec, __ldg(a.ap.b + t), a.ap.rS, t / N3, t % N3);
     } else {
       for (int blk = blockIdx.x; blk < nblk; blk += gridDim.x) {
         __syncthreads();  // the previous group is done with the shared blocks
@@ -716,9 +716,19 @@ __global__ void __launch_bounds__(EPB* N* N) coarse_smooth_kernel(const CoarseAr
     for (int un = blockIdx.x; un < a.n_units; un += gridDim.x)
       coarse_gemm_unit(a.invm, a.sg.ld, a.ap.rS, a.duS, a.units[un], a.alpha);
     if (!grid_barrier(a.bar, G, a.err)) return;
-    for (int e = blockIdx.x; e < E; e += gridDim.x)
-      scatter_element<float, float, false, true>(a.sg, a.duS, a.ap.col_of_elem, a.ap.orient, a.inv, a.shares,
-                                                 const_cast<float*>(a.ap.u), e);
+    // du_S and u were written by other CTAs of this kernel: read through L2 only
+    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < E * N3; t += gridDim.x * blockDim.x) {
+      int64_t idx[7];
+      int col[7];
+      float w[7];
+      scatter_look_up<N, float>(a.sg, a.ap.rec, a.shares, t / N3, t % N3, idx, col, w);
+      float acc = 0.0f;
+#pragma unroll
+      for (int sl = 0; sl < 7; ++sl)
+        if (idx[sl] >= 0) acc += w[sl] * __ldcg(a.duS + idx[sl]);
+      float* up = const_cast<float*>(a.ap.u) + t;
+      *up = __ldcg(up) + acc;
+    }
     if (it + 1 < a.iterations && !grid_barrier(a.bar, G, a.err)) return;
   }
 }

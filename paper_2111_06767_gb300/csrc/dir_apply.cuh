@@ -31,6 +31,7 @@
 #include "internal.h"
 #include "lines.cuh"
 #include "pdl.cuh"
+#include "schwarz_dev.cuh"
 
 namespace dg {
 
@@ -164,8 +165,7 @@ __device__ __forceinline__ void apply_dir_block(const ApplyArgs<T>& A, int blk, 
   T* su = sm;                    // the element
   T* sa = sm + EPB * R;          // sum over directions
   T* sx = sm + 2 * EPB * R;      // [direction][side][value, 2 x derivative][element][N^2]
-  __shared__ int s_col[EPB][7];
-  __shared__ int4 s_aff[EPB][7];
+  __shared__ int4 s_rec[EPB][7];  // subdomain records of the brick's elements
   if constexpr (PDL) pdl_launch_dependents();
   const OpGeom<T>& g = A.g;
   const T* __restrict__ u = A.u;
@@ -187,24 +187,11 @@ __device__ __forceinline__ void apply_dir_block(const ApplyArgs<T>& A, int blk, 
   in[4] = lz > 0; in[5] = lz + 1 < A.bz && has[5];
   if (A.rS) {
     for (int q = tid; q < EPB * 7; q += S::THREADS) {
-      const int el2 = q / 7, sl = q - el2 * 7;
-      int c3[3] = {(bx0 << A.bsx) + (el2 & ((1 << A.bsx) - 1)), (by0 << A.bsy) + ((el2 >> sx_) & ((1 << A.bsy) - 1)),
-                   bz0 * A.bz + (el2 >> sy_)};
-      bool ok = (el2 >> sy_) < A.bz && c3[0] < nx && c3[1] < ny && c3[2] < g.nz;
-      if (sl > 0) {
-        const int f = sl - 1, d = f >> 1, nd = d == 0 ? nx : (d == 1 ? ny : g.nz);
-        c3[d] += (f & 1) ? 1 : -1;
-        ok = ok && c3[d] >= 0 && c3[d] < nd;
-      }
-      int c = -1;
-      int4 af = make_int4(0, 0, 0, 0);
-      if (ok) {
-        const int r = c3[0] + nx * (c3[1] + ny * c3[2]);
-        c = A.col_of_elem[r];
-        af = A.aff[A.orient[r] * 7 + (sl == 0 ? 0 : 1 + ((sl - 1) ^ 1))];
-      }
-      s_col[el2][sl] = c;
-      s_aff[el2][sl] = af;
+      const int el2 = q / 7;
+      const int c0 = (bx0 << A.bsx) + (el2 & ((1 << A.bsx) - 1)), c1 = (by0 << A.bsy) + ((el2 >> sx_) & ((1 << A.bsy) - 1)),
+                c2 = bz0 * A.bz + (el2 >> sy_);
+      if ((el2 >> sy_) < A.bz && c0 < nx && c1 < ny && c2 < g.nz)
+        s_rec[el2][q - el2 * 7] = __ldg(A.rec + (int64_t)(c0 + nx * (c1 + ny * c2)) * 7 + (q - el2 * 7));
     }
   }
   const T wa = __ldg(A.w + t0) * __ldg(A.w + t1);
@@ -333,26 +320,20 @@ __device__ __forceinline__ void apply_dir_block(const ApplyArgs<T>& A, int blk, 
     for (int l = 0; l < N; ++l) A.out[base + l * N2] = acc[l];
     return;
   }
-  // Straight into the subdomain vectors: the element's own subdomain (slot 0) and, for points within
-  // the overlap layers of a face, that neighbour's subdomain (slot 1 + (f ^ 1)). The row of a point
-  // is affine in its indices for each slot and orientation, so no table is read per point; every
-  // row holds one point, so the stores never collide.
+  // Straight into the subdomain vectors that contain the point; every row holds one point, so the stores
+  // never collide.
 #pragma unroll
   for (int sl = 0; sl < 7; ++sl) {
-    const int c = s_col[el][sl];
-    if (c < 0 || !DG_IN_BOUNDS(c, A.E)) continue;
     const int f = sl - 1;
-    if (sl > 0 && f < 4) {
-      const int cc = f < 2 ? t0 : t1;
-      if (((f & 1) ? N - 1 - cc : cc) >= A.ov) continue;
-    }
-    const int4 af = s_aff[el][sl];
-    const int row0 = af.x + af.y * t0 + af.z * t1;
-    T* colp = A.rS + (int64_t)c * A.ld;
+    if (sl > 0 && f < 4 && !slot_covers<N>(sl, t0, t1, 0, A.ov)) continue;
+    const int4 rc = s_rec[el][sl];
+    if (rc.x < 0 || !DG_IN_BOUNDS(rc.x, A.E)) continue;
+    const int row0 = record_row(rc, t0, t1, 0), dk = (int)(short)(rc.w & 0xFFFF);
+    T* colp = A.rS + (int64_t)rc.x * A.ld;
 #pragma unroll
     for (int l = 0; l < N; ++l) {
       if (f >= 4 && ((f & 1) ? N - 1 - l : l) >= A.ov) continue;
-      const int row = row0 + af.w * l;
+      const int row = row0 + dk * l;
       if (DG_IN_BOUNDS(row, A.ld)) colp[row] = acc[l];
     }
   }
@@ -377,8 +358,8 @@ __device__ __forceinline__ void apply_par_block(const ApplyArgs<T>& A, int blk, 
   using L = DirLine<N, T, CT>;
   constexpr int N2 = S::N2, N3 = S::N3, LN = S::LN, XW = S::XW, PS = EPB * N2 * LN;
   T* sx = sm + 3 * PS;  // exchange, as above; sm: [direction][element][k][j][LN]
-  __shared__ int s_e[EPB], s_col[EPB][7];
-  __shared__ int4 s_aff[EPB][7];
+  __shared__ int s_e[EPB];
+  __shared__ int4 s_rec[EPB][7];
   if constexpr (PDL) pdl_launch_dependents();
   const OpGeom<T>& g = A.g;
   const T* __restrict__ u = A.u;
@@ -400,25 +381,12 @@ __device__ __forceinline__ void apply_par_block(const ApplyArgs<T>& A, int blk, 
   const bool in0 = lc > 0, in1 = lc + 1 < bn && has1;
   for (int q = tid; q < EPB * 7; q += S::THREADS) {
     const int el2 = q / 7, sl = q - el2 * 7;
-    int c3[3] = {(bx0 << A.bsx) + (el2 & ((1 << A.bsx) - 1)), (by0 << A.bsy) + ((el2 >> sx_) & ((1 << A.bsy) - 1)),
-                 bz0 * A.bz + (el2 >> sy_)};
-    bool ok = (el2 >> sy_) < A.bz && c3[0] < nx && c3[1] < ny && c3[2] < g.nz;
-    if (sl == 0) s_e[el2] = ok ? c3[0] + nx * (c3[1] + ny * c3[2]) : -1;
-    if (!A.rS) continue;
-    if (sl > 0) {
-      const int f = sl - 1, dd = f >> 1, nd = dd == 0 ? nx : (dd == 1 ? ny : g.nz);
-      c3[dd] += (f & 1) ? 1 : -1;
-      ok = ok && c3[dd] >= 0 && c3[dd] < nd;
-    }
-    int col = -1;
-    int4 af = make_int4(0, 0, 0, 0);
-    if (ok) {
-      const int rr = c3[0] + nx * (c3[1] + ny * c3[2]);
-      col = A.col_of_elem[rr];
-      af = A.aff[A.orient[rr] * 7 + (sl == 0 ? 0 : 1 + ((sl - 1) ^ 1))];
-    }
-    s_col[el2][sl] = col;
-    s_aff[el2][sl] = af;
+    const int c0 = (bx0 << A.bsx) + (el2 & ((1 << A.bsx) - 1)), c1 = (by0 << A.bsy) + ((el2 >> sx_) & ((1 << A.bsy) - 1)),
+              c2 = bz0 * A.bz + (el2 >> sy_);
+    const bool ok = (el2 >> sy_) < A.bz && c0 < nx && c1 < ny && c2 < g.nz;
+    const int e2 = c0 + nx * (c1 + ny * c2);
+    if (sl == 0) s_e[el2] = ok ? e2 : -1;
+    if (A.rS && ok) s_rec[el2][sl] = __ldg(A.rec + (int64_t)e2 * 7 + sl);
   }
   // first point and stride of the line: x-lines (j, k) = (t0, t1), y-lines (i, k), z-lines (i, j)
   const int t0 = t % N, t1 = t / N;
@@ -510,15 +478,12 @@ __device__ __forceinline__ void apply_par_block(const ApplyArgs<T>& A, int blk, 
       A.out[at] = val;
       continue;
     }
-    const int cc[3] = {i, j, k};
 #pragma unroll
     for (int sl = 0; sl < 7; ++sl) {
-      const int col = s_col[el2][sl], f = sl - 1;
-      if (col < 0 || !DG_IN_BOUNDS(col, A.E)) continue;
-      if (sl > 0 && ((f & 1) ? N - 1 - cc[f >> 1] : cc[f >> 1]) >= A.ov) continue;
-      const int4 af = s_aff[el2][sl];
-      const int row = af.x + af.y * i + af.z * j + af.w * k;
-      if (DG_IN_BOUNDS(row, A.ld)) A.rS[(int64_t)col * A.ld + row] = val;
+      if (!slot_covers<N>(sl, i, j, k, A.ov)) continue;
+      const int4 rc = s_rec[el2][sl];
+      const int row = record_row(rc, i, j, k);
+      if (rc.x >= 0 && DG_IN_BOUNDS(rc.x, A.E) && DG_IN_BOUNDS(row, A.ld)) A.rS[(int64_t)rc.x * A.ld + row] = val;
     }
   }
 }

@@ -23,9 +23,9 @@ struct SchwarzLevel {
   std::vector<int> patch;          // per class: 49 ints describing the representative's patch
   std::vector<int> class_key;      // per class: canonical boundary-code key
   double inv_scale = 1.0;          // stored inverses are built at unit element width: A_S^-1 = inv_scale x stored
-  DevBuf<int> elem_of_col;         // subdomain column -> element
   DevBuf<int> col_of_elem;         // element -> subdomain column
   DevBuf<int> class_of_col;        // subdomain column -> class
+  DevBuf<int4> rec;                // subdomain records [E][7], built with the inverses
   DevBuf<int> xform_of_elem;       // orientation index 8 perm + flips (canonical -> actual frame)
   DevBuf<double> inv64;            // [n_classes][nS][nS] explicit inverses (FP64 mode)
   DevBuf<float> inv32;             // FP32 copies (mixed mode)
@@ -61,7 +61,8 @@ template <typename T>
 struct LevelWork {
   DevBuf<T> b, u, r, rS, duS;
   // puncture subdomain GMRES (finest level only)
-  DevBuf<T> gV, gZ, gW, gD, gH;
+  DevBuf<T> gV, gZ, gD, gH;
+  bool gD_current = false;  // gD holds the diagonal of the current linearization
   // per-subdomain linearized inverses (finest level only): class matrices A_S at the actual
   // element widths [n_classes][nS][nS] and the inverses of A_S + D_S [E][nS][nS]
   DevBuf<T> linA, linv;
@@ -138,11 +139,9 @@ struct dg_domain {
   dg::DevBuf<float> D32, w32, Ilo32, Ihi32;
   std::vector<dg::Level> levels;
   dg::DevBuf<double> X, Y, Z, mass;
-  dg::DevBuf<double> shares64;  // Schwarz weight shares [64 neighbour patterns][N^3][7]
+  dg::DevBuf<double> shares64;  // Schwarz weight shares [64 neighbour patterns][7][N^3]
   dg::DevBuf<float> shares32;
-  dg::DevBuf<int> orient_map;   // [48][nS]: canonical subdomain row -> (actual slot, point)
-  dg::DevBuf<int> orient_inv;   // [48][7][N^3]: (actual slot, point) -> canonical row or -1
-  dg::DevBuf<int4> orient_aff;  // [48][7]: the same as an affine map, row = x + y i + z j + w k
+  dg::DevBuf<int4> orient_aff;  // [48][7]: canonical row of point (i, j, k) of an actual slot, x + y i + z j + w k
   // puncture
   dg::DevBuf<double> alpha, beta, lin64;
   dg::DevBuf<float> lin32;

@@ -162,9 +162,7 @@ struct SubdomainOut {
   void* rS = nullptr;            // T*: [columns][ld]
   int ld = 0;
   int ov = 0;                    // N_overlap
-  const int* col_of_elem = nullptr;
-  const int* orient = nullptr;   // orientation index per element
-  const int4* aff = nullptr;     // [48][7]: canonical row of point (i, j, k) = x + y i + z j + w k
+  const int4* rec = nullptr;     // subdomain records [E][7]
 };
 
 // Everything one DG apply reads and writes (rS != nullptr: write into the subdomain vectors).
@@ -180,9 +178,7 @@ struct ApplyArgs {
   int E;
   T* rS;
   int ld, ov;
-  const int* col_of_elem;
-  const int* orient;
-  const int4* aff;
+  const int4* rec;
   // direction-by-direction kernel: brick of (1 << bsx) x (1 << bsy) x bz elements, bricks along x and y
   int bsx, bsy, bz, nbx, nby;
 };
@@ -210,12 +206,16 @@ struct SubdomainGeom {
   int E, N, ov, nS;
   int ld;  // column stride of subdomain vectors and row stride of inverses: nS rounded up to 32
 };
+// Subdomain records [E][7] (schwarz_dev.cuh) from the columns, orientations and affine row maps.
+void launch_subdomain_records(const SubdomainGeom& g, const int* col_of_elem, const int* orient, const int4* aff,
+                              int4* rec, cudaStream_t s);
+// r_S = R_S r. Rows that no point maps to are not written: the caller's buffer holds zeros there.
 template <typename T>
-void launch_gather_tab(const SubdomainGeom& g, const T* r, const int* elem_of_col, const int* orient, const int* map,
-                       T* rS, cudaStream_t s);
-template <typename T, typename TU>
-void launch_scatter_tab(const SubdomainGeom& g, const T* duS, const int* col_of_elem, const int* orient,
-                        const int* inv, const T* shares, TU* u, cudaStream_t s);
+void launch_gather(const SubdomainGeom& g, const T* r, const int4* rec, T* rS, cudaStream_t s);
+// u += sum_S R_S^T w_S du_S, du_S = X (m = 0, y unused) or sum_{c < m} y[column][c] X_c, X_c = X + c stride.
+template <typename T>
+void launch_scatter(const SubdomainGeom& g, const T* X, const T* y, int m, int64_t stride, const int4* rec,
+                    const T* shares, T* u, cudaStream_t s);
 template <typename S, typename T>
 void launch_pad_convert(const S* src, int n, int ld, int n_classes, T* dst, cudaStream_t s);
 
@@ -225,10 +225,7 @@ void launch_pad_convert(const S* src, int n, int ld, int n_classes, T* dst, cuda
 struct CoarseArgs {
   ApplyArgs<float> ap;       // residual r = b - A u written into r_S (ap.rS)
   SubdomainGeom sg;
-  const int* elem_of_col;    // gather of the first step when u = 0
-  const int* map;
   const float* shares;       // scatter weights
-  const int* inv;            // [48][7][N^3]: canonical row of a point
   int n_bricks;              // bricks of the residual (set by the launcher)
   float* duS;
   const float* invm;         // class inverses [class][ld][ld] (unit width)
@@ -282,13 +279,12 @@ bool tune_log();  // DG_TUNE_LOG=1
 int autotune(const std::vector<int64_t>& key, const std::vector<int>& candidates,
              const std::function<void(int)>& run, cudaStream_t s);
 
-// Subdomain GMRES for linearized problems (columns of n_S values, E columns per basis vector).
+// Arnoldi step j of m of the subdomain GMRES for linearized problems, on columns of ld values (E per
+// block): r_S, D, V_1.. and Z_0.. blocks, H [E][m + 1][m], beta [E]; the last step leaves the factors of the
+// Z_c in y [E][m]. V holds m blocks.
 template <typename T>
-void launch_sub_normalize(int E, int nS, const T* rS, T* V0, T* beta, cudaStream_t s);
-template <typename T>
-void launch_sub_arnoldi(int E, int nS, int j, int m, const T* D, T* V, const T* Z, T* H, cudaStream_t s);
-template <typename T>
-void launch_sub_lsq_combine(int E, int nS, int m, const T* beta, const T* H, const T* Z, T* duS, cudaStream_t s);
+void launch_sub_arnoldi(int E, int ld, int j, int m, const T* r, const T* D, T* V, const T* Z, T* H, T* beta, T* y,
+                        cudaStream_t s);
 
 // Curved (mapped) elements and variable coefficients: metric [11][ndof] (J, then G^j_i = dxi^j/dx^i
 // at 1 + 3 j + i, then the coefficient K at 10), penalty

@@ -374,58 +374,131 @@ template void launch_pad_convert<float, float>(const float*, int, int, int, floa
 
 
 // ------------------------------------------------------------------ gather / scatter
-
-
-// ------------------------------------------------------------------ table-driven gather / scatter
 //
-// The point maps depend only on (N, N_overlap) and the subdomain's orientation (48 reflections x
-// axis permutations), so they are tabulated once per domain: map[o][q] = (actual slot << 16) |
-// actual point for canonical subdomain row q, and its inverse inv[o][slot][p] = canonical row of
-// point p of the given actual slot (or -1 outside the subdomain). One CTA per subdomain column
-// (gather) or per element (scatter) resolves its neighbours once in shared memory; each point then
-// costs one table load instead of a chain of integer divisions.
+// One thread per point of the level, with the level's subdomain records (schwarz_dev.cuh) in place of
+// per-point row tables: the look-ups of a point are one or a few 16-byte broadcasts and coalesced weight
+// loads, all static, so they precede the wait for the previous kernel. The scatter is bound by latency
+// at the sizes of one level (16^3 elements, N = 6: 15.1 us a launch with one CTA per element, tables of
+// rows and interleaved weights), the gather likewise (9.3 us).
 
-template <typename T>
-__global__ void gather_tab_kernel(SubdomainGeom g, const T* __restrict__ r, const int* __restrict__ elem_of_col,
-                                  const int* __restrict__ orient, const int* __restrict__ map, T* __restrict__ rS) {
-  pdl_launch_dependents();
-  gather_column<T, true>(g, r, elem_of_col, orient, map, rS, blockIdx.x);
+__global__ void record_kernel(SubdomainGeom g, const int* __restrict__ col_of_elem, const int* __restrict__ orient,
+                              const int4* __restrict__ aff, int4* __restrict__ rec) {
+  const int q = blockIdx.x * blockDim.x + threadIdx.x;
+  if (q >= g.E * 7) return;
+  const int e = q / 7, sl = q - e * 7;
+  int pat = 0;
+  for (int f = 0; f < 6; ++f) pat |= (nbr_elem(g, e, f) >= 0) << f;
+  const int n = sl == 0 ? e : nbr_elem(g, e, sl - 1);
+  // element e is in its own subdomain's slot 0, and neighbour n sees it across the opposite face
+  int4 r = make_int4(-1, 0, 0, 0);
+  if (n >= 0) {
+    const int4 a = aff[orient[n] * 7 + (sl == 0 ? 0 : 1 + ((sl - 1) ^ 1))];
+    r = make_int4(col_of_elem[n], a.x, (a.y & 0xFFFF) | (a.z << 16), a.w & 0xFFFF);
+  }
+  if (sl == 0) r.w |= pat << 16;
+  rec[q] = r;
 }
 
-template <typename T, typename TU>
-__global__ void scatter_tab_kernel(SubdomainGeom g, const T* __restrict__ duS, const int* __restrict__ col_of_elem,
-                                   const int* __restrict__ orient, const int* __restrict__ inv,
-                                   const T* __restrict__ shares, TU* __restrict__ u) {
-  pdl_launch_dependents();
-  scatter_element<T, TU, true>(g, duS, col_of_elem, orient, inv, shares, u, blockIdx.x);
-}
-
-template <typename T>
-void launch_gather_tab(const SubdomainGeom& g, const T* r, const int* elem_of_col, const int* orient, const int* map,
-                       T* rS, cudaStream_t s) {
+void launch_subdomain_records(const SubdomainGeom& g, const int* col_of_elem, const int* orient, const int4* aff,
+                              int4* rec, cudaStream_t s) {
   if (g.E == 0) return;
-  launch_pdl(gather_tab_kernel<T>, dim3(g.E), dim3(256), 0, s, g, r, elem_of_col, orient, map, rS);
+  record_kernel<<<(g.E * 7 + 255) / 256, 256, 0, s>>>(g, col_of_elem, orient, aff, rec);
   DG_LAUNCHED(1);
 }
 
-template <typename T, typename TU>
-void launch_scatter_tab(const SubdomainGeom& g, const T* duS, const int* col_of_elem, const int* orient,
-                        const int* inv, const T* shares, TU* u, cudaStream_t s) {
+template <int N, typename T>
+__global__ void __launch_bounds__(256) gather_kernel(SubdomainGeom g, const T* __restrict__ r,
+                                                     const int4* __restrict__ rec, T* __restrict__ rS) {
+  constexpr int N3 = N * N * N;
+  const int t = blockIdx.x * 256 + threadIdx.x;
+  pdl_launch_dependents();
+  pdl_wait();
+  if (t >= g.E * N3) return;
+  const int e = t / N3;
+  gather_point<N, T>(g, rec, r[t], rS, e, t - e * N3);
+}
+
+// u += sum_S R_S^T w_S du_S with du_S = X (m = 0), or du_S = sum_{c < m} y[column][c] X_c, the X_c
+// `stride` values apart.
+template <int N, typename T, int M>
+__global__ void __launch_bounds__(256) scatter_kernel(SubdomainGeom g, const T* __restrict__ X,
+                                                      const T* __restrict__ y, int m, int64_t stride,
+                                                      const int4* __restrict__ rec, const T* __restrict__ shares,
+                                                      T* __restrict__ u) {
+  constexpr int N3 = N * N * N;
+  const int t = blockIdx.x * 256 + threadIdx.x;
+  pdl_launch_dependents();
+  const bool act = t < g.E * N3;
+  const int e = act ? t / N3 : 0;
+  int64_t idx[7];
+  int col[7];
+  T w[7], v[7];
+  scatter_look_up<N, T>(g, rec, shares, e, act ? t - e * N3 : 0, idx, col, w);
+  pdl_wait();
+  if (!act) return;
+  const T u0 = u[t];
+  if constexpr (M == 0) {
+#pragma unroll
+    for (int sl = 0; sl < 7; ++sl) v[sl] = idx[sl] >= 0 ? X[idx[sl]] : T(0);
+  } else {
+#pragma unroll
+    for (int sl = 0; sl < 7; ++sl) v[sl] = T(0);
+    const int mm = M > 0 ? M : m;  // M < 0: any m
+#pragma unroll
+    for (int c = 0; c < mm; ++c)
+#pragma unroll
+      for (int sl = 0; sl < 7; ++sl)
+        if (idx[sl] >= 0) v[sl] += y[(int64_t)col[sl] * mm + c] * X[c * stride + idx[sl]];
+  }
+  T acc = w[0] * v[0];
+#pragma unroll
+  for (int sl = 1; sl < 7; ++sl) acc += w[sl] * v[sl];
+  u[t] = u0 + acc;
+}
+
+template <int N, typename T>
+void launch_scatter_n(const SubdomainGeom& g, const T* X, const T* y, int m, int64_t stride, const int4* rec,
+                      const T* shares, T* u, cudaStream_t s) {
+  const dim3 grid((g.E * N * N * N + 255) / 256);
+  if (m == 0) launch_pdl(scatter_kernel<N, T, 0>, grid, dim3(256), 0, s, g, X, y, m, stride, rec, shares, u);
+  else if (m == 3) launch_pdl(scatter_kernel<N, T, 3>, grid, dim3(256), 0, s, g, X, y, m, stride, rec, shares, u);
+  else launch_pdl(scatter_kernel<N, T, -1>, grid, dim3(256), 0, s, g, X, y, m, stride, rec, shares, u);
+}
+
+template <typename T>
+void launch_gather(const SubdomainGeom& g, const T* r, const int4* rec, T* rS, cudaStream_t s) {
   if (g.E == 0) return;
-  const int N3 = g.N * g.N * g.N;
-  launch_pdl(scatter_tab_kernel<T, TU>, dim3(g.E), dim3(N3 > 512 ? 512 : (N3 < 32 ? 32 : N3)), 0, s, g, duS,
-             col_of_elem, orient, inv, shares, u);
+  const dim3 grid((g.E * g.N * g.N * g.N + 255) / 256);
+  switch (g.N) {
+#define DG_CASE(NN) \
+  case NN: launch_pdl(gather_kernel<NN, T>, grid, dim3(256), 0, s, g, r, rec, rS); break;
+    DG_CASE(2) DG_CASE(3) DG_CASE(4) DG_CASE(5) DG_CASE(6) DG_CASE(7) DG_CASE(8) DG_CASE(9) DG_CASE(10)
+#undef DG_CASE
+    default: fail(DG_ERR_INVALID_ARG, "unsupported N");
+  }
   DG_LAUNCHED(1);
 }
 
-template void launch_gather_tab<double>(const SubdomainGeom&, const double*, const int*, const int*, const int*,
-                                        double*, cudaStream_t);
-template void launch_gather_tab<float>(const SubdomainGeom&, const float*, const int*, const int*, const int*, float*,
-                                       cudaStream_t);
-template void launch_scatter_tab<double, double>(const SubdomainGeom&, const double*, const int*, const int*,
-                                                 const int*, const double*, double*, cudaStream_t);
-template void launch_scatter_tab<float, float>(const SubdomainGeom&, const float*, const int*, const int*, const int*,
-                                               const float*, float*, cudaStream_t);
+template <typename T>
+void launch_scatter(const SubdomainGeom& g, const T* X, const T* y, int m, int64_t stride, const int4* rec,
+                    const T* shares, T* u, cudaStream_t s) {
+  if (g.E == 0) return;
+  switch (g.N) {
+#define DG_CASE(NN) \
+  case NN: launch_scatter_n<NN, T>(g, X, y, m, stride, rec, shares, u, s); break;
+    DG_CASE(2) DG_CASE(3) DG_CASE(4) DG_CASE(5) DG_CASE(6) DG_CASE(7) DG_CASE(8) DG_CASE(9) DG_CASE(10)
+#undef DG_CASE
+    default: fail(DG_ERR_INVALID_ARG, "unsupported N");
+  }
+  DG_LAUNCHED(1);
+}
+
+template void launch_gather<double>(const SubdomainGeom&, const double*, const int4*, double*, cudaStream_t);
+template void launch_gather<float>(const SubdomainGeom&, const float*, const int4*, float*, cudaStream_t);
+template void launch_scatter<double>(const SubdomainGeom&, const double*, const double*, int, int64_t, const int4*,
+                                     const double*, double*, cudaStream_t);
+template void launch_scatter<float>(const SubdomainGeom&, const float*, const float*, int, int64_t, const int4*,
+                                    const float*, float*, cudaStream_t);
 
 // ------------------------------------------------------------------ class GEMM (SIMT)
 
@@ -657,246 +730,193 @@ struct SubVec<double> {
   }
 };
 
-// V_0 = r_S / ||r_S|| per column; beta[col] = ||r_S||
+// What an Arnoldi step of one level's subdomain GMRES reads and writes. V_0 = r_S / ||r_S|| is never
+// formed: the first product is Z_0 ||r_S|| = A_S^-1 r_S, and every use of V_0 or Z_0 divides by beta. The
+// last step stores no V_m (nothing reads it) but solves the least-squares problem
+// y = argmin || beta e1 - H y || and leaves the factors of the stored Z_c, y_0 / beta and y_c, in y, for the
+// scatter to combine. H is [column][m + 1][m]; V_1 .. V_{m-1} and Z_0 .. Z_{m-1} are blocks `stride` apart.
 template <typename T>
-__global__ void __launch_bounds__(32 * kSubWarps)
-    sub_normalize_kernel(int E, int nS, const T* __restrict__ rS, T* __restrict__ V0, T* __restrict__ beta) {
-  const int col = blockIdx.x * kSubWarps + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-  if (col >= E) return;  // whole warps
-  const T* r = rS + (size_t)col * nS;
-  T acc = 0;
-  for (int i = lane; i < nS; i += 32) acc += r[i] * r[i];
-  const T nrm = sqrt(warp_total(acc));
-  const T inv = nrm > T(0) ? T(1) / nrm : T(0);
-  for (int i = lane; i < nS; i += 32) V0[(size_t)col * nS + i] = r[i] * inv;
-  if (lane == 0) beta[col] = nrm;
+struct SubKrylov {
+  int E, ld, j, m;
+  int64_t stride;
+  const T* r;
+  const T* D;
+  const T* Z;
+  T* V;
+  T* H;
+  T* beta;
+  T* y;
+};
+
+// Givens rotations on the column's Hessenberg matrix and back substitution (one thread).
+template <typename T>
+__device__ void sub_least_squares(const SubKrylov<T>& a, int col) {
+  const int m = a.m;
+  T R[17][16], g[17];
+  const T* h = a.H + (size_t)col * (m + 1) * m;
+  for (int i = 0; i <= m; ++i) {
+    g[i] = 0;
+    for (int c = 0; c < m; ++c) R[i][c] = h[i * m + c];
+  }
+  const T beta = a.beta[col];
+  g[0] = beta;
+  int k = m;  // stop at a (happy) breakdown: zero subdiagonal
+  for (int c = 0; c < m; ++c) {
+    const T x = R[c][c], b = R[c + 1][c];
+    const T den = sqrt(x * x + b * b);
+    if (den == T(0)) { k = c; break; }
+    const T cs = x / den, sn = b / den;
+    for (int cc = c; cc < m; ++cc) {
+      const T x0 = R[c][cc], x1 = R[c + 1][cc];
+      R[c][cc] = cs * x0 + sn * x1;
+      R[c + 1][cc] = -sn * x0 + cs * x1;
+    }
+    const T g0 = g[c];
+    g[c] = cs * g0;
+    g[c + 1] = -sn * g0;
+    if (b == T(0)) { k = c + 1; break; }
+  }
+  T* y = a.y + (size_t)col * m;
+  for (int c = k; c < m; ++c) y[c] = 0;
+  for (int i = k - 1; i >= 0; --i) {
+    T acc = g[i];
+    for (int c = i + 1; c < k; ++c) acc -= R[i][c] * y[c];
+    y[i] = acc / R[i][i];
+  }
+  y[0] = beta == T(0) ? T(0) : y[0] / beta;  // a NaN stays one
 }
 
-// Arnoldi step j: w = V_j + D Z_j, modified Gram-Schmidt against V_0..V_j, V_{j+1} = w / ||w||.
-// H is [col][m+1][m]; V and Z are blocks of E*nS values per basis index. w is built in place in
-// V_{j+1}; every lane reads back only the entries it wrote.
-template <typename T>
-__global__ void __launch_bounds__(32 * kSubWarps)
-    sub_arnoldi_kernel(int E, int nS, int64_t stride, int j, int m, const T* __restrict__ D, T* V,
-                       const T* __restrict__ Z, T* __restrict__ H) {
+// Arnoldi step j: w = V_j + D Z_j, modified Gram-Schmidt against V_0..V_j, V_{j+1} = w / ||w||. One warp per
+// column. G > 0: the column's w and the current V_i stay in registers as G 16-byte vectors per lane (lane
+// l holds elements 16/sizeof(T) x (32 g + l) + 0..), so every vector is read or written once. G = 0, for
+// longer columns: w is built in place in V_{j+1} (block j; the last step uses one too), every lane reading
+// back only the entries it wrote.
+template <typename T, int G>
+__global__ void __launch_bounds__(32 * kSubWarps) sub_arnoldi_kernel(const SubKrylov<T> a) {
+  using SV = SubVec<T>;
+  constexpr int EV = SV::E, GG = G > 0 ? G : 1;
   const int col = blockIdx.x * kSubWarps + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-  if (col >= E) return;  // whole warps
-  const size_t off = (size_t)col * nS;
-  const T* vj = V + (size_t)j * stride + off;
-  const T* zj = Z + (size_t)j * stride + off;
-  T* w = V + (size_t)(j + 1) * stride + off;
+  if (col >= a.E) return;  // whole warps
+  const int j = a.j, m = a.m, ld = a.ld;
+  const size_t off = (size_t)col * ld;
+  const T* r = a.r + off;
+  const T* D = a.D + off;
+  const T* zj = a.Z + (size_t)j * a.stride + off;
+  const T* vj = j == 0 ? r : a.V + (size_t)(j - 1) * a.stride + off;
+  T* wout = a.V + (size_t)j * a.stride + off;
+  T* h = a.H + (size_t)col * (m + 1) * m;
+  T w[GG][EV], b2 = 0;
+  if constexpr (G > 0) {
+#pragma unroll
+    for (int g = 0; g < G; ++g) {
+      const int i = (g * 32 + lane) * EV;
+#pragma unroll
+      for (int e = 0; e < EV; ++e) w[g][e] = 0;
+      if (i >= ld) continue;
+      T x[EV], d[EV], z[EV];
+      SV::ld(vj + i, x);
+      SV::ld(D + i, d);
+      SV::ld(zj + i, z);
+#pragma unroll
+      for (int e = 0; e < EV; ++e) {
+        w[g][e] = x[e] + d[e] * z[e];
+        b2 += x[e] * x[e];
+      }
+    }
+  } else {
+    for (int i = lane; i < ld; i += 32) {
+      wout[i] = vj[i] + D[i] * zj[i];
+      b2 += vj[i] * vj[i];
+    }
+  }
+  T beta;  // ||r_S||
+  if (j == 0) {
+    beta = sqrt(warp_total(b2));
+    if (lane == 0) a.beta[col] = beta;
+  } else {
+    beta = a.beta[col];
+  }
+  const T inv_beta = beta > T(0) ? T(1) / beta : T(0);
+  const T s0 = j == 0 ? inv_beta : T(1);  // step 0 worked on beta V_0 and beta Z_0
   T acc0 = 0;
-  for (int i = lane; i < nS; i += 32) {
-    const T x = vj[i] + D[off + i] * zj[i];
-    w[i] = x;
-    acc0 += x * x;
+  if constexpr (G > 0) {
+#pragma unroll
+    for (int g = 0; g < G; ++g)
+#pragma unroll
+      for (int e = 0; e < EV; ++e) {
+        w[g][e] *= s0;
+        acc0 += w[g][e] * w[g][e];
+      }
+  } else {
+    for (int i = lane; i < ld; i += 32) {
+      wout[i] *= s0;
+      acc0 += wout[i] * wout[i];
+    }
   }
   const T w0 = sqrt(warp_total(acc0));  // ||w|| before orthogonalisation
-  T* h = H + (size_t)col * (m + 1) * m;
-  for (int i = 0; i <= j; ++i) {
-    const T* vi = V + (size_t)i * stride + off;
+  for (int ii = 0; ii <= j; ++ii) {
+    const T* vi = ii == 0 ? r : a.V + (size_t)(ii - 1) * a.stride + off;
+    const T sc = ii == 0 ? inv_beta : T(1);
     T acc = 0;
-    for (int t = lane; t < nS; t += 32) acc += w[t] * vi[t];
+    T v[GG][EV];
+    if constexpr (G > 0) {
+#pragma unroll
+      for (int g = 0; g < G; ++g) {
+        const int i = (g * 32 + lane) * EV;
+#pragma unroll
+        for (int e = 0; e < EV; ++e) v[g][e] = 0;
+        if (i < ld) SV::ld(vi + i, v[g]);
+#pragma unroll
+        for (int e = 0; e < EV; ++e) {
+          v[g][e] *= sc;
+          acc += w[g][e] * v[g][e];
+        }
+      }
+    } else {
+      for (int t = lane; t < ld; t += 32) acc += wout[t] * (sc * vi[t]);
+    }
     const T hij = warp_total(acc);
-    for (int t = lane; t < nS; t += 32) w[t] -= hij * vi[t];
-    if (lane == 0) h[i * m + j] = hij;
+    if constexpr (G > 0) {
+#pragma unroll
+      for (int g = 0; g < G; ++g)
+#pragma unroll
+        for (int e = 0; e < EV; ++e) w[g][e] -= hij * v[g][e];
+    } else {
+      for (int t = lane; t < ld; t += 32) wout[t] -= hij * (sc * vi[t]);
+    }
+    if (lane == 0) h[ii * m + j] = hij;
   }
   T acc = 0;
-  for (int t = lane; t < nS; t += 32) acc += w[t] * w[t];
+  if constexpr (G > 0) {
+#pragma unroll
+    for (int g = 0; g < G; ++g)
+#pragma unroll
+      for (int e = 0; e < EV; ++e) acc += w[g][e] * w[g][e];
+  } else {
+    for (int t = lane; t < ld; t += 32) acc += wout[t] * wout[t];
+  }
   T hn = sqrt(warp_total(acc));
   // what is left after orthogonalisation at the level of the cancellation error is rounding noise,
   // not a new direction: treat it as a (happy) breakdown so that the least-squares step ignores it
   if (hn <= T(64) * std::numeric_limits<T>::epsilon() * w0) hn = T(0);
-  if (lane == 0) h[(j + 1) * m + j] = hn;
-  const T inv = hn > T(0) ? T(1) / hn : T(0);
-  for (int t = lane; t < nS; t += 32) w[t] *= inv;
-}
-
-// y = argmin || beta e1 - H y || (Givens, by lane 0 of the column's warp), then du_S = sum_j y_j Z_j.
-template <typename T, int G = 0>
-__global__ void __launch_bounds__(32 * kSubWarps)
-    sub_lsq_combine_kernel(int E, int nS, int64_t stride, int m, const T* __restrict__ beta,
-                           const T* __restrict__ H, const T* __restrict__ Z, T* __restrict__ duS) {
-  __shared__ T ys[kSubWarps][16];
-  const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int col = blockIdx.x * kSubWarps + wid;
-  if (col >= E) return;  // whole warps
-  T* y = ys[wid];
   if (lane == 0) {
-    T R[17][16], g[17];
-    const T* h = H + (size_t)col * (m + 1) * m;
-    for (int i = 0; i <= m; ++i) {
-      g[i] = 0;
-      for (int c = 0; c < m; ++c) R[i][c] = h[i * m + c];
-    }
-    g[0] = beta[col];
-    int k = m;  // stop at a (happy) breakdown: zero subdiagonal
-    for (int c = 0; c < m; ++c) {
-      const T a = R[c][c], b = R[c + 1][c];
-      const T den = sqrt(a * a + b * b);
-      if (den == T(0)) { k = c; break; }
-      const T cs = a / den, sn = b / den;
-      for (int cc = c; cc < m; ++cc) {
-        const T x0 = R[c][cc], x1 = R[c + 1][cc];
-        R[c][cc] = cs * x0 + sn * x1;
-        R[c + 1][cc] = -sn * x0 + cs * x1;
-      }
-      const T g0 = g[c];
-      g[c] = cs * g0;
-      g[c + 1] = -sn * g0;
-      if (b == T(0)) { k = c + 1; break; }
-    }
-    for (int c = 0; c < m; ++c) y[c] = 0;
-    for (int i = k - 1; i >= 0; --i) {
-      T acc = g[i];
-      for (int c = i + 1; c < k; ++c) acc -= R[i][c] * y[c];
-      y[i] = acc / R[i][i];
-    }
+    h[(j + 1) * m + j] = hn;
+    for (int i = j + 2; i <= m; ++i) h[i * m + j] = T(0);
+    if (j == m - 1) sub_least_squares(a, col);
   }
-  __syncwarp();
-  const size_t off = (size_t)col * nS;
-  if constexpr (G == 0) {
-    for (int t = lane; t < nS; t += 32) {
-      T acc = 0;
-      for (int c = 0; c < m; ++c) acc += y[c] * Z[(size_t)c * stride + off + t];
-      duS[off + t] = acc;
+  if (j == m - 1) return;
+  const T inv = hn > T(0) ? T(1) / hn : T(0);
+  if constexpr (G > 0) {
+#pragma unroll
+    for (int g = 0; g < G; ++g) {
+      const int i = (g * 32 + lane) * EV;
+      if (i >= ld) continue;
+#pragma unroll
+      for (int e = 0; e < EV; ++e) w[g][e] *= inv;
+      SV::st(wout + i, w[g]);
     }
   } else {
-    // 16-byte vectors per lane, as the register forms of the other two kernels
-    using SV = SubVec<T>;
-    constexpr int EV = SV::E;
-    T acc[G][EV] = {};
-    for (int c = 0; c < m; ++c) {
-      const T yc = y[c];
-      const T* zc = Z + (size_t)c * stride + off;
-#pragma unroll
-      for (int g = 0; g < G; ++g) {
-        const int i = (g * 32 + lane) * EV;
-        if (i >= nS) continue;
-        T z[EV];
-        SV::ld(zc + i, z);
-#pragma unroll
-        for (int e = 0; e < EV; ++e) acc[g][e] += yc * z[e];
-      }
-    }
-#pragma unroll
-    for (int g = 0; g < G; ++g) {
-      const int i = (g * 32 + lane) * EV;
-      if (i < nS) SV::st(duS + off + i, acc[g]);
-    }
-  }
-}
-
-// Register-resident forms of the two per-subdomain kernels above: a warp keeps its column's w
-// (and the current V_i) in registers as G 16-byte vectors per lane (lane l holds elements
-// 16/sizeof(T) x (32 g + l) + 0..), so every vector of the column is read or written once per call
-// with 16-byte coalesced accesses instead of once per Gram-Schmidt pass. Same operations in the
-// same order per element as the kernels above; only the partial sums of each inner product are
-// grouped differently across the lanes.
-template <typename T, int G>
-__global__ void __launch_bounds__(32 * kSubWarps)
-    sub_normalize_reg_kernel(int E, int ld, const T* __restrict__ rS, T* __restrict__ V0, T* __restrict__ beta) {
-  using SV = SubVec<T>;
-  constexpr int EV = SV::E;
-  const int col = blockIdx.x * kSubWarps + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-  if (col >= E) return;  // whole warps
-  const size_t off = (size_t)col * ld;
-  T r[G][EV];
-  T acc = 0;
-#pragma unroll
-  for (int g = 0; g < G; ++g) {
-    const int i = (g * 32 + lane) * EV;
-    if (i < ld) SV::ld(rS + off + i, r[g]);
-    else
-#pragma unroll
-      for (int e = 0; e < EV; ++e) r[g][e] = 0;
-#pragma unroll
-    for (int e = 0; e < EV; ++e) acc += r[g][e] * r[g][e];
-  }
-  const T nrm = sqrt(warp_total(acc));
-  const T inv = nrm > T(0) ? T(1) / nrm : T(0);
-#pragma unroll
-  for (int g = 0; g < G; ++g) {
-    const int i = (g * 32 + lane) * EV;
-    if (i >= ld) continue;
-#pragma unroll
-    for (int e = 0; e < EV; ++e) r[g][e] *= inv;
-    SV::st(V0 + off + i, r[g]);
-  }
-  if (lane == 0) beta[col] = nrm;
-}
-
-template <typename T, int G>
-__global__ void __launch_bounds__(32 * kSubWarps)
-    sub_arnoldi_reg_kernel(int E, int ld, int64_t stride, int j, int m, const T* __restrict__ D, T* V,
-                           const T* __restrict__ Z, T* __restrict__ H) {
-  using SV = SubVec<T>;
-  constexpr int EV = SV::E;
-  const int col = blockIdx.x * kSubWarps + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-  if (col >= E) return;  // whole warps
-  const size_t off = (size_t)col * ld;
-  const T* vj = V + (size_t)j * stride + off;
-  const T* zj = Z + (size_t)j * stride + off;
-  T w[G][EV];
-  T acc0 = 0;
-#pragma unroll
-  for (int g = 0; g < G; ++g) {
-    const int i = (g * 32 + lane) * EV;
-    if (i < ld) {
-      T a[EV], d[EV], z[EV];
-      SV::ld(vj + i, a);
-      SV::ld(D + off + i, d);
-      SV::ld(zj + i, z);
-#pragma unroll
-      for (int e = 0; e < EV; ++e) w[g][e] = a[e] + d[e] * z[e];
-    } else {
-#pragma unroll
-      for (int e = 0; e < EV; ++e) w[g][e] = 0;
-    }
-#pragma unroll
-    for (int e = 0; e < EV; ++e) acc0 += w[g][e] * w[g][e];
-  }
-  const T w0 = sqrt(warp_total(acc0));  // ||w|| before orthogonalisation
-  T* h = H + (size_t)col * (m + 1) * m;
-  for (int ii = 0; ii <= j; ++ii) {
-    const T* vi = V + (size_t)ii * stride + off;
-    T v[G][EV];
-    T acc = 0;
-#pragma unroll
-    for (int g = 0; g < G; ++g) {
-      const int i = (g * 32 + lane) * EV;
-      if (i < ld) SV::ld(vi + i, v[g]);
-      else
-#pragma unroll
-        for (int e = 0; e < EV; ++e) v[g][e] = 0;
-#pragma unroll
-      for (int e = 0; e < EV; ++e) acc += w[g][e] * v[g][e];
-    }
-    const T hij = warp_total(acc);
-#pragma unroll
-    for (int g = 0; g < G; ++g)
-#pragma unroll
-      for (int e = 0; e < EV; ++e) w[g][e] -= hij * v[g][e];
-    if (lane == 0) h[ii * m + j] = hij;
-  }
-  T acc = 0;
-#pragma unroll
-  for (int g = 0; g < G; ++g)
-#pragma unroll
-    for (int e = 0; e < EV; ++e) acc += w[g][e] * w[g][e];
-  T hn = sqrt(warp_total(acc));
-  // rounding noise after orthogonalisation is a (happy) breakdown, as in sub_arnoldi_kernel
-  if (hn <= T(64) * std::numeric_limits<T>::epsilon() * w0) hn = T(0);
-  if (lane == 0) h[(j + 1) * m + j] = hn;
-  const T inv = hn > T(0) ? T(1) / hn : T(0);
-  T* wout = V + (size_t)(j + 1) * stride + off;
-#pragma unroll
-  for (int g = 0; g < G; ++g) {
-    const int i = (g * 32 + lane) * EV;
-    if (i >= ld) continue;
-#pragma unroll
-    for (int e = 0; e < EV; ++e) w[g][e] *= inv;
-    SV::st(wout + i, w[g]);
+    for (int t = lane; t < ld; t += 32) wout[t] *= inv;
   }
 }
 
@@ -912,59 +932,25 @@ int sub_reg_groups(int ld) {
 }
 
 template <typename T>
-void launch_sub_normalize(int E, int nS, const T* rS, T* V0, T* beta, cudaStream_t s) {
+void launch_sub_arnoldi(int E, int ld, int j, int m, const T* r, const T* D, T* V, const T* Z, T* H, T* beta, T* y,
+                        cudaStream_t s) {
   if (E == 0) return;
   const dim3 grid((E + kSubWarps - 1) / kSubWarps), block(32 * kSubWarps);
-  switch (sub_reg_groups<T>(nS)) {
-#define DG_SUB_NORM(GG) \
-  case GG: sub_normalize_reg_kernel<T, GG><<<grid, block, 0, s>>>(E, nS, rS, V0, beta); break;
-    DG_SUB_NORM(1) DG_SUB_NORM(2) DG_SUB_NORM(3) DG_SUB_NORM(4) DG_SUB_NORM(6) DG_SUB_NORM(8) DG_SUB_NORM(10)
-    DG_SUB_NORM(12) DG_SUB_NORM(14) DG_SUB_NORM(16)
-#undef DG_SUB_NORM
-    default: sub_normalize_kernel<T><<<grid, block, 0, s>>>(E, nS, rS, V0, beta);
-  }
-  DG_LAUNCHED(1);
-}
-template <typename T>
-void launch_sub_arnoldi(int E, int nS, int j, int m, const T* D, T* V, const T* Z, T* H, cudaStream_t s) {
-  if (E == 0) return;
-  const dim3 grid((E + kSubWarps - 1) / kSubWarps), block(32 * kSubWarps);
-  const int64_t stride = (int64_t)E * nS;
-  switch (sub_reg_groups<T>(nS)) {
+  const SubKrylov<T> a{E, ld, j, m, (int64_t)E * ld, r, D, Z, V, H, beta, y};
+  switch (sub_reg_groups<T>(ld)) {
 #define DG_SUB_ARN(GG) \
-  case GG: sub_arnoldi_reg_kernel<T, GG><<<grid, block, 0, s>>>(E, nS, stride, j, m, D, V, Z, H); break;
+  case GG: sub_arnoldi_kernel<T, GG><<<grid, block, 0, s>>>(a); break;
     DG_SUB_ARN(1) DG_SUB_ARN(2) DG_SUB_ARN(3) DG_SUB_ARN(4) DG_SUB_ARN(6) DG_SUB_ARN(8) DG_SUB_ARN(10)
     DG_SUB_ARN(12) DG_SUB_ARN(14) DG_SUB_ARN(16)
 #undef DG_SUB_ARN
-    default: sub_arnoldi_kernel<T><<<grid, block, 0, s>>>(E, nS, stride, j, m, D, V, Z, H);
+    default: sub_arnoldi_kernel<T, 0><<<grid, block, 0, s>>>(a);
   }
   DG_LAUNCHED(1);
 }
-template <typename T>
-void launch_sub_lsq_combine(int E, int nS, int m, const T* beta, const T* H, const T* Z, T* duS, cudaStream_t s) {
-  if (E == 0) return;
-  const dim3 grid((E + kSubWarps - 1) / kSubWarps), block(32 * kSubWarps);
-  const int64_t stride = (int64_t)E * nS;
-  switch (sub_reg_groups<T>(nS)) {
-#define DG_SUB_LSQ(GG) \
-  case GG: sub_lsq_combine_kernel<T, GG><<<grid, block, 0, s>>>(E, nS, stride, m, beta, H, Z, duS); break;
-    DG_SUB_LSQ(1) DG_SUB_LSQ(2) DG_SUB_LSQ(3) DG_SUB_LSQ(4) DG_SUB_LSQ(6) DG_SUB_LSQ(8) DG_SUB_LSQ(10)
-    DG_SUB_LSQ(12) DG_SUB_LSQ(14) DG_SUB_LSQ(16)
-#undef DG_SUB_LSQ
-    default: sub_lsq_combine_kernel<T><<<grid, block, 0, s>>>(E, nS, stride, m, beta, H, Z, duS);
-  }
-  DG_LAUNCHED(1);
-}
-template void launch_sub_normalize<double>(int, int, const double*, double*, double*, cudaStream_t);
-template void launch_sub_normalize<float>(int, int, const float*, float*, float*, cudaStream_t);
-template void launch_sub_arnoldi<double>(int, int, int, int, const double*, double*, const double*, double*,
-                                         cudaStream_t);
-template void launch_sub_arnoldi<float>(int, int, int, int, const float*, float*, const float*, float*, cudaStream_t);
-template void launch_sub_lsq_combine<double>(int, int, int, const double*, const double*, const double*, double*,
-                                             cudaStream_t);
-template void launch_sub_lsq_combine<float>(int, int, int, const float*, const float*, const float*, float*,
-                                            cudaStream_t);
-
+template void launch_sub_arnoldi<double>(int, int, int, int, const double*, const double*, double*, const double*,
+                                         double*, double*, double*, cudaStream_t);
+template void launch_sub_arnoldi<float>(int, int, int, int, const float*, const float*, float*, const float*, float*,
+                                        float*, float*, cudaStream_t);
 
 template void launch_class_gemm_tiles<double>(const double*, const double*, double*, int, const int4*, int,
                                                const int*, double, cudaStream_t, int);

@@ -193,7 +193,6 @@ void classify_schwarz(dg_domain* dom, Level& L) {
     }
   }
   cudaStream_t s = dom->stream;
-  upload(sw.elem_of_col, elem_of_col, s);
   upload(sw.col_of_elem, sw.position, s);
   {
     std::vector<int> class_of_col(E);
@@ -295,7 +294,7 @@ void classify_schwarz(dg_domain* dom, Level& L) {
 void build_orientation_tables(dg_domain* dom) {
   const int N = dom->N, N2 = N * N, N3 = N2 * N, ov = dom->desc.overlap;
   const int nS = N3 + 6 * ov * N2;
-  std::vector<int> map((size_t)48 * nS), inv((size_t)48 * 7 * N3, -1);
+  std::vector<int> inv((size_t)48 * 7 * N3, -1);
   for (int pi = 0; pi < 6; ++pi)
     for (int fl = 0; fl < 8; ++fl) {
       const int o = pi * 8 + fl;
@@ -326,7 +325,6 @@ void build_orientation_tables(dg_domain* dom) {
           ca[d] = ((fl >> a) & 1) ? N - 1 - cc[a] : cc[a];
         }
         const int p = (ca[2] * N + ca[1]) * N + ca[0];
-        map[(size_t)o * nS + q] = (slot << 16) | p;
         inv[((size_t)o * 7 + slot) * N3 + p] = q;
       }
     }
@@ -346,8 +344,6 @@ void build_orientation_tables(dg_domain* dom) {
       DG_REQUIRE(row[p] < 0 || row[p] == aff[os].x + s[0] * (p % N) + s[1] * ((p / N) % N) + s[2] * (p / N2),
                  "subdomain rows are not affine in the point indices");
   }
-  upload(dom->orient_map, map, dom->stream);
-  upload(dom->orient_inv, inv, dom->stream);
   upload(dom->orient_aff, aff, dom->stream);
 }
 
@@ -363,7 +359,9 @@ void build_shares(dg_domain* dom) {
     }
     for (int p = 0; p < N3; ++p) {
       const int c[3] = {p % N, (p / N) % N, p / (N * N)};
-      point_shares(dom->lgl, ov, has_lo, has_hi, c, &sh[((size_t)pat * N3 + p) * 7]);
+      double share[7];
+      point_shares(dom->lgl, ov, has_lo, has_hi, c, share);
+      for (int sl = 0; sl < 7; ++sl) sh[((size_t)pat * 7 + sl) * N3 + p] = share[sl];
     }
   }
   if (dom->mixed) {
@@ -619,6 +617,9 @@ void ensure_schwarz(dg_domain* dom, int level) {
   Level& L = dom->levels[level];
   SchwarzLevel& sw = L.sw;
   if (sw.built) return;
+  sw.rec.alloc((size_t)7 * L.E);
+  launch_subdomain_records(sw.geom, sw.col_of_elem.get(), sw.xform_of_elem.get(), dom->orient_aff.get(), sw.rec.get(),
+                           dom->stream);
   if (dom->curved) {
     cudaStream_t s = dom->stream;
     sw.inv_scale = 1.0;
@@ -770,22 +771,22 @@ size_t domain_device_bytes(const dg_domain* dom) {
              dom->lin64.bytes() + dom->lin32.bytes() + dom->V.bytes() + dom->Zb.bytes() + dom->w.bytes() +
              dom->r.bytes() + dom->du.bytes() + dom->ut.bytes() + dom->rt.bytes() + dom->tmp.bytes() +
              dom->partial.bytes() + dom->dots.bytes() + dom->vin32.bytes() + dom->shares64.bytes() +
-             dom->shares32.bytes() + dom->orient_map.bytes() + dom->orient_inv.bytes() + dom->orient_aff.bytes() + dom->vin64.bytes() +
+             dom->shares32.bytes() + dom->orient_aff.bytes() + dom->vin64.bytes() +
              dom->vout64.bytes() + dom->err_flag.bytes();
   for (const auto& L : dom->levels) {
     const auto& sw = L.sw;
     b += L.geo64.bytes() + L.geo32.bytes() + L.sig64.bytes() + L.sig32.bytes() + L.trace64.bytes() +
          L.trace32.bytes();
-    b += sw.elem_of_col.bytes() + sw.col_of_elem.bytes() + sw.class_of_col.bytes() + sw.xform_of_elem.bytes() +
+    b += sw.rec.bytes() + sw.col_of_elem.bytes() + sw.class_of_col.bytes() + sw.xform_of_elem.bytes() +
          sw.inv64.bytes() +
          sw.inv32.bytes() + sw.inv16.bytes() + sw.inv16_scale.bytes() + sw.tiles.bytes() + sw.tiles_tc.bytes() +
          sw.tiles_tc128.bytes() + sw.tiles_tc256.bytes() +
          sw.units.bytes() + sw.bar.bytes() + sw.inv_digits.bytes() + sw.inv_row_exp.bytes() + sw.x_digits.bytes() +
          sw.x_exp.bytes() + sw.inv_hexp.bytes() + sw.tiles_f64.bytes();
-    for (auto* p : {&L.w64.b, &L.w64.u, &L.w64.r, &L.w64.rS, &L.w64.duS, &L.w64.gV, &L.w64.gZ, &L.w64.gW, &L.w64.gD,
+    for (auto* p : {&L.w64.b, &L.w64.u, &L.w64.r, &L.w64.rS, &L.w64.duS, &L.w64.gV, &L.w64.gZ, &L.w64.gD,
                     &L.w64.gH, &L.w64.linA, &L.w64.linv})
       b += p->bytes();
-    for (auto* p : {&L.w32.b, &L.w32.u, &L.w32.r, &L.w32.rS, &L.w32.duS, &L.w32.gV, &L.w32.gZ, &L.w32.gW, &L.w32.gD,
+    for (auto* p : {&L.w32.b, &L.w32.u, &L.w32.r, &L.w32.rS, &L.w32.duS, &L.w32.gV, &L.w32.gZ, &L.w32.gD,
                     &L.w32.gH, &L.w32.linA, &L.w32.linv})
       b += p->bytes();
   }

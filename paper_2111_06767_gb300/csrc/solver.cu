@@ -74,8 +74,7 @@ void curved_apply(dg_domain* dom, Level& L, const T* u, T* out, const T* b, cuda
   DG_REQUIRE(a.out != nullptr, "curved residual needs the level's work vectors");
   launch_curved_apply<T>(dom->N, a, L.E, s);
   if (so)
-    launch_gather_tab<T>(L.sw.geom, a.out, L.sw.elem_of_col.get(), L.sw.xform_of_elem.get(), dom->orient_map.get(),
-                         static_cast<T*>(so->rS), s);
+    launch_gather<T>(L.sw.geom, a.out, so->rec, static_cast<T*>(so->rS), s);
 }
 }  // namespace
 
@@ -310,6 +309,25 @@ void class_gemm<float>(dg_domain* dom, Level& L, const float* X, float* Y, cudaS
 }
 }  // namespace
 
+namespace {
+// gD = R_S D, the linearization's diagonal in the finest level's subdomain columns. It changes only
+// with the linearization, so the smoothing steps (and the graphs that replay them) share one gather.
+template <typename T>
+void gather_linearization(dg_domain* dom, cudaStream_t s) {
+  Level& L = dom->levels[0];
+  LevelWork<T>& W = work<T>(L);
+  if (W.gD_current) return;
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  DG_CUDA(cudaStreamIsCapturing(s, &cap));
+  if (W.gD.count < (size_t)L.E * L.sw.ld) {
+    W.gD.alloc((size_t)L.E * L.sw.ld);
+    DG_CUDA(cudaMemsetAsync(W.gD.get(), 0, W.gD.bytes(), s));  // rows that no point maps to
+  }
+  launch_gather<T>(L.sw.geom, lin_diag<T>(dom), L.sw.rec.get(), W.gD.get(), s);
+  W.gD_current = cap == cudaStreamCaptureStatusNone;
+}
+}  // namespace
+
 // Levels with at most this many elements are smoothed by the fused cooperative kernel (MIXED).
 constexpr int kCoarseFusedElems = 64;
 
@@ -334,11 +352,8 @@ void schwarz_smooth(dg_domain* dom, int level, const T* b, T* u, int iterations,
       CoarseArgs a{};
       const float* diag = (level == 0 && dom->lin_set && dom->lin32.get()) ? dom->lin32.get() : nullptr;
       a.ap = ApplyArgs<float>{L.g32, dom->D32.get(), dom->w32.get(), u, diag, b, nullptr, L.E, W.rS.get(), sw.ld,
-                              dom->desc.overlap, sw.col_of_elem.get(), sw.xform_of_elem.get(), dom->orient_aff.get()};
-      a.inv = dom->orient_inv.get();
+                              dom->desc.overlap, sw.rec.get()};
       a.sg = sw.geom;
-      a.elem_of_col = sw.elem_of_col.get();
-      a.map = dom->orient_map.get();
       a.shares = dom->shares32.get();
       a.duS = W.duS.get();
       a.invm = sw.inv32.get();
@@ -362,21 +377,20 @@ void schwarz_smooth(dg_domain* dom, int level, const T* b, T* u, int iterations,
   so.rS = W.rS.get();
   so.ld = sw.ld;
   so.ov = dom->desc.overlap;
-  so.col_of_elem = sw.col_of_elem.get();
-  so.orient = sw.xform_of_elem.get();
-  so.aff = dom->orient_aff.get();
+  so.rec = sw.rec.get();
   for (int it = 0; it < iterations; ++it) {
     const double sz = sizeof(T), vec = (double)L.E * sw.nS * sz;
     const int ld = sw.ld;
     if (it == 0 && u_is_zero) {
       // with u = 0 the residual is b itself: gather it into the subdomain vectors
       PhaseScope ps(dom->prof, DG_PHASE_GATHER, s, L.ndof * sz + vec, 0.0);
-      launch_gather_tab<T>(sw.geom, b, sw.elem_of_col.get(), sw.xform_of_elem.get(), dom->orient_map.get(), W.rS.get(),
-                           s);
+      launch_gather<T>(sw.geom, b, sw.rec.get(), W.rS.get(), s);
     } else {
       apply_T<T>(dom, level, u, nullptr, b, s, &so);  // r = b - A u, written straight into r_S
     }
     const bool linearized = linearized_level;
+    const int m = linearized && dom->subdomain_solver == 0 ? dom->subdomain_iterations : 0;
+    T *beta = nullptr, *y = nullptr;
     auto gemm = [&](const T* X, T* Y) {
       const double isz = (sizeof(T) == 4 && sw.inv16.get()) ? 2.0 : sz;  // FP16-stored inverses
       // algorithmic: each class's inverse and vectors at its real subdomain size (slots present)
@@ -393,39 +407,31 @@ void schwarz_smooth(dg_domain* dom, int level, const T* b, T* u, int iterations,
       launch_lin_gemv<T>(W.linv.get(), W.rS.get(), sw.nS, ld, L.E, W.duS.get(), s);
     } else {
       // GMRES on (A_S + D_S), right-preconditioned by the Poisson inverse A_S^-1 (Sec. III.E)
-      const int m = dom->subdomain_iterations;
       const size_t blk = (size_t)L.E * ld;
-      if (W.gV.count < (m + 1) * blk) {
-        W.gV.alloc((m + 1) * blk);
+      if (W.gV.count < (size_t)m * blk) {
+        W.gV.alloc(m * blk);
         W.gZ.alloc(m * blk);
-        W.gD.alloc(blk);
-        W.gH.alloc((size_t)L.E * ((m + 1) * m + 1));
+        W.gH.alloc((size_t)L.E * ((m + 1) * m + 1 + m));
       }
-      T* beta = W.gH.get() + (size_t)L.E * (m + 1) * m;
-      launch_gather_tab<T>(sw.geom, lin_diag<T>(dom), sw.elem_of_col.get(), sw.xform_of_elem.get(),
-                           dom->orient_map.get(), W.gD.get(), s);
-      // the per-subdomain vector kernels count as Krylov work, the preconditioner GEMMs as GEMM
-      {
-        PhaseScope ps(dom->prof, DG_PHASE_KRYLOV, s, 2.0 * blk * sz, 2.0 * blk);
-        launch_sub_normalize<T>(L.E, ld, W.rS.get(), W.gV.get(), beta, s);
-      }
+      gather_linearization<T>(dom, s);
+      beta = W.gH.get() + (size_t)L.E * (m + 1) * m;
+      y = beta + L.E;
       for (int j = 0; j < m; ++j) {
-        gemm(W.gV.get() + j * blk, W.gZ.get() + j * blk);
-        // read V_j, D, Z_j and V_0..V_j, write V_{j+1}
-        PhaseScope ps(dom->prof, DG_PHASE_KRYLOV, s, (double)blk * sz * (j + 5.0), 4.0 * blk * (j + 2.0));
-        launch_sub_arnoldi<T>(L.E, ld, j, m, W.gD.get(), W.gV.get(), W.gZ.get(), W.gH.get(), s);
-      }
-      {
-        PhaseScope ps(dom->prof, DG_PHASE_KRYLOV, s, (double)blk * sz * (m + 1.0), 2.0 * blk * m);
-        launch_sub_lsq_combine<T>(L.E, ld, m, beta, W.gH.get(), W.gZ.get(), W.duS.get(), s);
+        // Z_j = A_S^-1 V_j (V_0 as r_S, unscaled)
+        gemm(j == 0 ? W.rS.get() : W.gV.get() + (j - 1) * blk, W.gZ.get() + j * blk);
+        // the per-subdomain vector kernels count as Krylov work, the preconditioner GEMMs as GEMM: read
+        // V_j, D, Z_j and V_0..V_{j-1}, write V_{j+1} (but the last)
+        PhaseScope ps(dom->prof, DG_PHASE_KRYLOV, s, (double)blk * sz * (j + (j + 1 < m ? 4.0 : 3.0)),
+                      4.0 * blk * (j + 2.0));
+        launch_sub_arnoldi<T>(L.E, ld, j, m, W.rS.get(), W.gD.get(), W.gV.get(), W.gZ.get(), W.gH.get(), beta, y, s);
       }
     }
     {
       // mode 3: the fine level's scatter also overlaps the GEMM before it
       const PdlScope pdl_scatter(sizeof(T) == 4 && level == 0 && pdl_vcycle_mode() == 3);
-      PhaseScope ps(dom->prof, DG_PHASE_SCATTER, s, vec + 2.0 * L.ndof * sz, 0.0);
-      launch_scatter_tab<T, T>(sw.geom, W.duS.get(), sw.col_of_elem.get(), sw.xform_of_elem.get(),
-                               dom->orient_inv.get(), shares<T>(dom), u, s);
+      PhaseScope ps(dom->prof, DG_PHASE_SCATTER, s, std::max(m, 1) * vec + 2.0 * L.ndof * sz, 0.0);
+      launch_scatter<T>(sw.geom, m > 0 ? W.gZ.get() : W.duS.get(), y, m, (int64_t)L.E * ld, sw.rec.get(),
+                        shares<T>(dom), u, s);
     }
   }
 }
@@ -1205,11 +1211,9 @@ void build_linearized_inverses(dg_domain* dom, cudaStream_t s) {
     DG_CUDA(cudaStreamSynchronize(s));
   }
   if (W.linv.count < (size_t)E * n2) W.linv.alloc((size_t)E * n2);
-  if (W.gD.count < (size_t)E * ld) W.gD.alloc((size_t)E * ld);
   const double sz = sizeof(T);
   PhaseScope ps(dom->prof, DG_PHASE_SUBDOMAIN_BUILD, s, 3.0 * E * n2 * sz, 2.0 * E * (double)n2 * nS);
-  launch_gather_tab<T>(sw.geom, lin_diag<T>(dom), sw.elem_of_col.get(), sw.xform_of_elem.get(), dom->orient_map.get(),
-                       W.gD.get(), s);
+  gather_linearization<T>(dom, s);
   launch_lin_assemble<T>(W.linA.get(), sw.class_of_col.get(), W.gD.get(), nS, ld, E, W.linv.get(), s);
   constexpr int kMaxBatch = 65535;  // grid z limit of the Gauss-Jordan update kernel
   for (int c0 = 0; c0 < E; c0 += kMaxBatch)
@@ -1228,7 +1232,14 @@ void set_linearization(dg_domain* dom, const double* u, cudaStream_t s) {
                                 dom->lin64.get(), dom->lin32.get(), s);
   dom->lin_set = true;
   dom->linv_current = false;
-  if (dom->subdomain_solver == 1) build_linearized(dom, s);
+  Level& L = dom->levels[0];
+  L.w64.gD_current = L.w32.gD_current = false;
+  if (dom->subdomain_solver == 1) {
+    build_linearized(dom, s);
+  } else if (L.sw.built) {  // replayed graphs hold the smoothing steps only
+    if (dom->mixed) gather_linearization<float>(dom, s);
+    else gather_linearization<double>(dom, s);
+  }
 }
 
 // r = b - A(u)
