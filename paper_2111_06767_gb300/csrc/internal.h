@@ -213,9 +213,10 @@ void launch_subdomain_records(const SubdomainGeom& g, const int* col_of_elem, co
 template <typename T>
 void launch_gather(const SubdomainGeom& g, const T* r, const int4* rec, T* rS, cudaStream_t s);
 // u += sum_S R_S^T w_S du_S, du_S = X (m = 0, y unused) or sum_{c < m} y[column][c] X_c, X_c = X + c stride.
+// u_zero: u counts as zero and is not read.
 template <typename T>
 void launch_scatter(const SubdomainGeom& g, const T* X, const T* y, int m, int64_t stride, const int4* rec,
-                    const T* shares, T* u, cudaStream_t s);
+                    const T* shares, T* u, bool u_zero, cudaStream_t s);
 template <typename S, typename T>
 void launch_pad_convert(const S* src, int n, int ld, int n_classes, T* dst, cudaStream_t s);
 
@@ -359,6 +360,7 @@ void launch_add_combination(int64_t n, int m, const double* Z, int64_t ld, const
 int multidot_partial_blocks();
 
 // Device-resident flexible GMRES (krylov_dev.cu): the state of one solve, in device memory.
+constexpr int kKrGraphCap = 40;  // Arnoldi columns a captured solve holds
 enum { KR_RUNNING = 0, KR_CONVERGED = 1, KR_BREAKDOWN = 2, KR_CAP = 3, KR_CANCELLED = 4 };
 struct KrylovState {
   int j;           // column the running iteration computes (V_j, Z_j)
@@ -367,6 +369,7 @@ struct KrylovState {
   int max_it;      // columns allowed (input)
   int rel_to_b;    // tolerance relative to ||b|| (input) instead of ||b - A x0||
   int runs;        // loop bodies executed (Arnoldi iterations attempted)
+  unsigned arrived;  // blocks of the running reduction that have finished
   double tol;      // relative tolerance (input)
   double tol_abs;  // absolute threshold on the residual estimate
   double beta;     // ||b - A x0||
@@ -376,19 +379,15 @@ struct KrylovState {
 void launch_kr_start(KrylovState* st, double tol, int max_it, bool rel_to_b, const double* nrm2, double* g,
                      cudaGraphConditionalHandle loop, cudaStream_t s);
 void launch_kr_report(const KrylovState* st, const double* nrm2, double* out, cudaStream_t s);
-void launch_kr_scale_into_v(int64_t n, const double* x, const KrylovState* st, double* V, int64_t ld, cudaStream_t s);
 template <typename T>
-void launch_kr_load_v(int64_t n, const double* V, int64_t ld, const KrylovState* st, T* out, cudaStream_t s);
+void launch_kr_next_v(int64_t n, const double* x, const KrylovState* st, double* V, int64_t ld, T* vin,
+                      cudaStream_t s);
 template <typename T>
 void launch_kr_store_z(int64_t n, const T* z, const KrylovState* st, double* Z, int64_t ld, double* zfix,
                        cudaStream_t s);
-void launch_kr_multidot(int64_t n, int cap, const double* V, int64_t ld, const double* w, const KrylovState* st,
-                        double* partial, double* out, cudaStream_t s);
-void launch_kr_sub_comb(int64_t n, const double* V, int64_t ld, const double* h, const KrylovState* st, double* w,
-                        cudaStream_t s);
-void launch_kr_givens(KrylovState* st, double* H, int ldh, double* cs, double* sn, double* g, const double* h1,
-                      const double* h2, const double* nrm2, const volatile int* cancel,
-                      cudaGraphConditionalHandle loop, cudaStream_t s);
+void launch_kr_orthogonalize(int64_t n, const double* V, int64_t ld, double* w, KrylovState* st, double* partial,
+                             double* H, int ldh, double* cs, double* sn, double* g, double* h1, double* h2,
+                             const volatile int* cancel, cudaGraphConditionalHandle loop, cudaStream_t s);
 void launch_kr_trisolve(const KrylovState* st, const double* H, int ldh, const double* g, double* y, cudaStream_t s);
 void launch_kr_add_comb(int64_t n, const double* Z, int64_t ld, const double* y, const KrylovState* st, double* x,
                         cudaStream_t s);

@@ -5,10 +5,15 @@
 //
 // Every kernel here reads the iteration index j (and the column count m = j + 1) from the solve's
 // state in device memory rather than from launch arguments, so the same captured launches serve
-// every iteration: V_j and Z_j are addressed as V + j ld and Z + j ld inside the kernels. The
-// reductions are the same fixed-shape two-pass trees as the host-driven solver's multi-dot
-// (per-block partial sums over the same chunks, summed in the same order), so the inner products,
-// and with them the Krylov basis, are the same bit for bit.
+// every iteration: V_j and Z_j are addressed as V + j ld and Z + j ld inside the kernels.
+//
+// An iteration's vector work is four launches besides Z_j: the first Gram-Schmidt pass's inner products;
+// its update fused with the second pass's products (a block's tile of every V_k is read twice, the second
+// time from L1); the second update fused with the norm, the rotations and the stopping decision; V_{j+1}
+// together with the next preconditioner input. The block that arrives last at a counter in the state sums
+// the partial products in a fixed order, so the results do not depend on which block that is. At 262,144
+// points the ten kernels this replaces (a partial and a final reduction kernel per pass and 40 rows of
+// blocks of which most returned at once) took about twice as long: 4.21 -> 3.85 ms a solve of 10 iterations.
 #include "internal.h"
 #include "pdl.cuh"
 
@@ -37,6 +42,7 @@ __global__ void kr_start_kernel(KrylovState* st, double tol, int max_it, int rel
   st->j = 0;
   st->k = 0;
   st->runs = 0;
+  st->arrived = 0;
   st->est = beta;
   g[0] = beta;
   int status = KR_RUNNING;
@@ -48,27 +54,21 @@ __global__ void kr_start_kernel(KrylovState* st, double tol, int max_it, int rel
   cudaGraphSetConditional(loop, status == KR_RUNNING ? 1u : 0u);
 }
 
-// V_j = scale x while the loop runs (j and scale from the state)
-__global__ void kr_scale_into_v_kernel(int64_t n, const double* __restrict__ x, const KrylovState* __restrict__ st,
-                                       double* __restrict__ V, int64_t ld) {
+// V_j = scale x and the preconditioner's input, V_j in FP32 (MIXED) or FP64, while the loop runs (j and
+// scale from the state)
+template <typename T>
+__global__ void kr_next_v_kernel(int64_t n, const double* __restrict__ x, const KrylovState* __restrict__ st,
+                                 double* __restrict__ V, int64_t ld, T* __restrict__ vin) {
   pdl_launch_dependents();
   pdl_wait();  // the state and vectors come from the previous kernel
   if (st->status != KR_RUNNING) return;
   const double a = st->scale;
   double* v = V + (int64_t)st->j * ld;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-    v[i] = a * x[i];
-}
-
-// the preconditioner's input: V_j, in FP32 (MIXED) or FP64
-template <typename T>
-__global__ void kr_load_v_kernel(int64_t n, const double* __restrict__ V, int64_t ld,
-                                 const KrylovState* __restrict__ st, T* __restrict__ out) {
-  pdl_launch_dependents();
-  pdl_wait();  // the state and vectors come from the previous kernel
-  const double* v = V + (int64_t)st->j * ld;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-    out[i] = (T)v[i];
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+    const double y = a * x[i];
+    v[i] = y;
+    vin[i] = (T)y;
+  }
 }
 
 // Z_j = z (the flexible basis keeps every preconditioned vector) and zfix = z, the fixed input of
@@ -86,75 +86,129 @@ __global__ void kr_store_z_kernel(int64_t n, const T* __restrict__ z, const Kryl
   }
 }
 
-// partial[k * blocks + bx] = this block's chunk of V_k . w for k <= j: the host solver's multi-dot
-// partial pass with the vector count read from the state (rows k > j of the grid exit at once)
-__global__ void kr_multidot_partial_kernel(int64_t n, const double* __restrict__ V, int64_t ld,
-                                           const double* __restrict__ w, const KrylovState* __restrict__ st,
-                                           double* __restrict__ partial, int blocks) {
-  pdl_launch_dependents();
-  pdl_wait();  // the state and vectors come from the previous kernel
-  const int k = blockIdx.y;
-  if (k > st->j) return;
-  __shared__ double red[kThreads / 32];
-  const double* v = V + (int64_t)k * ld;
-  const int64_t chunk = (n + blocks - 1) / blocks;
-  const int64_t lo = blockIdx.x * chunk, hi = min(n, lo + chunk);
-  double acc = 0.0;
-  for (int64_t i = lo + threadIdx.x; i < hi; i += blockDim.x) acc += v[i] * w[i];
+constexpr int kTile = 1024;                        // points of a block's tile, 4 per thread
+constexpr int kKrWarps = kThreads / 32;
+constexpr int kVecsPerWarp = (kKrGraphCap + kKrWarps - 1) / kKrWarps;  // inner products a warp accumulates
+static_assert(kTile == 4 * kThreads, "a thread updates four points of a tile");
+
+__device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+  return v;
+}
+
+// Inner products of a tile (in shared memory, `count` points, zeros after them) with V_0 .. V_{m-1}: warp
+// wid adds its vectors wid, wid + 8, ..; with few vectors the warps share a vector's points in ns parts.
+__device__ __forceinline__ void tile_dots(const double* sw, int64_t lo, int count, const double* V, int64_t ld, int m,
+                                          int ns, double (&acc)[kVecsPerWarp]) {
+  const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int part = wid % ns, first = wid / ns, step = kKrWarps / ns, per = kTile / ns;
+#pragma unroll
+  for (int q = 0; q < kVecsPerWarp; ++q) {
+    const int k = first + q * step;
+    if (k >= m) break;
+    const double* v = V + (int64_t)k * ld + lo;
+    double a0 = 0.0, a1 = 0.0;
+#pragma unroll 4
+    for (int i = part * per + lane; i < (part + 1) * per; i += 64) {
+      if (i < count) a0 += sw[i] * v[i];
+      if (i + 32 < count) a1 += sw[i + 32] * v[i + 32];
+    }
+    acc[q] += a0 + a1;
+  }
+}
+
+// True in the block that arrives last of the launch (whose writes, and everyone's before, it then sees).
+__device__ __forceinline__ bool last_block(KrylovState* st) {
+  __shared__ int s_last;
+  __threadfence();
   __syncthreads();
   if (threadIdx.x == 0) {
+    s_last = atomicAdd(&st->arrived, 1u) == gridDim.x - 1;
+    if (s_last) st->arrived = 0;
+  }
+  __syncthreads();
+  if (s_last) __threadfence();
+  return s_last;
+}
+
+// The block's accumulated products into partial[k * blocks + block], the last block's sums into h[k].
+__device__ __forceinline__ void finish_dots(KrylovState* st, int m, int ns, const double (&acc)[kVecsPerWarp],
+                                            double* partial, double* __restrict__ h) {
+  __shared__ double red[kKrWarps][kVecsPerWarp];
+  const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31, blocks = gridDim.x;
+#pragma unroll
+  for (int q = 0; q < kVecsPerWarp; ++q) {
+    const double t = warp_sum(acc[q]);
+    if (lane == 0) red[wid][q] = t;
+  }
+  __syncthreads();
+  const int step = kKrWarps / ns;
+  for (int k = threadIdx.x; k < m; k += kThreads) {
     double t = 0.0;
-    for (int q = 0; q < kThreads / 32; ++q) t += red[q];
+    for (int p = 0; p < ns; ++p) t += red[(k % step) * ns + p][k / step];
     partial[(int64_t)k * blocks + blockIdx.x] = t;
   }
-}
-
-__global__ void kr_multidot_final_kernel(const double* __restrict__ partial, const KrylovState* __restrict__ st,
-                                         double* __restrict__ out, int blocks) {
-  pdl_launch_dependents();
-  pdl_wait();  // the state and vectors come from the previous kernel
-  const int k = blockIdx.x;
-  if (k > st->j) return;
-  __shared__ double red[kThreads / 32];
-  double acc = 0.0;
-  for (int q = threadIdx.x; q < blocks; q += blockDim.x) acc += partial[(int64_t)k * blocks + q];
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
-  __syncthreads();
-  if (threadIdx.x == 0) {
+  if (!last_block(st)) return;
+  for (int k = wid; k < m; k += kKrWarps) {
     double t = 0.0;
-    for (int q = 0; q < kThreads / 32; ++q) t += red[q];
-    out[k] = t;
+    for (int b = lane; b < blocks; b += 32) t += __ldcg(partial + (int64_t)k * blocks + b);
+    t = warp_sum(t);
+    if (lane == 0) h[k] = t;
   }
 }
 
-// w -= sum_{k <= j} h[k] V_k
-__global__ void kr_sub_comb_kernel(int64_t n, const double* __restrict__ V, int64_t ld, const double* __restrict__ h,
-                                   const KrylovState* __restrict__ st, double* __restrict__ w) {
+__device__ __forceinline__ int vector_parts(int m) { return m == 1 ? 8 : (m == 2 ? 4 : (m <= 4 ? 2 : 1)); }
+
+// UPDATE = false: h2 = V^T w. UPDATE = true: w -= V h1, then h2 = V^T w.
+template <bool UPDATE>
+__global__ void __launch_bounds__(kThreads) kr_dots_kernel(int64_t n, const double* __restrict__ V, int64_t ld,
+                                                           const double* __restrict__ h1, double* w, KrylovState* st,
+                                                           double* partial, double* __restrict__ h2) {
+  __shared__ double sw[kTile];
   pdl_launch_dependents();
   pdl_wait();  // the state and vectors come from the previous kernel
-  const int m = st->j + 1;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    double acc = w[i];
-    for (int k = 0; k < m; ++k) acc -= h[k] * V[(int64_t)k * ld + i];
-    w[i] = acc;
+  const int m = st->j + 1, ns = vector_parts(m);
+  double acc[kVecsPerWarp] = {};
+  for (int64_t lo = blockIdx.x * (int64_t)kTile; lo < n; lo += gridDim.x * (int64_t)kTile) {
+    const int count = (int)min((int64_t)kTile, n - lo);
+    double x[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int i = threadIdx.x + q * kThreads;
+      x[q] = i < count ? w[lo + i] : 0.0;
+    }
+    if constexpr (UPDATE) {
+#pragma unroll 2
+      for (int k = 0; k < m; ++k) {
+        const double c = h1[k];
+        const double* v = V + (int64_t)k * ld + lo;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const int i = threadIdx.x + q * kThreads;
+          if (i < count) x[q] -= c * v[i];
+        }
+      }
+    }
+    __syncthreads();  // the previous tile has been read
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int i = threadIdx.x + q * kThreads;
+      sw[i] = x[q];
+      if (UPDATE && i < count) w[lo + i] = x[q];
+    }
+    __syncthreads();
+    tile_dots(sw, lo, count, V, ld, m, ns, acc);
   }
+  finish_dots(st, m, ns, acc, partial, h2);
 }
 
 // Column j of the Hessenberg matrix from the two Gram-Schmidt passes, the previous rotations
 // applied to it, the new rotation, the residual estimate |g_{j+1}| and the stopping decision; while
 // the loop continues, the scale 1 / h_{j+1,j} of the next basis vector and j + 1. One thread.
-__global__ void kr_givens_kernel(KrylovState* st, double* __restrict__ H, int ldh, double* __restrict__ cs,
-                                 double* __restrict__ sn, double* __restrict__ g, const double* __restrict__ h1,
-                                 const double* __restrict__ h2, const double* __restrict__ nrm2,
-                                 const volatile int* cancel, cudaGraphConditionalHandle loop) {
-  pdl_launch_dependents();
-  pdl_wait();  // the state and vectors come from the previous kernel
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
+__device__ void kr_givens(KrylovState* st, double* __restrict__ H, int ldh, double* __restrict__ cs,
+                          double* __restrict__ sn, double* __restrict__ g, const double* h1, const double* h2,
+                          double nrm2, const volatile int* cancel, cudaGraphConditionalHandle loop) {
   if (st->status != KR_RUNNING) {
     cudaGraphSetConditional(loop, 0u);
     return;
@@ -163,7 +217,7 @@ __global__ void kr_givens_kernel(KrylovState* st, double* __restrict__ H, int ld
   st->runs = j + 1;
   double* col = H + (int64_t)j * ldh;
   for (int i = 0; i <= j; ++i) col[i] = h1[i] + h2[i];
-  const double hn = sqrt(fmax(0.0, nrm2[0]));
+  const double hn = sqrt(fmax(0.0, nrm2));
   col[j + 1] = hn;
   for (int i = 0; i < j; ++i) {  // previous rotations
     const double a = col[i], c = col[i + 1];
@@ -195,6 +249,58 @@ __global__ void kr_givens_kernel(KrylovState* st, double* __restrict__ H, int ld
     st->j = j + 1;
   }
   cudaGraphSetConditional(loop, status == KR_RUNNING ? 1u : 0u);
+}
+
+// w -= V h2, its norm, then in the last block the rotations and the stopping decision.
+__global__ void __launch_bounds__(kThreads)
+    kr_finish_kernel(int64_t n, const double* __restrict__ V, int64_t ld, const double* __restrict__ h1,
+                     const double* __restrict__ h2, double* w, KrylovState* st, double* partial, double* __restrict__ H,
+                     int ldh, double* __restrict__ cs, double* __restrict__ sn, double* __restrict__ g,
+                     const volatile int* cancel, cudaGraphConditionalHandle loop) {
+  __shared__ double red[kKrWarps];
+  pdl_launch_dependents();
+  pdl_wait();  // the state and vectors come from the previous kernel
+  const int m = st->j + 1;
+  double acc = 0.0;
+  for (int64_t lo = blockIdx.x * (int64_t)kTile; lo < n; lo += gridDim.x * (int64_t)kTile) {
+    const int count = (int)min((int64_t)kTile, n - lo);
+    double x[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int i = threadIdx.x + q * kThreads;
+      x[q] = i < count ? w[lo + i] : 0.0;
+    }
+#pragma unroll 2
+    for (int k = 0; k < m; ++k) {
+      const double c = h2[k];
+      const double* v = V + (int64_t)k * ld + lo;
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int i = threadIdx.x + q * kThreads;
+        if (i < count) x[q] -= c * v[i];
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int i = threadIdx.x + q * kThreads;
+      if (i < count) w[lo + i] = x[q];
+      acc += x[q] * x[q];
+    }
+  }
+  const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  acc = warp_sum(acc);
+  if (lane == 0) red[wid] = acc;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double t = 0.0;
+    for (int q = 0; q < kKrWarps; ++q) t += red[q];
+    partial[blockIdx.x] = t;
+  }
+  if (!last_block(st) || wid != 0) return;
+  double t = 0.0;
+  for (int b = lane; b < gridDim.x; b += 32) t += __ldcg(partial + b);
+  t = warp_sum(t);
+  if (lane == 0) kr_givens(st, H, ldh, cs, sn, g, h1, h2, t, cancel, loop);
 }
 
 // y = R^-1 g over the k completed columns (back substitution). One thread.
@@ -259,19 +365,17 @@ void launch_kr_report(const KrylovState* st, const double* nrm2, double* out, cu
   launch_pdl(kr_report_kernel, dim3(1), dim3(32), 0, s, st, nrm2, out);
   DG_LAUNCHED(1);
 }
-void launch_kr_scale_into_v(int64_t n, const double* x, const KrylovState* st, double* V, int64_t ld, cudaStream_t s) {
-  const PdlScope pdl(pdl_krylov_enabled());
-  launch_pdl(kr_scale_into_v_kernel, dim3(grid_for(n)), dim3(kThreads), 0, s, n, x, st, V, ld);
-  DG_LAUNCHED(1);
-}
 template <typename T>
-void launch_kr_load_v(int64_t n, const double* V, int64_t ld, const KrylovState* st, T* out, cudaStream_t s) {
+void launch_kr_next_v(int64_t n, const double* x, const KrylovState* st, double* V, int64_t ld, T* vin,
+                      cudaStream_t s) {
   const PdlScope pdl(pdl_krylov_enabled());
-  launch_pdl(kr_load_v_kernel<T>, dim3(grid_for(n)), dim3(kThreads), 0, s, n, V, ld, st, out);
+  launch_pdl(kr_next_v_kernel<T>, dim3(grid_for(n)), dim3(kThreads), 0, s, n, x, st, V, ld, vin);
   DG_LAUNCHED(1);
 }
-template void launch_kr_load_v<float>(int64_t, const double*, int64_t, const KrylovState*, float*, cudaStream_t);
-template void launch_kr_load_v<double>(int64_t, const double*, int64_t, const KrylovState*, double*, cudaStream_t);
+template void launch_kr_next_v<float>(int64_t, const double*, const KrylovState*, double*, int64_t, float*,
+                                      cudaStream_t);
+template void launch_kr_next_v<double>(int64_t, const double*, const KrylovState*, double*, int64_t, double*,
+                                       cudaStream_t);
 template <typename T>
 void launch_kr_store_z(int64_t n, const T* z, const KrylovState* st, double* Z, int64_t ld, double* zfix,
                        cudaStream_t s) {
@@ -283,27 +387,17 @@ template void launch_kr_store_z<float>(int64_t, const float*, const KrylovState*
                                        cudaStream_t);
 template void launch_kr_store_z<double>(int64_t, const double*, const KrylovState*, double*, int64_t, double*,
                                         cudaStream_t);
-void launch_kr_multidot(int64_t n, int cap, const double* V, int64_t ld, const double* w, const KrylovState* st,
-                        double* partial, double* out, cudaStream_t s) {
+// w orthogonalised against V_0 .. V_j (classical Gram-Schmidt, twice), column j and the decision.
+void launch_kr_orthogonalize(int64_t n, const double* V, int64_t ld, double* w, KrylovState* st, double* partial,
+                             double* H, int ldh, double* cs, double* sn, double* g, double* h1, double* h2,
+                             const volatile int* cancel, cudaGraphConditionalHandle loop, cudaStream_t s) {
   const PdlScope pdl(pdl_krylov_enabled());
-  const int blocks = multidot_partial_blocks();
-  launch_pdl(kr_multidot_partial_kernel, dim3(blocks, cap), dim3(kThreads), 0, s, n, V, ld, w, st, partial,
-             blocks);
-  launch_pdl(kr_multidot_final_kernel, dim3(cap), dim3(kThreads), 0, s, partial, st, out, blocks);
-  DG_LAUNCHED(2);
-}
-void launch_kr_sub_comb(int64_t n, const double* V, int64_t ld, const double* h, const KrylovState* st, double* w,
-                        cudaStream_t s) {
-  const PdlScope pdl(pdl_krylov_enabled());
-  launch_pdl(kr_sub_comb_kernel, dim3(grid_for(n)), dim3(kThreads), 0, s, n, V, ld, h, st, w);
-  DG_LAUNCHED(1);
-}
-void launch_kr_givens(KrylovState* st, double* H, int ldh, double* cs, double* sn, double* g, const double* h1,
-                      const double* h2, const double* nrm2, const volatile int* cancel,
-                      cudaGraphConditionalHandle loop, cudaStream_t s) {
-  const PdlScope pdl(pdl_krylov_enabled());
-  launch_pdl(kr_givens_kernel, dim3(1), dim3(32), 0, s, st, H, ldh, cs, sn, g, h1, h2, nrm2, cancel, loop);
-  DG_LAUNCHED(1);
+  const dim3 grid((unsigned)std::min<int64_t>((n + kTile - 1) / kTile, multidot_partial_blocks()));
+  launch_pdl(kr_dots_kernel<false>, grid, dim3(kThreads), 0, s, n, V, ld, (const double*)nullptr, w, st, partial, h1);
+  launch_pdl(kr_dots_kernel<true>, grid, dim3(kThreads), 0, s, n, V, ld, (const double*)h1, w, st, partial, h2);
+  launch_pdl(kr_finish_kernel, grid, dim3(kThreads), 0, s, n, V, ld, (const double*)h1, (const double*)h2, w, st,
+             partial, H, ldh, cs, sn, g, cancel, loop);
+  DG_LAUNCHED(3);
 }
 void launch_kr_trisolve(const KrylovState* st, const double* H, int ldh, const double* g, double* y, cudaStream_t s) {
   const PdlScope pdl(pdl_krylov_enabled());

@@ -424,7 +424,7 @@ template <int N, typename T, int M>
 __global__ void __launch_bounds__(256) scatter_kernel(SubdomainGeom g, const T* __restrict__ X,
                                                       const T* __restrict__ y, int m, int64_t stride,
                                                       const int4* __restrict__ rec, const T* __restrict__ shares,
-                                                      T* __restrict__ u) {
+                                                      T* __restrict__ u, int u_zero) {
   constexpr int N3 = N * N * N;
   const int t = blockIdx.x * 256 + threadIdx.x;
   pdl_launch_dependents();
@@ -436,7 +436,7 @@ __global__ void __launch_bounds__(256) scatter_kernel(SubdomainGeom g, const T* 
   scatter_look_up<N, T>(g, rec, shares, e, act ? t - e * N3 : 0, idx, col, w);
   pdl_wait();
   if (!act) return;
-  const T u0 = u[t];
+  const T u0 = u_zero ? T(0) : u[t];
   if constexpr (M == 0) {
 #pragma unroll
     for (int sl = 0; sl < 7; ++sl) v[sl] = idx[sl] >= 0 ? X[idx[sl]] : T(0);
@@ -458,11 +458,11 @@ __global__ void __launch_bounds__(256) scatter_kernel(SubdomainGeom g, const T* 
 
 template <int N, typename T>
 void launch_scatter_n(const SubdomainGeom& g, const T* X, const T* y, int m, int64_t stride, const int4* rec,
-                      const T* shares, T* u, cudaStream_t s) {
+                      const T* shares, T* u, int u_zero, cudaStream_t s) {
   const dim3 grid((g.E * N * N * N + 255) / 256);
-  if (m == 0) launch_pdl(scatter_kernel<N, T, 0>, grid, dim3(256), 0, s, g, X, y, m, stride, rec, shares, u);
-  else if (m == 3) launch_pdl(scatter_kernel<N, T, 3>, grid, dim3(256), 0, s, g, X, y, m, stride, rec, shares, u);
-  else launch_pdl(scatter_kernel<N, T, -1>, grid, dim3(256), 0, s, g, X, y, m, stride, rec, shares, u);
+  if (m == 0) launch_pdl(scatter_kernel<N, T, 0>, grid, dim3(256), 0, s, g, X, y, m, stride, rec, shares, u, u_zero);
+  else if (m == 3) launch_pdl(scatter_kernel<N, T, 3>, grid, dim3(256), 0, s, g, X, y, m, stride, rec, shares, u, u_zero);
+  else launch_pdl(scatter_kernel<N, T, -1>, grid, dim3(256), 0, s, g, X, y, m, stride, rec, shares, u, u_zero);
 }
 
 template <typename T>
@@ -481,11 +481,11 @@ void launch_gather(const SubdomainGeom& g, const T* r, const int4* rec, T* rS, c
 
 template <typename T>
 void launch_scatter(const SubdomainGeom& g, const T* X, const T* y, int m, int64_t stride, const int4* rec,
-                    const T* shares, T* u, cudaStream_t s) {
+                    const T* shares, T* u, bool u_zero, cudaStream_t s) {
   if (g.E == 0) return;
   switch (g.N) {
 #define DG_CASE(NN) \
-  case NN: launch_scatter_n<NN, T>(g, X, y, m, stride, rec, shares, u, s); break;
+  case NN: launch_scatter_n<NN, T>(g, X, y, m, stride, rec, shares, u, u_zero ? 1 : 0, s); break;
     DG_CASE(2) DG_CASE(3) DG_CASE(4) DG_CASE(5) DG_CASE(6) DG_CASE(7) DG_CASE(8) DG_CASE(9) DG_CASE(10)
 #undef DG_CASE
     default: fail(DG_ERR_INVALID_ARG, "unsupported N");
@@ -496,9 +496,9 @@ void launch_scatter(const SubdomainGeom& g, const T* X, const T* y, int m, int64
 template void launch_gather<double>(const SubdomainGeom&, const double*, const int4*, double*, cudaStream_t);
 template void launch_gather<float>(const SubdomainGeom&, const float*, const int4*, float*, cudaStream_t);
 template void launch_scatter<double>(const SubdomainGeom&, const double*, const double*, int, int64_t, const int4*,
-                                     const double*, double*, cudaStream_t);
+                                     const double*, double*, bool, cudaStream_t);
 template void launch_scatter<float>(const SubdomainGeom&, const float*, const float*, int, int64_t, const int4*,
-                                    const float*, float*, cudaStream_t);
+                                    const float*, float*, bool, cudaStream_t);
 
 // ------------------------------------------------------------------ class GEMM (SIMT)
 

@@ -431,7 +431,7 @@ void schwarz_smooth(dg_domain* dom, int level, const T* b, T* u, int iterations,
       const PdlScope pdl_scatter(sizeof(T) == 4 && level == 0 && pdl_vcycle_mode() == 3);
       PhaseScope ps(dom->prof, DG_PHASE_SCATTER, s, std::max(m, 1) * vec + 2.0 * L.ndof * sz, 0.0);
       launch_scatter<T>(sw.geom, m > 0 ? W.gZ.get() : W.duS.get(), y, m, (int64_t)L.E * ld, sw.rec.get(),
-                        shares<T>(dom), u, s);
+                        shares<T>(dom), u, it == 0 && u_is_zero, s);
     }
   }
 }
@@ -449,7 +449,11 @@ void vcycle(dg_domain* dom, const T* r, T* z, cudaStream_t s) {
   for (int l = 0; l < nl; ++l) ensure_schwarz(dom, l);
   auto B = [&](int l) -> const T* { return l == 0 ? r : work<T>(dom->levels[l]).b.get(); };
   auto U = [&](int l) -> T* { return l == 0 ? z : work<T>(dom->levels[l]).u.get(); };
-  for (int l = 0; l < nl; ++l) DG_CUDA(cudaMemsetAsync(U(l), 0, sizeof(T) * dom->levels[l].ndof, s));
+  // the first smoothing step of a level stores u instead of adding to it; only a level without one (and
+  // the fused coarse smoother) starts from a zeroed u
+  for (int l = 0; l < nl; ++l)
+    if ((pre == 0 && l < nl - 1) || dom->coarse_fused)
+      DG_CUDA(cudaMemsetAsync(U(l), 0, sizeof(T) * dom->levels[l].ndof, s));
   const PdlScope pdl(sizeof(T) == 4 && pdl_vcycle_mode() >= 2);  // transfers and residuals
   for (int l = 0; l < nl - 1; ++l) {
     Level& L = dom->levels[l];
@@ -734,13 +738,13 @@ LinearResult fgmres(dg_domain* dom, const double* b, double* x, double tol, doub
 //
 // The same method as fgmres() above with the Hessenberg column, the Givens rotations and the
 // stopping test on the device (krylov_dev.cu). A solve is one graph launch: prologue (r = b - A x,
-// norms, g_0, V_0), a conditional WHILE node whose body is one Arnoldi iteration (V_j into the
-// V-cycle's input, the V-cycle itself, Z_j, A Z_j, two classical Gram-Schmidt passes, the rotation
-// kernel that sets the loop condition, V_{j+1}), and the epilogue (y = R^-1 g, x += Z y, the true
+// norms, g_0, V_0), a conditional WHILE node whose body is one Arnoldi iteration (the
+// V-cycle, Z_j, A Z_j, two classical Gram-Schmidt passes with the rotations that set the loop condition,
+// V_{j+1} and the next V-cycle's input), and the epilogue (y = R^-1 g, x += Z y, the true
 // residual). The graph works on fixed buffers (b and x are copied in and out around the launch),
 // and holds at most kGraphCap Arnoldi columns: a solve that needs more continues host-driven from
 // the graph's iterate (a restart).
-constexpr int kGraphCap = 40;
+constexpr int kGraphCap = kKrGraphCap;
 
 // The captured solve's small device arrays, carved from one buffer.
 struct KrylovLayout {
@@ -865,7 +869,11 @@ void capture_solve_branch(dg_domain* dom, cudaGraph_t graph, int cap, double tol
     launch_multidot(n, 1, r, n, r, part, nrm, gs);
     if (rel_to_b) launch_multidot(n, 1, kb, n, kb, part, nrm + 1, gs);
     launch_kr_start(st, tol, cap, rel_to_b, nrm, g, loop, gs);
-    launch_kr_scale_into_v(n, r, st, V, n, gs);
+    auto next_v = [&](const double* x, cudaStream_t q) {  // V_j and the V-cycle's input
+      if (dom->mixed) launch_kr_next_v<float>(n, x, st, V, n, dom->vin32.get(), q);
+      else launch_kr_next_v<double>(n, x, st, V, n, dom->vin64.get(), q);
+    };
+    next_v(r, gs);
     // the Arnoldi loop: a conditional WHILE node after the prologue
     cudaStreamCaptureStatus cst;
     const cudaGraphNode_t* deps = nullptr;
@@ -886,22 +894,15 @@ void capture_solve_branch(dg_domain* dom, cudaGraph_t graph, int cap, double tol
     try {
       if (dom->mixed) {
         float* v32 = dom->vin32.get();
-        launch_kr_load_v<float>(n, V, n, st, v32, bs);
         vcycle<float>(dom, v32, v32 + n, bs);
         launch_kr_store_z<float>(n, v32 + n, st, Z, n, dom->zfix.get(), bs);
       } else {
-        launch_kr_load_v<double>(n, V, n, st, dom->vin64.get(), bs);
         vcycle<double>(dom, dom->vin64.get(), dom->vout64.get(), bs);
         launch_kr_store_z<double>(n, dom->vout64.get(), st, Z, n, dom->zfix.get(), bs);
       }
       apply_level(dom, 0, dom->zfix.get(), w, nullptr, true, bs);
-      launch_kr_multidot(n, cap, V, n, w, st, part, h1, bs);  // classical Gram-Schmidt, twice
-      launch_kr_sub_comb(n, V, n, h1, st, w, bs);
-      launch_kr_multidot(n, cap, V, n, w, st, part, h2, bs);
-      launch_kr_sub_comb(n, V, n, h2, st, w, bs);
-      launch_multidot(n, 1, w, n, w, part, nrm, bs);
-      launch_kr_givens(st, H, ldh, cs, sn, g, h1, h2, nrm, dom->cancel_dev, loop, bs);
-      launch_kr_scale_into_v(n, w, st, V, n, bs);
+      launch_kr_orthogonalize(n, V, n, w, st, part, H, ldh, cs, sn, g, h1, h2, dom->cancel_dev, loop, bs);
+      next_v(w, bs);
     } catch (...) {
       cudaGraph_t t = nullptr;
       cudaStreamEndCapture(bs, &t);
