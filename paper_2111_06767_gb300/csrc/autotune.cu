@@ -59,10 +59,9 @@ void keep_pool_memory() {
 AllocStreamScope::AllocStreamScope(cudaStream_t s) : prev(tl_alloc_stream) { tl_alloc_stream = s; }
 AllocStreamScope::~AllocStreamScope() { tl_alloc_stream = prev; }
 
-// Off by default for every launch: measured on the 8^3, N = 8 workload it slowed the FP64 solve
-// from 339 to 630 ms (dependent CTAs parked on the SMs during the long FP64 GEMMs) and the mixed one
-// from 5.55 to 5.78 ms. DG_PDL=1 turns it on everywhere; a PdlScope turns it on for the launches
-// made inside it on this thread (the coarse levels of the V-cycle, see schwarz_smooth).
+// Off by default for every launch: on levels with long kernels the dependent CTAs only hold SMs that
+// other work would use. DG_PDL=1 turns it on everywhere; a PdlScope turns it on for the launches made
+// inside it on this thread (levels small enough to gain, see level_pdl in solver.cu).
 namespace {
 thread_local int tl_pdl_scope = 0;
 }

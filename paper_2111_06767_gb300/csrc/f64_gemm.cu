@@ -172,7 +172,16 @@ __global__ void __launch_bounds__(THREADS, 1)
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = *tmem_slot;
+  // the inverse's first tiles, which nothing writes, overlap the previous kernel
   pdl_launch_dependents();
+  const int ahead = min(A_STAGES, nk * S);
+  if (warp == 8 && lane == 0) {
+    for (int q = 0; q < ahead; ++q) {
+      mbar_expect_tx(a_full + 8 * q, A_BYTES);
+      tma_load_3d(smem_u32(sA + q * A_BYTES), &mapA, a_full + 8 * q, kl[q / S] * BK, row0, cls * S + q % S);
+    }
+    s_count[0] = ahead;
+  }
   pdl_wait();
 
   bool ok = true;
@@ -188,7 +197,8 @@ __global__ void __launch_bounds__(THREADS, 1)
         s_count[2] = kc + 1;
         for (int i = 0; i < S; ++i) {
           const int q = kc * S + i, st = q % A_STAGES;
-          if (q >= A_STAGES && !(ok = mbar_wait(a_empty + 8 * st, ((q / A_STAGES) - 1) & 1, err))) break;
+          if (q < ahead) continue;
+          if (!(ok = mbar_wait(a_empty + 8 * st, ((q / A_STAGES) - 1) & 1, err))) break;
           mbar_expect_tx(a_full + 8 * st, A_BYTES);
           tma_load_3d(smem_u32(sA + st * A_BYTES), &mapA, a_full + 8 * st, k0, row0, cls * S + i);
           s_count[0] = q + 1;

@@ -331,12 +331,23 @@ void gather_linearization(dg_domain* dom, cudaStream_t s) {
 // Levels with at most this many elements are smoothed by the fused cooperative kernel (MIXED).
 constexpr int kCoarseFusedElems = 64;
 
+// Levels whose kernels are launched with programmatic dependent launch: those where each kernel is a
+// short latency chain, so that the next one's launch, set-up and first tiles of the inverse overlap it.
+// Above these sizes the waiting CTAs cost more than they hide. Mixed solve, 8^3 elements at N = 8: coarse
+// levels only 4.03 ms, all three levels 3.96; 20 uneven solves in one graph 23.2 and 22.5 ms; punctures with
+// 16^3 elements on the finest level 14.74 and 14.79. FP64 steps (tensor-core product, one CTA per SM): at 8
+// elements of N = 8 29.4 -> 27.0 us, at 64 elements 44.7 -> 67.8. DG_PDL_COARSE: 0 none, 2 every level.
+template <typename T>
+bool level_pdl(const Level& L) {
+  const int mode = pdl_vcycle_mode();
+  if (mode == 0 || (sizeof(T) == 8 && !L.sw.f64_tc)) return false;
+  return mode >= 2 || L.E <= (sizeof(T) == 4 ? 1024 : 32);
+}
+
 template <typename T>
 void schwarz_smooth(dg_domain* dom, int level, const T* b, T* u, int iterations, bool u_is_zero, cudaStream_t s) {
-  // FP32 coarse levels: each kernel is a short latency chain, so the next one's launch and set-up
-  // overlap it (programmatic dependent launch); the fine level and FP64 keep plain stream order
-  const PdlScope pdl(sizeof(T) == 4 && pdl_vcycle_mode() >= (level > 0 ? 1 : 2));
   ensure_schwarz(dom, level);
+  const PdlScope pdl(level_pdl<T>(dom->levels[level]));
   Level& L = dom->levels[level];
   LevelWork<T>& W = work<T>(L);
   SchwarzLevel& sw = L.sw;
@@ -427,8 +438,6 @@ void schwarz_smooth(dg_domain* dom, int level, const T* b, T* u, int iterations,
       }
     }
     {
-      // mode 3: the fine level's scatter also overlaps the GEMM before it
-      const PdlScope pdl_scatter(sizeof(T) == 4 && level == 0 && pdl_vcycle_mode() == 3);
       PhaseScope ps(dom->prof, DG_PHASE_SCATTER, s, std::max(m, 1) * vec + 2.0 * L.ndof * sz, 0.0);
       launch_scatter<T>(sw.geom, m > 0 ? W.gZ.get() : W.duS.get(), y, m, (int64_t)L.E * ld, sw.rec.get(),
                         shares<T>(dom), u, it == 0 && u_is_zero, s);
@@ -454,10 +463,11 @@ void vcycle(dg_domain* dom, const T* r, T* z, cudaStream_t s) {
   for (int l = 0; l < nl; ++l)
     if ((pre == 0 && l < nl - 1) || dom->coarse_fused)
       DG_CUDA(cudaMemsetAsync(U(l), 0, sizeof(T) * dom->levels[l].ndof, s));
-  const PdlScope pdl(sizeof(T) == 4 && pdl_vcycle_mode() >= 2);  // transfers and residuals
   for (int l = 0; l < nl - 1; ++l) {
     Level& L = dom->levels[l];
     schwarz_smooth<T>(dom, l, B(l), U(l), pre, true, s);
+    // residual and transfers as the level's smoothing (FP64 transfers are long: 602 against 578 us a V-cycle)
+    const PdlScope pdl(sizeof(T) == 4 && level_pdl<T>(L));
     apply_T<T>(dom, l, U(l), work<T>(L).r.get(), B(l), s);  // Eq. mg_res
     PhaseScope ps(dom->prof, DG_PHASE_TRANSFER, s, (double)(L.ndof + dom->levels[l + 1].ndof) * sizeof(T),
                   6.0 * N * L.ndof);
@@ -469,6 +479,7 @@ void vcycle(dg_domain* dom, const T* r, T* z, cudaStream_t s) {
   for (int l = nl - 2; l >= 0; --l) {
     Level& L = dom->levels[l];
     {
+      const PdlScope pdl(sizeof(T) == 4 && level_pdl<T>(L));
       PhaseScope ps(dom->prof, DG_PHASE_TRANSFER, s, (double)(2 * L.ndof + dom->levels[l + 1].ndof) * sizeof(T),
                     6.0 * N * L.ndof);
       launch_prolongate_add<T>(N, L.n, dom->levels[l + 1].n, Ilo<T>(dom), Ihi<T>(dom), U(l + 1), U(l), s);

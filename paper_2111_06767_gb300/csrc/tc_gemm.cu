@@ -101,18 +101,27 @@ __global__ void __launch_bounds__(128, TcShape<BN>::PER_SM)
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = *tmem_slot;
-  // set-up above overlaps the previous kernel; X (and Y) belong to the stream order from here on
+  // set-up above overlaps the previous kernel, and so do the first tiles of the inverse, which nothing
+  // writes; X (and Y) belong to the stream order from pdl_wait() on
   pdl_launch_dependents();
+  if (warp == 0 && lane == 0) {
+    for (int kc = 0; kc < nk && kc < STAGES; ++kc) {
+      mbar_expect_tx(full0 + 8 * kc, STAGE_BYTES);
+      tma_load_3d(smem_u32(sA + kc * A_BYTES), &mapA, full0 + 8 * kc, kl[kc0 + kc] * BK, row0, cls);
+    }
+  }
   pdl_wait();
 
   if (warp == 0 && lane == 0) {
-    // producer: TMA loads into the ring
+    // producer: TMA loads into the ring (its first round holds the inverse's tiles already)
     for (int kc = 0; kc < nk; ++kc) {
       const int s = kc % STAGES;
-      if (kc >= STAGES && !mbar_wait(empty0 + 8 * s, ((kc / STAGES) & 1) ^ 1, err)) break;
-      mbar_expect_tx(full0 + 8 * s, STAGE_BYTES);
       const int k0 = kl[kc0 + kc] * BK;
-      tma_load_3d(smem_u32(sA + s * A_BYTES), &mapA, full0 + 8 * s, k0, row0, cls);
+      if (kc >= STAGES) {
+        if (!mbar_wait(empty0 + 8 * s, ((kc / STAGES) & 1) ^ 1, err)) break;
+        mbar_expect_tx(full0 + 8 * s, STAGE_BYTES);
+        tma_load_3d(smem_u32(sA + s * A_BYTES), &mapA, full0 + 8 * s, k0, row0, cls);
+      }
       tma_load_2d(smem_u32(sB + s * B_BYTES), &mapB, full0 + 8 * s, k0, col0);
       *s_issued = kc + 1;
     }
