@@ -37,12 +37,11 @@ struct SchwarzLevel {
   DevBuf<int> kchunks32;           // the same for chunks of 32 (tensor-core GEMM)
   std::vector<int> class_nS;       // per class: rows of the slots present (its real subdomain size)
   double alg_inv = 0, alg_vec = 0, alg_mac = 0;  // sum_c nS_c^2, sum_c E_c nS_c, sum_c E_c nS_c^2
-  DevBuf<int4> tiles_tc;           // tensor-core GEMM tiles: 128 rows x 64 columns
-  int n_tiles_tc = 0;
-  DevBuf<int4> tiles_tc128;        // tensor-core GEMM tiles: 128 rows x 128 columns
-  int n_tiles_tc128 = 0;
-  DevBuf<int4> tiles_tc256;        // tensor-core GEMM tiles: 128 rows x 256 columns (one read of a
-  int n_tiles_tc256 = 0;           //   128-row slab of the inverse per class of at most 256 columns)
+  // tensor-core GEMM tiles: 128 rows x a class's columns in equal parts of at most 64 or 128
+  struct TcTiles {
+    DevBuf<int4> d;
+    int n = 0, widths = 0;  // tiles, mask of their width codes
+  } tiles_tc[2];
   // FP64 domains on the tensor cores: digit slices of the scaled inverses [class][8][ld][ld] with their
   // row and equilibration exponents [class][ld], tiles of 128 rows x 16..48 columns, K chunks of 64, and the slices of r_S
   bool f64_tc = false;

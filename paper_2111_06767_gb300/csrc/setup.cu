@@ -260,24 +260,21 @@ void classify_schwarz(dg_domain* dom, Level& L) {
   }
   sw.n_tiles_f64 = (int)tiles_f64.size();
   upload(sw.tiles_f64, tiles_f64, s);
-  std::vector<int4> tiles_tc;
-  for (int c = 0; c < (dom->curved ? 0 : nc); ++c)
-    for (int r0 = 0; r0 < sw.ld; r0 += 128)
-      for (int c0 = 0; c0 < sw.class_count[c]; c0 += 64) tiles_tc.push_back(tile(c, r0, 128, c0, 0));
-  sw.n_tiles_tc = (int)tiles_tc.size();
-  upload(sw.tiles_tc, tiles_tc, s);
-  std::vector<int4> tiles_tc128;
-  for (int c = 0; c < (dom->curved ? 0 : nc); ++c)
-    for (int r0 = 0; r0 < sw.ld; r0 += 128)
-      for (int c0 = 0; c0 < sw.class_count[c]; c0 += 128) tiles_tc128.push_back(tile(c, r0, 128, c0, 0));
-  sw.n_tiles_tc128 = (int)tiles_tc128.size();
-  upload(sw.tiles_tc128, tiles_tc128, s);
-  std::vector<int4> tiles_tc256;
-  for (int c = 0; c < (dom->curved ? 0 : nc); ++c)
-    for (int r0 = 0; r0 < sw.ld; r0 += 128)
-      for (int c0 = 0; c0 < sw.class_count[c]; c0 += 256) tiles_tc256.push_back(tile(c, r0, 128, c0, 0));
-  sw.n_tiles_tc256 = (int)tiles_tc256.size();
-  upload(sw.tiles_tc256, tiles_tc256, s);
+  for (int q = 0; q < 2 && dom->mixed && !dom->curved; ++q) {
+    const int cap = q ? 128 : 64;
+    std::vector<int4> list;
+    int mask = 0;
+    for (int c = 0; c < nc; ++c) {
+      const int parts = (sw.class_count[c] + cap - 1) / cap;
+      const int code = tc_tile_width_code((sw.class_count[c] + parts - 1) / parts), w = tc_tile_width(code);
+      mask |= 1 << code;
+      for (int r0 = 0; r0 < sw.ld; r0 += 128)
+        for (int c0 = 0; c0 < sw.class_count[c]; c0 += w) list.push_back(tile(c, r0, 128, c0, code));
+    }
+    sw.tiles_tc[q].n = (int)list.size();
+    sw.tiles_tc[q].widths = mask;
+    upload(sw.tiles_tc[q].d, list, s);
+  }
   std::vector<int4> units;
   for (int c = 0; c < (dom->curved ? 0 : nc); ++c)
     for (int r0 = 0; r0 < sw.ld; r0 += 16) units.push_back(make_int4(c, r0, sw.class_first[c], sw.class_count[c]));
@@ -779,8 +776,8 @@ size_t domain_device_bytes(const dg_domain* dom) {
          L.trace32.bytes();
     b += sw.rec.bytes() + sw.col_of_elem.bytes() + sw.class_of_col.bytes() + sw.xform_of_elem.bytes() +
          sw.inv64.bytes() +
-         sw.inv32.bytes() + sw.inv16.bytes() + sw.inv16_scale.bytes() + sw.tiles.bytes() + sw.tiles_tc.bytes() +
-         sw.tiles_tc128.bytes() + sw.tiles_tc256.bytes() +
+         sw.inv32.bytes() + sw.inv16.bytes() + sw.inv16_scale.bytes() + sw.tiles.bytes() + sw.tiles_tc[0].d.bytes() +
+         sw.tiles_tc[1].d.bytes() +
          sw.units.bytes() + sw.bar.bytes() + sw.inv_digits.bytes() + sw.inv_row_exp.bytes() + sw.x_digits.bytes() +
          sw.x_exp.bytes() + sw.inv_hexp.bytes() + sw.tiles_f64.bytes();
     for (auto* p : {&L.w64.b, &L.w64.u, &L.w64.r, &L.w64.rS, &L.w64.duS, &L.w64.gV, &L.w64.gZ, &L.w64.gD,
