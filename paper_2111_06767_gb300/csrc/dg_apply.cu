@@ -721,7 +721,7 @@ __global__ void __launch_bounds__(EPB* N* N) coarse_smooth_kernel(const CoarseAr
       int64_t idx[7];
       int col[7];
       float w[7];
-      scatter_look_up<N, float>(a.sg, a.ap.rec, a.shares, t / N3, t % N3, idx, col, w);
+      scatter_look_up<N, 7, float>(a.sg, a.ap.rec, a.shares, t / N3, t % N3, idx, col, w);
       float acc = 0.0f;
 #pragma unroll
       for (int sl = 0; sl < 7; ++sl)

@@ -420,7 +420,7 @@ __global__ void __launch_bounds__(256) gather_kernel(SubdomainGeom g, const T* _
 
 // u += sum_S R_S^T w_S du_S with du_S = X (m = 0), or du_S = sum_{c < m} y[column][c] X_c, the X_c
 // `stride` values apart.
-template <int N, typename T, int M>
+template <int N, typename T, int M, int SL>
 __global__ void __launch_bounds__(256) scatter_kernel(SubdomainGeom g, const T* __restrict__ X,
                                                       const T* __restrict__ y, int m, int64_t stride,
                                                       const int4* __restrict__ rec, const T* __restrict__ shares,
@@ -430,39 +430,38 @@ __global__ void __launch_bounds__(256) scatter_kernel(SubdomainGeom g, const T* 
   pdl_launch_dependents();
   const bool act = t < g.E * N3;
   const int e = act ? t / N3 : 0;
-  int64_t idx[7];
-  int col[7];
-  T w[7], v[7];
-  scatter_look_up<N, T>(g, rec, shares, e, act ? t - e * N3 : 0, idx, col, w);
+  int64_t idx[SL];
+  int col[SL];
+  T w[SL], v[SL];
+  scatter_look_up<N, SL, T>(g, rec, shares, e, act ? t - e * N3 : 0, idx, col, w);
   pdl_wait();
   if (!act) return;
   const T u0 = u_zero ? T(0) : u[t];
   if constexpr (M == 0) {
 #pragma unroll
-    for (int sl = 0; sl < 7; ++sl) v[sl] = idx[sl] >= 0 ? X[idx[sl]] : T(0);
+    for (int q = 0; q < SL; ++q) v[q] = idx[q] >= 0 ? X[idx[q]] : T(0);
   } else {
 #pragma unroll
-    for (int sl = 0; sl < 7; ++sl) v[sl] = T(0);
+    for (int q = 0; q < SL; ++q) v[q] = T(0);
     const int mm = M > 0 ? M : m;  // M < 0: any m
 #pragma unroll
     for (int c = 0; c < mm; ++c)
 #pragma unroll
-      for (int sl = 0; sl < 7; ++sl)
-        if (idx[sl] >= 0) v[sl] += y[(int64_t)col[sl] * mm + c] * X[c * stride + idx[sl]];
+      for (int q = 0; q < SL; ++q)
+        if (idx[q] >= 0) v[q] += y[(int64_t)col[q] * mm + c] * X[c * stride + idx[q]];
   }
   T acc = w[0] * v[0];
 #pragma unroll
-  for (int sl = 1; sl < 7; ++sl) acc += w[sl] * v[sl];
+  for (int q = 1; q < SL; ++q) acc += w[q] * v[q];
   u[t] = u0 + acc;
 }
 
-template <int N, typename T>
+template <int N, typename T, int SL>
 void launch_scatter_n(const SubdomainGeom& g, const T* X, const T* y, int m, int64_t stride, const int4* rec,
                       const T* shares, T* u, int u_zero, cudaStream_t s) {
   const dim3 grid((g.E * N * N * N + 255) / 256);
-  if (m == 0) launch_pdl(scatter_kernel<N, T, 0>, grid, dim3(256), 0, s, g, X, y, m, stride, rec, shares, u, u_zero);
-  else if (m == 3) launch_pdl(scatter_kernel<N, T, 3>, grid, dim3(256), 0, s, g, X, y, m, stride, rec, shares, u, u_zero);
-  else launch_pdl(scatter_kernel<N, T, -1>, grid, dim3(256), 0, s, g, X, y, m, stride, rec, shares, u, u_zero);
+  auto k = m == 0 ? scatter_kernel<N, T, 0, SL> : (m == 3 ? scatter_kernel<N, T, 3, SL> : scatter_kernel<N, T, -1, SL>);
+  launch_pdl(k, grid, dim3(256), 0, s, g, X, y, m, stride, rec, shares, u, u_zero);
 }
 
 template <typename T>
@@ -485,7 +484,10 @@ void launch_scatter(const SubdomainGeom& g, const T* X, const T* y, int m, int64
   if (g.E == 0) return;
   switch (g.N) {
 #define DG_CASE(NN) \
-  case NN: launch_scatter_n<NN, T>(g, X, y, m, stride, rec, shares, u, u_zero ? 1 : 0, s); break;
+  case NN: \
+    if (2 * g.ov <= NN) launch_scatter_n<NN, T, 4>(g, X, y, m, stride, rec, shares, u, u_zero ? 1 : 0, s); \
+    else launch_scatter_n<NN, T, 7>(g, X, y, m, stride, rec, shares, u, u_zero ? 1 : 0, s); \
+    break;
     DG_CASE(2) DG_CASE(3) DG_CASE(4) DG_CASE(5) DG_CASE(6) DG_CASE(7) DG_CASE(8) DG_CASE(9) DG_CASE(10)
 #undef DG_CASE
     default: fail(DG_ERR_INVALID_ARG, "unsupported N");
@@ -689,11 +691,11 @@ void launch_class_gemm_tiles(const T* inv, const T* X, T* Y, int ld, const int4*
 // diagonal linearization term) is solved by GMRES from du_S = 0 for a fixed number of iterations,
 // right-preconditioned by the explicit inverse of the Poisson subdomain matrix A_S (the
 // Laplacian approximation). With z = A_S^-1 v, (A_S + D_S) z = v + D_S z, so every iteration is
-// one class GEMM plus per-subdomain vector work. One warp per subdomain column (8 per CTA): the
+// one class GEMM plus per-subdomain vector work. One warp per subdomain column: the
 // reductions are warp shuffles in a fixed order, with no CTA barrier, and every subdomain of a
 // level is resident at once.
 
-constexpr int kSubWarps = 8;  // subdomain columns (warps) per CTA
+constexpr int kSubWarps = 4;  // subdomain columns (warps) per CTA: 8 leave a longer tail (punctures 13.93 against 13.75 ms)
 
 // Sum over the warp's lanes in a fixed order, returned to every lane.
 template <typename T>
@@ -805,24 +807,30 @@ __global__ void __launch_bounds__(32 * kSubWarps) sub_arnoldi_kernel(const SubKr
   const T* vj = j == 0 ? r : a.V + (size_t)(j - 1) * a.stride + off;
   T* wout = a.V + (size_t)j * a.stride + off;
   T* h = a.H + (size_t)col * (m + 1) * m;
-  T w[GG][EV], b2 = 0;
-  if constexpr (G > 0) {
+  T w[GG][EV], x[GG][EV], v[GG][EV], b2 = 0;
+  // a block of the column's vector, scaled (zeros past its end)
+  auto load = [&](const T* p, T (&d)[GG][EV]) {
 #pragma unroll
-    for (int g = 0; g < G; ++g) {
+    for (int g = 0; g < GG; ++g) {
       const int i = (g * 32 + lane) * EV;
+      if (i < ld) SV::ld(p + i, d[g]);
+      else
 #pragma unroll
-      for (int e = 0; e < EV; ++e) w[g][e] = 0;
-      if (i >= ld) continue;
-      T x[EV], d[EV], z[EV];
-      SV::ld(vj + i, x);
-      SV::ld(D + i, d);
-      SV::ld(zj + i, z);
+        for (int e = 0; e < EV; ++e) d[g][e] = 0;
+    }
+  };
+  if constexpr (G > 0) {
+    load(vj, x);
+    load(zj, w);
+    load(D, v);
+#pragma unroll
+    for (int g = 0; g < G; ++g)
 #pragma unroll
       for (int e = 0; e < EV; ++e) {
-        w[g][e] = x[e] + d[e] * z[e];
-        b2 += x[e] * x[e];
+        w[g][e] = x[g][e] + v[g][e] * w[g][e];
+        b2 += x[g][e] * x[g][e];
       }
-    }
+    if (j > 0) load(r, v);  // V_0, in flight during the first reductions
   } else {
     for (int i = lane; i < ld; i += 32) {
       wout[i] = vj[i] + D[i] * zj[i];
@@ -858,20 +866,20 @@ __global__ void __launch_bounds__(32 * kSubWarps) sub_arnoldi_kernel(const SubKr
     const T* vi = ii == 0 ? r : a.V + (size_t)(ii - 1) * a.stride + off;
     const T sc = ii == 0 ? inv_beta : T(1);
     T acc = 0;
-    T v[GG][EV];
     if constexpr (G > 0) {
+      if (ii == j) {  // V_j is here already
 #pragma unroll
-      for (int g = 0; g < G; ++g) {
-        const int i = (g * 32 + lane) * EV;
+        for (int g = 0; g < G; ++g)
 #pragma unroll
-        for (int e = 0; e < EV; ++e) v[g][e] = 0;
-        if (i < ld) SV::ld(vi + i, v[g]);
+          for (int e = 0; e < EV; ++e) v[g][e] = x[g][e];
+      }
+#pragma unroll
+      for (int g = 0; g < G; ++g)
 #pragma unroll
         for (int e = 0; e < EV; ++e) {
           v[g][e] *= sc;
           acc += w[g][e] * v[g][e];
         }
-      }
     } else {
       for (int t = lane; t < ld; t += 32) acc += wout[t] * (sc * vi[t]);
     }
@@ -881,6 +889,7 @@ __global__ void __launch_bounds__(32 * kSubWarps) sub_arnoldi_kernel(const SubKr
       for (int g = 0; g < G; ++g)
 #pragma unroll
         for (int e = 0; e < EV; ++e) w[g][e] -= hij * v[g][e];
+      if (ii + 1 < j) load(a.V + (size_t)ii * a.stride + off, v);
     } else {
       for (int t = lane; t < ld; t += 32) wout[t] -= hij * (sc * vi[t]);
     }

@@ -75,27 +75,39 @@ __device__ __forceinline__ void gather_point(const SubdomainGeom& g, const int4*
 }
 
 // The static part of a point's scatter: its place in the subdomain vectors (-1: not in that slot) and
-// the weight of each ([64 patterns][7][N^3] shares).
-template <int N, typename T>
+// the weight of each ([64 patterns][7][N^3] shares). SL = 7: every slot. SL = 4 where 2 ov <= N, so that a
+// point lies in the overlap of at most one side per dimension: its own subdomain and one candidate along
+// x, y and z (the same terms in the same order, with fewer registers and predicates).
+template <int N, int SL, typename T>
 __device__ __forceinline__ void scatter_look_up(const SubdomainGeom& g, const int4* __restrict__ rec,
-                                                const T* __restrict__ shares, int e, int p, int64_t (&idx)[7],
-                                                int (&col)[7], T (&w)[7]) {
+                                                const T* __restrict__ shares, int e, int p, int64_t (&idx)[SL],
+                                                int (&col)[SL], T (&w)[SL]) {
   constexpr int N3 = N * N * N;
-  const int i = p % N, j = (p / N) % N, k = p / (N * N);
+  const int c[3] = {p % N, (p / N) % N, p / (N * N)};
   const int4 r0 = __ldg(rec + e * 7);
   const T* sh = shares + (size_t)(r0.w >> 16) * 7 * N3 + p;
 #pragma unroll
-  for (int sl = 0; sl < 7; ++sl) {
-    idx[sl] = -1;
-    col[sl] = 0;
-    w[sl] = T(0);
-    if (!slot_covers<N>(sl, i, j, k, g.ov)) continue;
-    const int4 r = sl == 0 ? r0 : __ldg(rec + e * 7 + sl);
-    const int row = record_row(r, i, j, k);
+  for (int q = 0; q < SL; ++q) {
+    idx[q] = -1;
+    col[q] = 0;
+    w[q] = T(0);
+    int sl = q;
+    if constexpr (SL == 4) {
+      if (q > 0) {
+        const int cd = c[q - 1];
+        if (cd < g.ov) sl = 2 * q - 1;
+        else if (N - 1 - cd < g.ov) sl = 2 * q;
+        else continue;
+      }
+    } else {
+      if (!slot_covers<N>(sl, c[0], c[1], c[2], g.ov)) continue;
+    }
+    const int4 r = q == 0 ? r0 : __ldg(rec + e * 7 + sl);
+    const int row = record_row(r, c[0], c[1], c[2]);
     if (r.x < 0 || !DG_IN_BOUNDS(r.x, g.E) || !DG_IN_BOUNDS(row, g.ld)) continue;
-    idx[sl] = (int64_t)r.x * g.ld + row;
-    col[sl] = r.x;
-    w[sl] = sh[sl * N3];
+    idx[q] = (int64_t)r.x * g.ld + row;
+    col[q] = r.x;
+    w[q] = sh[sl * N3];
   }
 }
 
