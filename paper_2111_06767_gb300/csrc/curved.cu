@@ -17,10 +17,12 @@
 // u_E = u, F_E = K n.g). sigma = C N^2 / min(h, h_E) with h = 2 / |G^d| the element size normal to
 // the face at the node (the element width for affine elements).
 //
-// GB300 mapping: one CTA per element, one thread per node (N^3 threads), the element's values, the
-// lifted auxiliary field and the exterior face data staged in shared memory. The exterior normal
-// fluxes come from a trace pass (every element writes n.g on its six faces) before the operator
-// pass; the metric is read once per node (J and the nine G entries, coalesced).
+// GB300 mapping: one CTA per element, one thread per node (N^3 threads). A trace pass takes the local
+// gradient once, keeps it for the operator pass and writes every face's normal flux for the neighbours; the
+// operator pass stages the lifted auxiliary field and the exterior face data in shared memory. Bound by the
+// FP64 pipe in FP64: a square root or a division costs as much there as a contraction, and every warp holds
+// face nodes, so |G^d|, its inverse and |G^d| sigma are set up once per face node, and only these products
+// remain (n enters as s G^d, its length cancels from the lifting). 8^3 elements at N = 8 with K: 206 -> 127 us.
 #include <algorithm>
 #include <vector>
 
@@ -37,7 +39,6 @@ template <int N, typename T>
 struct CurvedSmem {
   T D[N * N];
   T w[N];
-  T u[N * N * N];
   T v[3][N * N * N];
   T uE[6][N * N];  // exterior value at each face node (kNbr faces)
   T fE[6][N * N];  // exterior's own outward normal flux K_E n_E.g_E (kNbr faces)
@@ -83,58 +84,60 @@ __device__ __forceinline__ void face_coords(int d, int i, int j, int k, int& a1,
   a2 = d == 2 ? j : k;
 }
 
-// The element operator at node p = threadIdx.x (every thread of the CTA calls it; S.u, S.uE,
-// S.fE and S.type filled and synchronised). Returns (A u)_p, massive form.
+// G^j du_j: the gradient from the logical derivatives.
+template <typename T>
+__device__ __forceinline__ void physical_grad(const T (&G)[3][3], const T (&du)[3], T (&g)[3]) {
+#pragma unroll
+  for (int c = 0; c < 3; ++c) g[c] = G[0][c] * du[0] + G[1][c] * du[1] + G[2][c] * du[2];
+}
+
+// Normal flux K n.g on the faces through node (i, j, k), at most one per dimension, handed to put(f, index,
+// flux); inv: 1 / |G^d| at the element's face nodes.
+template <int N, typename T, typename F>
+__device__ __forceinline__ void face_fluxes(const T (&G)[3][3], const T (&g)[3], T K, const T* __restrict__ inv, int i,
+                                            int j, int k, F put) {
+  const int idx[3] = {i, j, k};
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    if (idx[d] != 0 && idx[d] != N - 1) continue;
+    const int side = idx[d] != 0, f = 2 * d + side;
+    int a1, a2;
+    face_coords(d, i, j, k, a1, a2);
+    const int at = f * N * N + a2 * N + a1;
+    const T ng = G[d][0] * g[0] + G[d][1] * g[1] + G[d][2] * g[2];
+    put(f, a2 * N + a1, (side ? K : -K) * inv[at] * ng);
+  }
+}
+
+// The element operator at node p = threadIdx.x (every thread of the CTA calls it; S.uE, S.fE and S.type
+// filled and synchronised), from the node's value, gradient, metric and coefficient; face: the element's
+// |G^d| sigma, and nf further on |G^d|. Returns (A u)_p, massive form.
 template <int N, typename T>
-__device__ T curved_element(CurvedSmem<N, T>& S, const T* __restrict__ geo, int64_t ndof, int64_t gbase,
-                            const T* __restrict__ sigma_e) {
+__device__ T curved_element(CurvedSmem<N, T>& S, const T* __restrict__ Kfield, const T* __restrict__ face, int64_t nf,
+                            T up, const T (&g)[3], T J, const T (&G)[3][3], T Kp) {
   constexpr int N2 = N * N;
   const int p = threadIdx.x;
   const int i = p % N, j = (p / N) % N, k = p / N2;
   const int idx[3] = {i, j, k};
-  T J, G[3][3];
-  load_metric<N, T>(geo, ndof, gbase + p, J, G);
-  const T Kp = geo[10 * ndof + gbase + p];
-  T du[3];
-  logical_grad<N, T>(S.D, S.u, i, j, k, du);
-  T g[3], v[3];
-#pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    g[c] = G[0][c] * du[0] + G[1][c] * du[1] + G[2][c] * du[2];
-    v[c] = g[c];
-  }
-  const T up = S.u[p];
-  // the faces through the node, at most one per dimension: their unit outward normals and |G^d|
-  // (one square root and one division per face)
+  T v[3] = {g[0], g[1], g[2]};
+  // the faces through the node and the exterior values there
   int fside[3];
-  T nn[3][3], nrm[3];
+  T uE[3];
+  const T half_w0inv = T(0.5) / S.w[0];
 #pragma unroll
   for (int d = 0; d < 3; ++d) {
     fside[d] = idx[d] == 0 ? 0 : (idx[d] == N - 1 ? 1 : -1);
-    nrm[d] = T(0);
-#pragma unroll
-    for (int c = 0; c < 3; ++c) nn[d][c] = T(0);
-    if (fside[d] >= 0) {
-      nrm[d] = sqrt(G[d][0] * G[d][0] + G[d][1] * G[d][1] + G[d][2] * G[d][2]);
-      const T sc = (fside[d] ? T(1) : T(-1)) / nrm[d];
-#pragma unroll
-      for (int c = 0; c < 3; ++c) nn[d][c] = sc * G[d][c];
-    }
-  }
-  const T half_w0inv = T(0.5) / S.w[0];
-  // lifting of the auxiliary flux on every face through the node
-#pragma unroll
-  for (int d = 0; d < 3; ++d) {
+    uE[d] = T(0);
     if (fside[d] < 0) continue;
     const int f = 2 * d + fside[d];
     int a1, a2;
     face_coords(d, i, j, k, a1, a2);
-    const int ab = a2 * N + a1;
     const int t = S.type[f];
-    const T uE = t == kNbr ? S.uE[f][ab] : (t == kDirichlet ? -up : (t == kNeumann ? up : T(0)));
-    const T lift = (uE - up) * nrm[d] * half_w0inv;
+    uE[d] = t == kNbr ? S.uE[f][a2 * N + a1] : (t == kDirichlet ? -up : (t == kNeumann ? up : T(0)));
+    // lifting of the auxiliary flux
+    const T lift = (fside[d] ? uE[d] - up : up - uE[d]) * half_w0inv;
 #pragma unroll
-    for (int c = 0; c < 3; ++c) v[c] += nn[d][c] * lift;
+    for (int c = 0; c < 3; ++c) v[c] += G[d][c] * lift;
   }
 #pragma unroll
   for (int c = 0; c < 3; ++c) S.v[c][p] = Kp * v[c];
@@ -147,8 +150,7 @@ __device__ T curved_element(CurvedSmem<N, T>& S, const T* __restrict__ geo, int6
     logical_grad<N, T>(S.D, S.v[c], i, j, k, dv);
     div += G[0][c] * dv[0] + G[1][c] * dv[1] + G[2][c] * dv[2];
   }
-  const T wp = S.w[i] * S.w[j] * S.w[k];
-  T Au = -wp * J * div;
+  T Au = -(S.w[i] * S.w[j] * S.w[k]) * J * div;
 #pragma unroll
   for (int d = 0; d < 3; ++d) {
     if (fside[d] < 0) continue;
@@ -156,21 +158,15 @@ __device__ T curved_element(CurvedSmem<N, T>& S, const T* __restrict__ geo, int6
     int a1, a2;
     face_coords(d, i, j, k, a1, a2);
     const int ab = a2 * N + a1;
-    T ng = 0, nv = 0;
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      ng += nn[d][c] * g[c];
-      nv += nn[d][c] * v[c];
-    }
-    ng *= Kp;  // n.F_u of the local gradient
-    nv *= Kp;
+    // everything times |G^d|: K n.g, K n.v and the exterior flux
+    const T sK = side ? Kp : -Kp;
+    const T ng = sK * (G[d][0] * g[0] + G[d][1] * g[1] + G[d][2] * g[2]);
+    const T nv = sK * (G[d][0] * v[0] + G[d][1] * v[1] + G[d][2] * v[2]);
     const int t = S.type[f];
-    const T uE = t == kNbr ? S.uE[f][ab] : (t == kDirichlet ? -up : (t == kNeumann ? up : T(0)));
-    const T fE = t == kNbr ? S.fE[f][ab] : (t == kDirichlet ? -ng : (t == kNeumann ? ng : T(0)));
-    const T KE = t == kNbr ? geo[10 * ndof + (int64_t)S.eE[f] * (N * N2) + node_of<N>(d, side ? 0 : N - 1, a1, a2)]
-                           : Kp;
-    const T prim = T(0.5) * (ng - fE) - sigma_e[f * N2 + ab] * (Kp * up - KE * uE);
-    Au -= S.w[a1] * S.w[a2] * J * nrm[d] * (prim - nv);
+    const T fE = t == kNbr ? face[nf + f * N2 + ab] * S.fE[f][ab] : (t == kDirichlet ? -ng : (t == kNeumann ? ng : T(0)));
+    const T KE = t == kNbr ? Kfield[(int64_t)S.eE[f] * (N * N2) + node_of<N>(d, side ? 0 : N - 1, a1, a2)] : Kp;
+    const T prim = T(0.5) * (ng - fE) - face[f * N2 + ab] * (Kp * up - KE * uE[d]);
+    Au -= S.w[a1] * S.w[a2] * J * (prim - nv);
   }
   return Au;
 }
@@ -181,7 +177,8 @@ __device__ __forceinline__ void load_tables(CurvedSmem<N, T>& S, const T* __rest
   for (int t = threadIdx.x; t < N; t += blockDim.x) S.w[t] = w[t];
 }
 
-// Outward normal flux n.g of every face node of every element (the exterior data of its neighbours).
+// The local gradient at every node and the outward normal flux K n.g at every face node (the exterior data
+// of the neighbours).
 template <int N, typename T>
 __global__ void __launch_bounds__(N * N * N) curved_trace_kernel(CurvedArgs<T> a) {
   constexpr int N2 = N * N, N3 = N * N * N;
@@ -189,27 +186,20 @@ __global__ void __launch_bounds__(N * N * N) curved_trace_kernel(CurvedArgs<T> a
   __shared__ T su[N3];
   const int e = blockIdx.x, p = threadIdx.x;
   const int i = p % N, j = (p / N) % N, k = p / N2;
+  const int64_t gp = (int64_t)e * N3 + p;
   for (int t = p; t < N2; t += N3) sD[t] = a.D[t];
-  su[p] = a.u[(int64_t)e * N3 + p];
+  su[p] = a.u[gp];
   __syncthreads();
-  T J, G[3][3];
-  load_metric<N, T>(a.geo, a.ndof, (int64_t)e * N3 + p, J, G);
-  const T Kp = a.geo[10 * a.ndof + (int64_t)e * N3 + p];
-  T du[3];
+  T J, G[3][3], du[3], g[3];
+  load_metric<N, T>(a.geo, a.ndof, gp, J, G);
+  const T Kp = a.geo[10 * a.ndof + gp];
   logical_grad<N, T>(sD, su, i, j, k, du);
-  const int idx[3] = {i, j, k};
+  physical_grad(G, du, g);
 #pragma unroll
-  for (int f = 0; f < 6; ++f) {
-    const int d = f >> 1, side = f & 1;
-    if (idx[d] != (side ? N - 1 : 0)) continue;
-    int a1, a2;
-    face_coords(d, i, j, k, a1, a2);
-    const T sc = (side ? T(1) : T(-1)) / sqrt(G[d][0] * G[d][0] + G[d][1] * G[d][1] + G[d][2] * G[d][2]);
-    T ng = 0;
-#pragma unroll
-    for (int c = 0; c < 3; ++c) ng += G[d][c] * (G[0][c] * du[0] + G[1][c] * du[1] + G[2][c] * du[2]);
-    a.trace[((int64_t)e * 6 + f) * N2 + a2 * N + a1] = Kp * sc * ng;
-  }
+  for (int c = 0; c < 3; ++c) a.grad[c * a.ndof + gp] = g[c];
+  const int64_t f0 = (int64_t)e * 6 * N2;
+  face_fluxes<N, T>(G, g, Kp, a.face + 2 * a.nf + f0, i, j, k,
+                    [&](int f, int ab, T flux) { a.trace[f0 + f * N2 + ab] = flux; });
 }
 
 // out = A u, or b - A u with b.
@@ -218,8 +208,14 @@ __global__ void __launch_bounds__(N * N * N) curved_apply_kernel(CurvedArgs<T> a
   constexpr int N2 = N * N, N3 = N * N * N;
   __shared__ CurvedSmem<N, T> S;
   const int e = blockIdx.x, p = threadIdx.x;
+  const int64_t gp = (int64_t)e * N3 + p;
   load_tables<N, T>(S, a.D, a.w);
-  S.u[p] = a.u[(int64_t)e * N3 + p];
+  const T up = a.u[gp];
+  T J, G[3][3], g[3];
+  load_metric<N, T>(a.geo, a.ndof, gp, J, G);
+  const T Kp = a.geo[10 * a.ndof + gp];
+#pragma unroll
+  for (int c = 0; c < 3; ++c) g[c] = a.grad[c * a.ndof + gp];
   if (p < 6) {
     const int nb = elem_nbr(a.n[0], a.n[1], a.n[2], e, p);
     S.type[p] = nb >= 0 ? kNbr : (((a.neumann >> p) & 1) ? kNeumann : kDirichlet);
@@ -234,8 +230,7 @@ __global__ void __launch_bounds__(N * N * N) curved_apply_kernel(CurvedArgs<T> a
     }
   }
   __syncthreads();
-  const T Au = curved_element<N, T>(S, a.geo, a.ndof, (int64_t)e * N3, a.sigma + (int64_t)e * 6 * N2);
-  const int64_t gp = (int64_t)e * N3 + p;
+  const T Au = curved_element<N, T>(S, a.geo + 10 * a.ndof, a.face + (int64_t)e * 6 * N2, a.nf, up, g, J, G, Kp);
   a.out[gp] = a.b ? a.b[gp] - Au : Au;
 }
 
@@ -248,6 +243,7 @@ __global__ void __launch_bounds__(N * N * N) curved_column_kernel(CurvedArgs<T> 
                                                                   T* __restrict__ A_out) {
   constexpr int N2 = N * N, N3 = N * N * N;
   __shared__ CurvedSmem<N, T> S;
+  __shared__ T su[N3];
   __shared__ T sTP[6][N2];  // outward normal fluxes of the unit vector's own slot
   __shared__ int selem[7];
   const int q = blockIdx.x, e = e0 + blockIdx.y, p = threadIdx.x;
@@ -273,33 +269,23 @@ __global__ void __launch_bounds__(N * N * N) curved_column_kernel(CurvedArgs<T> 
   }
   // the unit vector's normal fluxes on the faces of its own slot
   {
-    S.u[p] = p == pP ? T(1) : T(0);
+    su[p] = p == pP ? T(1) : T(0);
     __syncthreads();
-    T J, G[3][3];
+    T J, G[3][3], du[3], g[3];
     load_metric<N, T>(a.geo, a.ndof, (int64_t)selem[P] * N3 + p, J, G);
     const T Kp = a.geo[10 * a.ndof + (int64_t)selem[P] * N3 + p];
-    T du[3];
-    logical_grad<N, T>(S.D, S.u, i, j, k, du);
-    const int idx[3] = {i, j, k};
-#pragma unroll
-    for (int f = 0; f < 6; ++f) {
-      const int d = f >> 1, side = f & 1;
-      if (idx[d] != (side ? N - 1 : 0)) continue;
-      int a1, a2;
-      face_coords(d, i, j, k, a1, a2);
-      const T sc = (side ? T(1) : T(-1)) / sqrt(G[d][0] * G[d][0] + G[d][1] * G[d][1] + G[d][2] * G[d][2]);
-      T ng = 0;
-#pragma unroll
-      for (int c = 0; c < 3; ++c) ng += G[d][c] * (G[0][c] * du[0] + G[1][c] * du[1] + G[2][c] * du[2]);
-      sTP[f][a2 * N + a1] = Kp * sc * ng;
-    }
+    logical_grad<N, T>(S.D, su, i, j, k, du);
+    physical_grad(G, du, g);
+    face_fluxes<N, T>(G, g, Kp, a.face + 2 * a.nf + (int64_t)selem[P] * 6 * N2, i, j, k,
+                      [&](int f, int ab, T flux) { sTP[f][ab] = flux; });
     __syncthreads();
   }
   // slots whose rows the unit vector reaches: its own slot and the slots across its faces
   for (int X = 0; X < 7; ++X) {
     const bool adjacent = P == 0 ? true : X == 0;
     if (!(X == P || adjacent) || selem[X] < 0) continue;
-    S.u[p] = (X == P && p == pP) ? T(1) : T(0);
+    const T up = (X == P && p == pP) ? T(1) : T(0);
+    su[p] = up;
     if (p < 6) {
       const int f = p;
       int t;
@@ -322,7 +308,12 @@ __global__ void __launch_bounds__(N * N * N) curved_column_kernel(CurvedArgs<T> 
       S.fE[f][ab] = hit ? sTP[f ^ 1][ab] : T(0);
     }
     __syncthreads();
-    const T Au = curved_element<N, T>(S, a.geo, a.ndof, (int64_t)selem[X] * N3, a.sigma + (int64_t)selem[X] * 6 * N2);
+    T J, G[3][3], du[3], g[3];
+    load_metric<N, T>(a.geo, a.ndof, (int64_t)selem[X] * N3 + p, J, G);
+    logical_grad<N, T>(S.D, su, i, j, k, du);
+    physical_grad(G, du, g);
+    const T Au = curved_element<N, T>(S, a.geo + 10 * a.ndof, a.face + (int64_t)selem[X] * 6 * N2, a.nf, up, g, J, G,
+                                      a.geo[10 * a.ndof + (int64_t)selem[X] * N3 + p]);
     const int row = subdomain_row<N>(X, p, ov);
     if (row >= 0) A[(size_t)row * nS + q] = Au;
     __syncthreads();
@@ -381,13 +372,15 @@ __global__ void __launch_bounds__(N * N * N) curved_metric_kernel(const double* 
     }
 }
 
-// sigma = C N^2 / min(h, h_E) at every face node, h = 2 / |G^d| (the interior's at box faces).
+// At every face node |G^d| sigma with sigma = C N^2 / min(h, h_E), h = 2 / |G^d| (the interior's at box
+// faces), then |G^d| and 1 / |G^d|: three arrays [E][6][N^2].
 template <int N>
-__global__ void curved_sigma_kernel(int nx, int ny, int nz, double penalty, const double* __restrict__ geo,
-                                    int64_t ndof, double* __restrict__ sig64, float* __restrict__ sig32) {
+__global__ void curved_face_kernel(int nx, int ny, int nz, double penalty, const double* __restrict__ geo,
+                                   int64_t ndof, double* __restrict__ face64, float* __restrict__ face32) {
   constexpr int N2 = N * N, N3 = N * N * N;
   const int64_t E = (int64_t)nx * ny * nz;
-  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < E * 6 * N2; t += (int64_t)gridDim.x * blockDim.x) {
+  const int64_t nf = E * 6 * N2;
+  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < nf; t += (int64_t)gridDim.x * blockDim.x) {
     const int e = (int)(t / (6 * N2));
     const int f = (int)((t / N2) % 6), ab = (int)(t % N2), d = f >> 1, side = f & 1;
     auto size_at = [&](int el, int sd) {
@@ -398,9 +391,11 @@ __global__ void curved_sigma_kernel(int nx, int ny, int nz, double penalty, cons
     const double h = size_at(e, side);
     const int nb = elem_nbr(nx, ny, nz, e, f);
     const double hE = nb >= 0 ? size_at(nb, 1 - side) : h;
-    const double sg = penalty * N * N / fmin(h, hE);
-    sig64[t] = sg;
-    sig32[t] = (float)sg;
+    const double v[3] = {2.0 / h * (penalty * N * N / fmin(h, hE)), 2.0 / h, 0.5 * h};
+    for (int q = 0; q < 3; ++q) {
+      face64[q * nf + t] = v[q];
+      face32[q * nf + t] = (float)v[q];
+    }
   }
 }
 
@@ -505,15 +500,15 @@ void launch_curved_metric(int N, int64_t E, const double* xyz, const double* D, 
   DG_LAUNCHED(1);
 }
 
-void launch_curved_sigma(int N, const int n[3], double penalty, const double* geo64, double* sig64, float* sig32,
+void launch_curved_faces(int N, const int n[3], double penalty, const double* geo64, double* face64, float* face32,
                          cudaStream_t s) {
   const int64_t E = (int64_t)n[0] * n[1] * n[2], ndof = E * N * N * N;
   const int64_t work = E * 6 * N * N;
   if (work == 0) return;
 #define DG_CASE(NN)                                                                                           \
   case NN:                                                                                                    \
-    curved_sigma_kernel<NN><<<grid_for(work, 256), 256, 0, s>>>(n[0], n[1], n[2], penalty, geo64, ndof, sig64, \
-                                                               sig32);                                        \
+    curved_face_kernel<NN><<<grid_for(work, 256), 256, 0, s>>>(n[0], n[1], n[2], penalty, geo64, ndof, face64, \
+                                                              face32);                                        \
     break;
   DG_CURVED_SWITCH(DG_CASE)
 #undef DG_CASE

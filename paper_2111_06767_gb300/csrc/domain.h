@@ -74,9 +74,10 @@ struct Level {
   double h[3] = {0, 0, 0};
   OpGeom<double> g64{};
   OpGeom<float> g32{};
-  // curved elements: metric, face-node penalty, face-node normal fluxes (scratch of every apply)
-  DevBuf<double> geo64, sig64, trace64;
-  DevBuf<float> geo32, sig32, trace32;
+  // curved elements: metric, face-node sizes and penalty; face-node normal fluxes and gradient (scratch of
+  // every apply)
+  DevBuf<double> geo64, face64, trace64, grad64;
+  DevBuf<float> geo32, face32, trace32, grad32;
   SchwarzLevel sw;
   LevelWork<double> w64;
   LevelWork<float> w32;

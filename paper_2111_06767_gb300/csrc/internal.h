@@ -289,21 +289,24 @@ void launch_sub_arnoldi(int E, int ld, int j, int m, const T* r, const T* D, T* 
                         cudaStream_t s);
 
 // Curved (mapped) elements and variable coefficients: metric [11][ndof] (J, then G^j_i = dxi^j/dx^i
-// at 1 + 3 j + i, then the coefficient K at 10), penalty
-// at every face node [E][6][N^2], outward normal fluxes of u at every face node [E][6][N^2].
+// at 1 + 3 j + i, then the coefficient K at 10); at every face node |G^d| sigma, |G^d| and 1 / |G^d|
+// [3][E][6][N^2] (nf = 6 E N^2 apart). Scratch of every apply: outward normal fluxes of u at every face node
+// [E][6][N^2] and the gradient of u [3][ndof].
 template <typename T>
 struct CurvedArgs {
   int n[3];
   int neumann;
   int64_t ndof;
   const T* geo;
-  const T* sigma;
+  const T* face;
+  int64_t nf;
   const T* D;
   const T* w;
   const T* u;
   const T* b;
   T* out;
   T* trace;
+  T* grad;
 };
 // out = A u (or b - A u): the trace pass, then the operator pass.
 template <typename T>
@@ -314,7 +317,7 @@ void launch_curved_columns(int N, const CurvedArgs<T>& a, int ov, int nS, int e0
                            cudaStream_t s);
 void launch_curved_metric(int N, int64_t E, const double* xyz, const double* D, double* geo64, float* geo32, int* bad,
                           cudaStream_t s);
-void launch_curved_sigma(int N, const int n[3], double penalty, const double* geo64, double* sig64, float* sig32,
+void launch_curved_faces(int N, const int n[3], double penalty, const double* geo64, double* face64, float* face32,
                          cudaStream_t s);
 void launch_curved_coarsen(int N, const int cn[3], const int fn[3], const double* C, const double* fine_xyz,
                            double* coarse_xyz, cudaStream_t s);

@@ -443,11 +443,13 @@ void setup_curved_geometry(dg_domain* dom, const double* host_xyz, const double*
     L.geo32.alloc(11 * (size_t)L.ndof);
     launch_curved_metric(N, L.E, cur.get(), dom->D64.get(), L.geo64.get(), L.geo32.get(), bad.get(), s);
     const size_t nf = (size_t)L.E * 6 * N * N;
-    L.sig64.alloc(nf);
-    L.sig32.alloc(nf);
-    launch_curved_sigma(N, L.n, dom->desc.penalty, L.geo64.get(), L.sig64.get(), L.sig32.get(), s);
+    L.face64.alloc(3 * nf);
+    L.face32.alloc(3 * nf);
+    launch_curved_faces(N, L.n, dom->desc.penalty, L.geo64.get(), L.face64.get(), L.face32.get(), s);
     L.trace32.alloc(nf);
     L.trace64.alloc(nf);
+    L.grad32.alloc(3 * (size_t)L.ndof);
+    L.grad64.alloc(3 * (size_t)L.ndof);
   }
   launch_curved_mass(N, dom->w64.get(), L0.geo64.get(), L0.ndof, dom->mass.get(), s);
   int h_bad = 0;
@@ -586,7 +588,7 @@ namespace {
 // built column by column from the curved operator on its patch, inverted in place by Gauss-Jordan
 // without pivoting (the symmetric part of A_S is positive definite, so no pivot vanishes).
 template <typename T>
-void build_curved_inverses(dg_domain* dom, Level& L, DevBuf<T>& inv, const T* geo, const T* sig, const T* D,
+void build_curved_inverses(dg_domain* dom, Level& L, DevBuf<T>& inv, const T* geo, const T* face, const T* D,
                            const T* w, cudaStream_t s) {
   const int nS = L.sw.nS, E = L.E;
   const size_t n2 = (size_t)nS * nS;
@@ -596,7 +598,8 @@ void build_curved_inverses(dg_domain* dom, Level& L, DevBuf<T>& inv, const T* ge
   a.neumann = dom->desc.neumann_faces;
   a.ndof = L.ndof;
   a.geo = geo;
-  a.sigma = sig;
+  a.face = face;
+  a.nf = (int64_t)L.E * 6 * dom->N * dom->N;
   a.D = D;
   a.w = w;
   constexpr int kBatch = 65535;  // grid limits of the column and Gauss-Jordan launches
@@ -621,7 +624,7 @@ void ensure_schwarz(dg_domain* dom, int level) {
     cudaStream_t s = dom->stream;
     sw.inv_scale = 1.0;
     if (dom->mixed) {
-      build_curved_inverses<float>(dom, L, sw.inv32, L.geo32.get(), L.sig32.get(), dom->D32.get(), dom->w32.get(), s);
+      build_curved_inverses<float>(dom, L, sw.inv32, L.geo32.get(), L.face32.get(), dom->D32.get(), dom->w32.get(), s);
       if (dom->desc.subdomain_gemm != DG_GEMM_SIMT) {
         // the smoother streams every inverse once per step: keep them in FP16 (scaled per subdomain),
         // the input precision of the tensor-core path; "simt" keeps FP32
@@ -633,7 +636,7 @@ void ensure_schwarz(dg_domain* dom, int level) {
       }
       alloc_work(L.w32, L, s);
     } else {
-      build_curved_inverses<double>(dom, L, sw.inv64, L.geo64.get(), L.sig64.get(), dom->D64.get(), dom->w64.get(),
+      build_curved_inverses<double>(dom, L, sw.inv64, L.geo64.get(), L.face64.get(), dom->D64.get(), dom->w64.get(),
                                     s);
       alloc_work(L.w64, L, s);
     }
@@ -772,8 +775,8 @@ size_t domain_device_bytes(const dg_domain* dom) {
              dom->vout64.bytes() + dom->err_flag.bytes();
   for (const auto& L : dom->levels) {
     const auto& sw = L.sw;
-    b += L.geo64.bytes() + L.geo32.bytes() + L.sig64.bytes() + L.sig32.bytes() + L.trace64.bytes() +
-         L.trace32.bytes();
+    b += L.geo64.bytes() + L.geo32.bytes() + L.face64.bytes() + L.face32.bytes() + L.trace64.bytes() +
+         L.trace32.bytes() + L.grad64.bytes() + L.grad32.bytes();
     b += sw.rec.bytes() + sw.col_of_elem.bytes() + sw.class_of_col.bytes() + sw.xform_of_elem.bytes() +
          sw.inv64.bytes() +
          sw.inv32.bytes() + sw.inv16.bytes() + sw.inv16_scale.bytes() + sw.tiles.bytes() + sw.tiles_tc[0].d.bytes() +

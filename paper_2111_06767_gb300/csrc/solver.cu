@@ -58,18 +58,20 @@ namespace {
 // buffer and a gather.
 template <typename T>
 void curved_apply(dg_domain* dom, Level& L, const T* u, T* out, const T* b, cudaStream_t s, const SubdomainOut* so,
-                  const T* geo, const T* sig, T* trace, const T* D, const T* w, T* r_scratch) {
+                  const T* geo, const T* face, T* trace, T* grad, const T* D, const T* w, T* r_scratch) {
   CurvedArgs<T> a{};
   for (int i = 0; i < 3; ++i) a.n[i] = L.n[i];
   a.neumann = dom->desc.neumann_faces;
   a.ndof = L.ndof;
   a.geo = geo;
-  a.sigma = sig;
+  a.face = face;
+  a.nf = (int64_t)L.E * 6 * dom->N * dom->N;
   a.D = D;
   a.w = w;
   a.u = u;
   a.b = b;
   a.trace = trace;
+  a.grad = grad;
   a.out = so ? r_scratch : out;
   DG_REQUIRE(a.out != nullptr, "curved residual needs the level's work vectors");
   launch_curved_apply<T>(dom->N, a, L.E, s);
@@ -83,7 +85,7 @@ void apply_level(dg_domain* dom, int level, const double* u, double* out, const 
   Level& L = dom->levels[level];
   if (dom->curved) {
     PhaseScope ps(dom->prof, DG_PHASE_APPLY_FP64, s, (double)L.ndof * 8 * (b ? 3 : 2) + 80.0 * L.ndof, 0.0);
-    curved_apply<double>(dom, L, u, out, b, s, so, L.geo64.get(), L.sig64.get(), L.trace64.get(), dom->D64.get(),
+    curved_apply<double>(dom, L, u, out, b, s, so, L.geo64.get(), L.face64.get(), L.trace64.get(), L.grad64.get(), dom->D64.get(),
                          dom->w64.get(), L.w64.r.get());
     return;
   }
@@ -101,7 +103,7 @@ void apply_level_f32(dg_domain* dom, int level, const float* u, float* out, cons
   Level& L = dom->levels[level];
   if (dom->curved) {
     PhaseScope ps(dom->prof, DG_PHASE_APPLY_FP32, s, (double)L.ndof * 4 * (b ? 3 : 2) + 40.0 * L.ndof, 0.0);
-    curved_apply<float>(dom, L, u, out, b, s, so, L.geo32.get(), L.sig32.get(), L.trace32.get(), dom->D32.get(),
+    curved_apply<float>(dom, L, u, out, b, s, so, L.geo32.get(), L.face32.get(), L.trace32.get(), L.grad32.get(), dom->D32.get(),
                         dom->w32.get(), L.w32.r.get());
     return;
   }
