@@ -208,7 +208,7 @@ dg_status dg_mg_restrict(dg_domain* dom, int32_t level, const double* r_fine, do
     DG_REQUIRE(level >= 0 && level + 1 < (int)dom->levels.size(), "level out of range");
     DG_REQUIRE(r_fine && b_coarse, "null pointer");
     dg::launch_restrict<double>(dom->N, dom->levels[level].n, dom->levels[level + 1].n, dom->Ilo64.get(),
-                                dom->Ihi64.get(), r_fine, b_coarse, pick(dom, stream));
+                                dom->Ihi64.get(), r_fine, b_coarse, nullptr, nullptr, nullptr, pick(dom, stream));
   });
 }
 

@@ -215,9 +215,10 @@ void apply_level(dg_domain* dom, int level, const double* u, double* out, const 
 void apply_level_f32(dg_domain* dom, int level, const float* u, float* out, const float* b, bool with_lin,
                      cudaStream_t s, const SubdomainOut* so = nullptr);
 template <typename T>
-void schwarz_smooth(dg_domain* dom, int level, const T* b, T* u, int iterations, bool u_is_zero, cudaStream_t s);
+void schwarz_smooth(dg_domain* dom, int level, const T* b, T* u, int iterations, bool u_is_zero, cudaStream_t s,
+                    bool gathered = false);
 template <typename T>
-void vcycle(dg_domain* dom, const T* r, T* z, cudaStream_t s);
+void vcycle(dg_domain* dom, const T* r, T* z, cudaStream_t s, bool gathered = false);
 void precondition(dg_domain* dom, int mode, const double* v, double* z, cudaStream_t s);
 
 dg_status solve(dg_domain* dom, const double* b, double* u, double tol, const dg_solve_opts& o, dg_solve_report* rep);

@@ -340,9 +340,10 @@ void launch_lin_gemv_half(const uint16_t* Minv, const float* scale, const float*
 template <typename T>
 void launch_prolongate_add(int N, const int nf[3], const int nc[3], const T* Ilo, const T* Ihi, const T* uc, T* uf,
                            cudaStream_t s);
+// With rS the coarse residual also goes straight into the coarse level's subdomain vectors (launch_gather).
 template <typename T>
 void launch_restrict(int N, const int nf[3], const int nc[3], const T* Ilo, const T* Ihi, const T* rf, T* bc,
-                     cudaStream_t s);
+                     const SubdomainGeom* sg, const int4* rec, T* rS, cudaStream_t s);
 
 // Vector kernels.
 template <typename T>
@@ -385,7 +386,7 @@ void launch_kr_start(KrylovState* st, double tol, int max_it, bool rel_to_b, con
 void launch_kr_report(const KrylovState* st, const double* nrm2, double* out, cudaStream_t s);
 template <typename T>
 void launch_kr_next_v(int64_t n, const double* x, const KrylovState* st, double* V, int64_t ld, T* vin,
-                      cudaStream_t s);
+                      const SubdomainGeom& sg, const int4* rec, T* rS, cudaStream_t s);
 template <typename T>
 void launch_kr_store_z(int64_t n, const T* z, const KrylovState* st, double* Z, int64_t ld, double* zfix,
                        cudaStream_t s);

@@ -16,6 +16,7 @@
 // blocks of which most returned at once) took about twice as long: 4.21 -> 3.85 ms a solve of 10 iterations.
 #include "internal.h"
 #include "pdl.cuh"
+#include "schwarz_dev.cuh"
 
 namespace dg {
 
@@ -55,10 +56,13 @@ __global__ void kr_start_kernel(KrylovState* st, double tol, int max_it, int rel
 }
 
 // V_j = scale x and the preconditioner's input, V_j in FP32 (MIXED) or FP64, while the loop runs (j and
-// scale from the state)
-template <typename T>
-__global__ void kr_next_v_kernel(int64_t n, const double* __restrict__ x, const KrylovState* __restrict__ st,
-                                 double* __restrict__ V, int64_t ld, T* __restrict__ vin) {
+// scale from the state); the input also straight into the finest level's subdomain vectors, whose first
+// smoothing step starts from u = 0.
+template <int N, typename T>
+__global__ void kr_next_v_kernel(int n, const double* __restrict__ x, const KrylovState* __restrict__ st,
+                                 double* __restrict__ V, int64_t ld, T* __restrict__ vin, SubdomainGeom sg,
+                                 const int4* __restrict__ rec, T* __restrict__ rS) {
+  constexpr int N3 = N * N * N;
   pdl_launch_dependents();
   pdl_wait();  // the state and vectors come from the previous kernel
   if (st->status != KR_RUNNING) return;
@@ -68,6 +72,8 @@ __global__ void kr_next_v_kernel(int64_t n, const double* __restrict__ x, const 
     const double y = a * x[i];
     v[i] = y;
     vin[i] = (T)y;
+    const int e = (int)i / N3;
+    gather_point<N, T>(sg, rec, (T)y, rS, e, (int)i - e * N3);
   }
 }
 
@@ -367,15 +373,24 @@ void launch_kr_report(const KrylovState* st, const double* nrm2, double* out, cu
 }
 template <typename T>
 void launch_kr_next_v(int64_t n, const double* x, const KrylovState* st, double* V, int64_t ld, T* vin,
-                      cudaStream_t s) {
+                      const SubdomainGeom& sg, const int4* rec, T* rS, cudaStream_t s) {
   const PdlScope pdl(pdl_krylov_enabled());
-  launch_pdl(kr_next_v_kernel<T>, dim3(grid_for(n)), dim3(kThreads), 0, s, n, x, st, V, ld, vin);
+  switch (sg.N) {
+#define DG_CASE(NN)                                                                                                 \
+  case NN:                                                                                                          \
+    launch_pdl(kr_next_v_kernel<NN, T>, dim3(grid_for(n)), dim3(kThreads), 0, s, (int)n, x, st, V, ld, vin, sg, rec, \
+               rS);                                                                                                 \
+    break;
+    DG_CASE(2) DG_CASE(3) DG_CASE(4) DG_CASE(5) DG_CASE(6) DG_CASE(7) DG_CASE(8) DG_CASE(9) DG_CASE(10)
+#undef DG_CASE
+    default: fail(DG_ERR_INVALID_ARG, "unsupported N");
+  }
   DG_LAUNCHED(1);
 }
 template void launch_kr_next_v<float>(int64_t, const double*, const KrylovState*, double*, int64_t, float*,
-                                      cudaStream_t);
+                                      const SubdomainGeom&, const int4*, float*, cudaStream_t);
 template void launch_kr_next_v<double>(int64_t, const double*, const KrylovState*, double*, int64_t, double*,
-                                       cudaStream_t);
+                                       const SubdomainGeom&, const int4*, double*, cudaStream_t);
 template <typename T>
 void launch_kr_store_z(int64_t n, const T* z, const KrylovState* st, double* Z, int64_t ld, double* zfix,
                        cudaStream_t s) {

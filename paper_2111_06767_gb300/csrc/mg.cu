@@ -7,6 +7,7 @@
 // staged in shared memory, sums in a fixed order: deterministic, no atomics.
 #include "internal.h"
 #include "pdl.cuh"
+#include "schwarz_dev.cuh"
 
 namespace dg {
 
@@ -93,7 +94,9 @@ template <int N, typename T>
 __global__ void __launch_bounds__(RestrictShape<N>::threads) restrict_kernel(XferGeom x, const T* __restrict__ Ilo,
                                                                              const T* __restrict__ Ihi,
                                                                              const T* __restrict__ rf,
-                                                                             T* __restrict__ bc) {
+                                                                             T* __restrict__ bc, SubdomainGeom sg,
+                                                                             const int4* __restrict__ rec,
+                                                                             T* __restrict__ rS) {
   constexpr int N2 = N * N, N3 = N2 * N, NT = RestrictShape<N>::threads;
   __shared__ T sI[2 * N2];
   __shared__ T sz[4 * N2], sy[2 * N2];
@@ -160,6 +163,8 @@ __global__ void __launch_bounds__(RestrictShape<N>::threads) restrict_kernel(Xfe
         for (int l = 0; l < N; ++l) a += sI[dx * N2 + l * N + i] * sy[dx * N2 + b * N + l];
     }
     bc[(int64_t)ec * N3 + c * N2 + tid] = a;
+    // the coarse level's first smoothing step starts from u = 0: its residual is b
+    if (rS) gather_point<N, T>(sg, rec, a, rS, ec, c * N2 + tid);
   }
 }
 
@@ -180,12 +185,16 @@ void launch_prolongate_add(int N, const int nf[3], const int nc[3], const T* Ilo
 
 template <typename T>
 void launch_restrict(int N, const int nf[3], const int nc[3], const T* Ilo, const T* Ihi, const T* rf, T* bc,
-                     cudaStream_t s) {
+                     const SubdomainGeom* sg, const int4* rec, T* rS, cudaStream_t s) {
   XferGeom x{{nf[0], nf[1], nf[2]}, {nc[0], nc[1], nc[2]}};
   const int E = nc[0] * nc[1] * nc[2];
+  const SubdomainGeom g = sg ? *sg : SubdomainGeom{};
   switch (N) {
-#define DG_CASE(NN) \
-  case NN: launch_pdl(restrict_kernel<NN, T>, dim3(E * NN), dim3(RestrictShape<NN>::threads), 0, s, x, Ilo, Ihi, rf, bc); break;
+#define DG_CASE(NN)                                                                                                \
+  case NN:                                                                                                         \
+    launch_pdl(restrict_kernel<NN, T>, dim3(E * NN), dim3(RestrictShape<NN>::threads), 0, s, x, Ilo, Ihi, rf, bc, g, \
+               rec, rS);                                                                                           \
+    break;
     DG_CASE(2) DG_CASE(3) DG_CASE(4) DG_CASE(5) DG_CASE(6) DG_CASE(7) DG_CASE(8) DG_CASE(9) DG_CASE(10)
 #undef DG_CASE
     default: fail(DG_ERR_INVALID_ARG, "unsupported N");
@@ -198,8 +207,8 @@ template void launch_prolongate_add<double>(int, const int*, const int*, const d
 template void launch_prolongate_add<float>(int, const int*, const int*, const float*, const float*, const float*,
                                            float*, cudaStream_t);
 template void launch_restrict<double>(int, const int*, const int*, const double*, const double*, const double*,
-                                      double*, cudaStream_t);
+                                      double*, const SubdomainGeom*, const int4*, double*, cudaStream_t);
 template void launch_restrict<float>(int, const int*, const int*, const float*, const float*, const float*, float*,
-                                     cudaStream_t);
+                                     const SubdomainGeom*, const int4*, float*, cudaStream_t);
 
 }  // namespace dg

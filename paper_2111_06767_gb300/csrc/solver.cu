@@ -343,8 +343,10 @@ bool level_pdl(const Level& L) {
   return mode >= 2 || L.E <= (sizeof(T) == 4 ? 1024 : 32);
 }
 
+// gathered: r_S holds R_S b already (u_is_zero).
 template <typename T>
-void schwarz_smooth(dg_domain* dom, int level, const T* b, T* u, int iterations, bool u_is_zero, cudaStream_t s) {
+void schwarz_smooth(dg_domain* dom, int level, const T* b, T* u, int iterations, bool u_is_zero, cudaStream_t s,
+                    bool gathered) {
   ensure_schwarz(dom, level);
   const PdlScope pdl(level_pdl<T>(dom->levels[level]));
   Level& L = dom->levels[level];
@@ -391,7 +393,9 @@ void schwarz_smooth(dg_domain* dom, int level, const T* b, T* u, int iterations,
   for (int it = 0; it < iterations; ++it) {
     const double sz = sizeof(T), vec = (double)L.E * sw.nS * sz;
     const int ld = sw.ld;
-    if (it == 0 && u_is_zero) {
+    if (it == 0 && u_is_zero && gathered) {
+      // the kernel that made b wrote r_S as well
+    } else if (it == 0 && u_is_zero) {
       // with u = 0 the residual is b itself: gather it into the subdomain vectors
       PhaseScope ps(dom->prof, DG_PHASE_GATHER, s, L.ndof * sz + vec, 0.0);
       launch_gather<T>(sw.geom, b, sw.rec.get(), W.rS.get(), s);
@@ -444,12 +448,12 @@ void schwarz_smooth(dg_domain* dom, int level, const T* b, T* u, int iterations,
   }
 }
 
-template void schwarz_smooth<double>(dg_domain*, int, const double*, double*, int, bool, cudaStream_t);
-template void schwarz_smooth<float>(dg_domain*, int, const float*, float*, int, bool, cudaStream_t);
+template void schwarz_smooth<double>(dg_domain*, int, const double*, double*, int, bool, cudaStream_t, bool);
+template void schwarz_smooth<float>(dg_domain*, int, const float*, float*, int, bool, cudaStream_t, bool);
 
-// One V-cycle from a zero initial guess: z ~= A^-1 r.
+// One V-cycle from a zero initial guess: z ~= A^-1 r. gathered: the finest level's r_S holds R_S r already.
 template <typename T>
-void vcycle(dg_domain* dom, const T* r, T* z, cudaStream_t s) {
+void vcycle(dg_domain* dom, const T* r, T* z, cudaStream_t s, bool gathered) {
   const int nl = (int)dom->levels.size();
   const int pre = dom->desc.presmooth, post = dom->desc.postsmooth;
   const int N = dom->N;
@@ -464,17 +468,18 @@ void vcycle(dg_domain* dom, const T* r, T* z, cudaStream_t s) {
       DG_CUDA(cudaMemsetAsync(U(l), 0, sizeof(T) * dom->levels[l].ndof, s));
   for (int l = 0; l < nl - 1; ++l) {
     Level& L = dom->levels[l];
-    schwarz_smooth<T>(dom, l, B(l), U(l), pre, true, s);
+    schwarz_smooth<T>(dom, l, B(l), U(l), pre, true, s, l > 0 || gathered);
     // residual and transfers as the level's smoothing (FP64 transfers are long: 602 against 578 us a V-cycle)
     const PdlScope pdl(sizeof(T) == 4 && level_pdl<T>(L));
     apply_T<T>(dom, l, U(l), work<T>(L).r.get(), B(l), s);  // Eq. mg_res
     PhaseScope ps(dom->prof, DG_PHASE_TRANSFER, s, (double)(L.ndof + dom->levels[l + 1].ndof) * sizeof(T),
                   6.0 * N * L.ndof);
     launch_restrict<T>(N, L.n, dom->levels[l + 1].n, Ilo<T>(dom), Ihi<T>(dom), work<T>(L).r.get(),
-                       work<T>(dom->levels[l + 1]).b.get(), s);
+                       work<T>(dom->levels[l + 1]).b.get(), &dom->levels[l + 1].sw.geom,
+                       dom->levels[l + 1].sw.rec.get(), work<T>(dom->levels[l + 1]).rS.get(), s);
   }
-  schwarz_smooth<T>(dom, nl - 1, B(nl - 1), U(nl - 1), pre, true, s);
-  schwarz_smooth<T>(dom, nl - 1, B(nl - 1), U(nl - 1), post, pre == 0, s);
+  schwarz_smooth<T>(dom, nl - 1, B(nl - 1), U(nl - 1), pre, true, s, nl > 1 || gathered);
+  schwarz_smooth<T>(dom, nl - 1, B(nl - 1), U(nl - 1), post, pre == 0, s, nl > 1 || gathered);
   for (int l = nl - 2; l >= 0; --l) {
     Level& L = dom->levels[l];
     {
@@ -487,8 +492,8 @@ void vcycle(dg_domain* dom, const T* r, T* z, cudaStream_t s) {
   }
 }
 
-template void vcycle<double>(dg_domain*, const double*, double*, cudaStream_t);
-template void vcycle<float>(dg_domain*, const float*, float*, cudaStream_t);
+template void vcycle<double>(dg_domain*, const double*, double*, cudaStream_t, bool);
+template void vcycle<float>(dg_domain*, const float*, float*, cudaStream_t, bool);
 
 namespace {
 
@@ -880,8 +885,11 @@ void capture_solve_branch(dg_domain* dom, cudaGraph_t graph, int cap, double tol
     if (rel_to_b) launch_multidot(n, 1, kb, n, kb, part, nrm + 1, gs);
     launch_kr_start(st, tol, cap, rel_to_b, nrm, g, loop, gs);
     auto next_v = [&](const double* x, cudaStream_t q) {  // V_j and the V-cycle's input
-      if (dom->mixed) launch_kr_next_v<float>(n, x, st, V, n, dom->vin32.get(), q);
-      else launch_kr_next_v<double>(n, x, st, V, n, dom->vin64.get(), q);
+      const Level& L = dom->levels[0];
+      if (dom->mixed)
+        launch_kr_next_v<float>(n, x, st, V, n, dom->vin32.get(), L.sw.geom, L.sw.rec.get(), L.w32.rS.get(), q);
+      else
+        launch_kr_next_v<double>(n, x, st, V, n, dom->vin64.get(), L.sw.geom, L.sw.rec.get(), L.w64.rS.get(), q);
     };
     next_v(r, gs);
     // the Arnoldi loop: a conditional WHILE node after the prologue
@@ -904,10 +912,10 @@ void capture_solve_branch(dg_domain* dom, cudaGraph_t graph, int cap, double tol
     try {
       if (dom->mixed) {
         float* v32 = dom->vin32.get();
-        vcycle<float>(dom, v32, v32 + n, bs);
+        vcycle<float>(dom, v32, v32 + n, bs, true);
         launch_kr_store_z<float>(n, v32 + n, st, Z, n, dom->zfix.get(), bs);
       } else {
-        vcycle<double>(dom, dom->vin64.get(), dom->vout64.get(), bs);
+        vcycle<double>(dom, dom->vin64.get(), dom->vout64.get(), bs, true);
         launch_kr_store_z<double>(n, dom->vout64.get(), st, Z, n, dom->zfix.get(), bs);
       }
       apply_level(dom, 0, dom->zfix.get(), w, nullptr, true, bs);
