@@ -89,6 +89,12 @@ bool pdl_krylov_enabled() {
   }();
   return on;
 }
+namespace {
+thread_local int tl_shared_scope = 0;
+}
+SharedGpuScope::SharedGpuScope(bool on_) : on(on_) { tl_shared_scope += on; }
+SharedGpuScope::~SharedGpuScope() { tl_shared_scope -= on; }
+bool gpu_is_shared() { return tl_shared_scope > 0; }
 int pdl_vcycle_mode() {
   static const int mode = [] {
     const char* v = std::getenv("DG_PDL_COARSE");

@@ -62,6 +62,16 @@ struct PdlScope {
   PdlScope& operator=(const PdlScope&) = delete;
 };
 int pdl_vcycle_mode();
+// While alive on this thread: launches are for many solves that share the GPU (a batch's capture), so
+// launch shapes spend less of it on one solve's latency.
+struct SharedGpuScope {
+  bool on;
+  explicit SharedGpuScope(bool on_);
+  ~SharedGpuScope();
+  SharedGpuScope(const SharedGpuScope&) = delete;
+  SharedGpuScope& operator=(const SharedGpuScope&) = delete;
+};
+bool gpu_is_shared();
 bool pdl_krylov_enabled();  // the device-resident FGMRES kernels (DG_PDL_KRYLOV=1 turns it on)
 
 struct AllocStreamScope {
