@@ -40,7 +40,7 @@ namespace {
 // of the FMA instructions themselves: the LGL weights of every supported N and Dhat of N = 4.
 constexpr int wtab_off(int N) { return N * (N - 1) / 2 - 1; }  // sum_{m=2}^{N-1} m
 constexpr int kWTab = wtab_off(DG_MAX_N + 1);
-__constant__ float cD4[16];
+__constant__ float2 cDD4[16], cB4[8];
 __constant__ double cW64[kWTab];
 __constant__ float cW32[kWTab];
 
@@ -90,10 +90,17 @@ __device__ __forceinline__ void row4_g(const float* __restrict__ p, float (&r)[4
 // face point of a face normal to d. Values are held as pairs of x-neighbouring points, so that the
 // contractions and most face terms run as packed two-wide FP32 FMAs (one instruction per pair):
 // the thread's 64-value working set leaves too few warps per SM to hide latency otherwise.
+// What bounds it: the instructions of 8 warps per SM (255 registers a thread), with the wait for the staged box
+// between them; so the gradient stays in reference units (one scaling per direction, squared, at the divergence), a
+// face point is five operations, and Dhat is read from constant memory as pairs. Measured at 96^3 elements (56.6M
+// points): 162 us with scalar constants and scaled gradients, 147 us with the reference units, 129 us with the pairs
+// (0.52 of the HBM copy rate). Bricks staged without their edges (seven boxes): 136 us, 4 x 4 x 4 and
+// 8 x 4 x 2 bricks of that form 127 us, not worth four more tensor maps a launch.
 constexpr int kE4Slot = 68;  // words per staged element
 
 struct E4Tab {
-  static __device__ __forceinline__ float D(int o) { return cD4[o]; }
+  static __device__ __forceinline__ float2 DD(int o) { return cDD4[o]; }  // (D, D)
+  static __device__ __forceinline__ float2 B(int o) { return cB4[o]; }    // pairs of the x-contraction
   static __device__ __forceinline__ float w(int o) { return cW32[wtab_off(4) + o]; }
 };
 
@@ -122,41 +129,31 @@ __device__ __forceinline__ void ld4s(const float* p, float (&r)[4]) {
   r[3] = v.w;
 }
 
-// Lifting and flux of one face point, as face_point() above, with the flux added to the point's
-// pre-mass sum acc (cf = Bf / M of the point).
-__device__ __forceinline__ float e4_face(float s, float ui, float gi, float ue, float ge, bool has, bool neu,
-                                         float lift, float sml, float cf, float& acc) {
-  const float uE = has ? ue : (neu ? ui : -ui);
-  const float gE = has ? ge : (neu ? -gi : gi);
-  const float jump = uE - ui;
-  acc += cf * (0.5f * s * (gE - gi) + sml * jump);
-  return gi + s * jump * lift;
-}
-
-// Ghost-state blend of one face (Eq. bc): the exterior value is a ue + b ui and the exterior
-// normal derivative c ge + d gi, with (a, b, c, d) = (1, 0, 1, 0) where the neighbour exists, else
-// (0, -1, 0, 1) on a Dirichlet and (0, 1, 0, -1) on a Neumann face.
+// One face in reference units: gi and ge are the derivatives along the reference coordinate (physical / dxi), and
+// ue, ge are zero where there is no neighbour (the staged box is filled with zeros there). The jump uE - ui is then
+// ue + bj ui and the derivative's ge + bg gi, with (bj, bg) = (-1, -1) where the neighbour exists, (-2, 0) on a
+// Dirichlet and (0, -2) on a Neumann face, and a face point is five operations: two of these, the flux
+// cf (s / 2 dxi dg + sml jump) into the pre-mass sum (cf = Bf / M of the point), and the lifting.
 struct E4Face {
-  float2 a, b, c, d, hs, sl, sml, cf;  // hs = s / 2, sl = s lift (both halves equal)
-  __device__ __forceinline__ E4Face(float s, bool has, bool neu, float lift, float sml_, float cf_) {
-    const float bb = has ? 0.f : (neu ? 1.f : -1.f);
-    a = make_float2(has ? 1.f : 0.f, has ? 1.f : 0.f);
-    b = make_float2(bb, bb);
-    c = a;
-    d = make_float2(-bb, -bb);
-    hs = make_float2(0.5f * s, 0.5f * s);
-    sl = make_float2(s * lift, s * lift);
-    sml = make_float2(sml_, sml_);
-    cf = make_float2(cf_, cf_);
+  float bj, bg, ch, cs, sl;
+  __device__ __forceinline__ E4Face(float s, bool has, bool neu, float dxi, float lift, float sml, float cf) {
+    bj = has ? -1.f : (neu ? 0.f : -2.f);
+    bg = has ? -1.f : (neu ? -2.f : 0.f);
+    ch = 0.5f * s * dxi * cf;
+    cs = cf * sml;
+    sl = s * lift / dxi;
   }
-  // two face points at once: returns the lifted gradient component, adds the flux to acc
+  // returns the lifted derivative, adds the flux to acc
+  __device__ __forceinline__ float apply(float ui, float gi, float ue, float ge, float& acc) const {
+    const float jump = fmaf(bj, ui, ue), dg = fmaf(bg, gi, ge);
+    acc = fmaf(cs, jump, fmaf(ch, dg, acc));
+    return fmaf(sl, jump, gi);
+  }
+  // two face points at once
   __device__ __forceinline__ float2 apply(float2 ui, float2 gi, float2 ue, float2 ge, float2& acc) const {
-    const float2 uE = __ffma2_rn(a, ue, __fmul2_rn(b, ui));
-    const float2 gE = __ffma2_rn(c, ge, __fmul2_rn(d, gi));
-    const float2 jump = __fadd2_rn(uE, make_float2(-ui.x, -ui.y));
-    const float2 dg = __fadd2_rn(gE, make_float2(-gi.x, -gi.y));
-    acc = __ffma2_rn(cf, __ffma2_rn(hs, dg, __fmul2_rn(sml, jump)), acc);
-    return __ffma2_rn(sl, jump, gi);
+    const float2 jump = __ffma2_rn(make_float2(bj, bj), ui, ue), dg = __ffma2_rn(make_float2(bg, bg), gi, ge);
+    acc = __ffma2_rn(make_float2(cs, cs), jump, __ffma2_rn(make_float2(ch, ch), dg, acc));
+    return __ffma2_rn(make_float2(sl, sl), jump, gi);
   }
 };
 
@@ -167,7 +164,7 @@ __global__ void __launch_bounds__(BX* BY* BZ, E4Shape<BX, BY, BZ>::PER_SM)
   using S = E4Shape<BX, BY, BZ>;
   using C = E4Tab;
   constexpr int SL = kE4Slot, PX = S::PX, PY = S::PY;
-  constexpr int dO = 0, wO = 0;
+  constexpr int wO = 0;
   extern __shared__ __align__(128) unsigned char e4_raw[];
   // 128-byte aligned for TMA; offset from the shared array itself, so that the compiler keeps
   // every access in the shared window (LDS/STS rather than generic loads)
@@ -220,20 +217,11 @@ __global__ void __launch_bounds__(BX* BY* BZ, E4Shape<BX, BY, BZ>::PER_SM)
   const float w0 = C::w(wO);
   const float cfx = g.Jf[0] / (g.J * w0), cfy = g.Jf[1] / (g.J * w0), cfz = g.Jf[2] / (g.J * w0);
   const float smx = g.sigma[0] - g.lift[0], smy = g.sigma[1] - g.lift[1], smz = g.sigma[2] - g.lift[2];
-  const float2 dy2 = make_float2(g.dxi[1], g.dxi[1]), dz2 = make_float2(g.dxi[2], g.dxi[2]);
+  const float sx = g.dxi[0] * g.dxi[0], sy = g.dxi[1] * g.dxi[1], sz = g.dxi[2] * g.dxi[2];
+  const float2 dx2 = make_float2(sx, sx), dy2 = make_float2(sy, sy), dz2 = make_float2(sz, sz);
   // x: gradient component along the thread's lines, faces from the x-neighbours' lines, divergence.
   // Along a line the pairs multiply 2 x 2 blocks of Dhat: (y0, y1) = (D00, D11) (x0, x1) +
   // (D01, D10) (x1, x0) + (D02, D13) (x2, x3) + (D03, D12) (x3, x2), and likewise for (y2, y3).
-  float2 Bx[8];
-#pragma unroll
-  for (int q = 0; q < 2; ++q)      // output pair
-#pragma unroll
-    for (int c = 0; c < 2; ++c) {  // input pair
-      const int r0 = 2 * q, c0 = 2 * c;
-      Bx[4 * q + 2 * c] = make_float2(C::D(dO + r0 * 4 + c0), C::D(dO + (r0 + 1) * 4 + c0 + 1));
-      Bx[4 * q + 2 * c + 1] = make_float2(C::D(dO + r0 * 4 + c0 + 1), C::D(dO + (r0 + 1) * 4 + c0));
-    }
-  const float2 dx2 = make_float2(g.dxi[0], g.dxi[0]);
 #pragma unroll
   for (int k = 0; k < 4; ++k)
 #pragma unroll
@@ -241,13 +229,15 @@ __global__ void __launch_bounds__(BX* BY* BZ, E4Shape<BX, BY, BZ>::PER_SM)
       const float2 sw[2] = {make_float2(U[k][j][0].y, U[k][j][0].x), make_float2(U[k][j][1].y, U[k][j][1].x)};
 #pragma unroll
       for (int q = 0; q < 2; ++q) {
-        float2 a = __fmul2_rn(Bx[4 * q], U[k][j][0]);
-        a = __ffma2_rn(Bx[4 * q + 1], sw[0], a);
-        a = __ffma2_rn(Bx[4 * q + 2], U[k][j][1], a);
-        a = __ffma2_rn(Bx[4 * q + 3], sw[1], a);
-        G[k][j][q] = __fmul2_rn(dx2, a);
+        float2 a = __fmul2_rn(C::B(4 * q), U[k][j][0]);
+        a = __ffma2_rn(C::B(4 * q + 1), sw[0], a);
+        a = __ffma2_rn(C::B(4 * q + 2), U[k][j][1], a);
+        a = __ffma2_rn(C::B(4 * q + 3), sw[1], a);
+        G[k][j][q] = a;
       }
     }
+  const E4Face fmx(-1.f, hxm, g.neumann & 1, g.dxi[0], g.lift[0], smx, cfx),
+      fpx(1.f, hxp, (g.neumann >> 1) & 1, g.dxi[0], g.lift[0], smx, cfx);
 #pragma unroll
   for (int k = 0; k < 4; ++k)
 #pragma unroll
@@ -256,15 +246,13 @@ __global__ void __launch_bounds__(BX* BY* BZ, E4Shape<BX, BY, BZ>::PER_SM)
       ld4s(me - DX + k * 16 + j * 4, r);
       float ge = 0.f;
 #pragma unroll
-      for (int l = 0; l < 4; ++l) ge += C::D(dO + 12 + l) * r[l];
-      G[k][j][0].x = e4_face(-1.f, U[k][j][0].x, G[k][j][0].x, r[3], g.dxi[0] * ge, hxm, g.neumann & 1, g.lift[0],
-                             smx, cfx, ACC[k][j][0].x);
+      for (int l = 0; l < 4; ++l) ge += C::DD(12 + l).x * r[l];
+      G[k][j][0].x = fmx.apply(U[k][j][0].x, G[k][j][0].x, r[3], ge, ACC[k][j][0].x);
       ld4s(me + DX + k * 16 + j * 4, r);
       ge = 0.f;
 #pragma unroll
-      for (int l = 0; l < 4; ++l) ge += C::D(dO + l) * r[l];
-      G[k][j][1].y = e4_face(1.f, U[k][j][1].y, G[k][j][1].y, r[0], g.dxi[0] * ge, hxp, (g.neumann >> 1) & 1,
-                             g.lift[0], smx, cfx, ACC[k][j][1].y);
+      for (int l = 0; l < 4; ++l) ge += C::DD(l).x * r[l];
+      G[k][j][1].y = fpx.apply(U[k][j][1].y, G[k][j][1].y, r[0], ge, ACC[k][j][1].y);
     }
 #pragma unroll
   for (int k = 0; k < 4; ++k)
@@ -273,10 +261,10 @@ __global__ void __launch_bounds__(BX* BY* BZ, E4Shape<BX, BY, BZ>::PER_SM)
       const float2 sw[2] = {make_float2(G[k][j][0].y, G[k][j][0].x), make_float2(G[k][j][1].y, G[k][j][1].x)};
 #pragma unroll
       for (int q = 0; q < 2; ++q) {
-        float2 a = __fmul2_rn(Bx[4 * q], G[k][j][0]);
-        a = __ffma2_rn(Bx[4 * q + 1], sw[0], a);
-        a = __ffma2_rn(Bx[4 * q + 2], G[k][j][1], a);
-        a = __ffma2_rn(Bx[4 * q + 3], sw[1], a);
+        float2 a = __fmul2_rn(C::B(4 * q), G[k][j][0]);
+        a = __ffma2_rn(C::B(4 * q + 1), sw[0], a);
+        a = __ffma2_rn(C::B(4 * q + 2), G[k][j][1], a);
+        a = __ffma2_rn(C::B(4 * q + 3), sw[1], a);
         ACC[k][j][q] = __ffma2_rn(dx2, a, ACC[k][j][q]);
       }
     }
@@ -290,14 +278,13 @@ __global__ void __launch_bounds__(BX* BY* BZ, E4Shape<BX, BY, BZ>::PER_SM)
         float2 a = make_float2(0.f, 0.f);
 #pragma unroll
         for (int l = 0; l < 4; ++l) {
-          const float d = C::D(dO + j * 4 + l);
-          a = __ffma2_rn(make_float2(d, d), U[k][l][p], a);
+          a = __ffma2_rn(C::DD(j * 4 + l), U[k][l][p], a);
         }
-        G[k][j][p] = __fmul2_rn(dy2, a);
+        G[k][j][p] = a;
       }
   {
-    const E4Face fm(-1.f, hym, (g.neumann >> 2) & 1, g.lift[1], smy, cfy), fp(1.f, hyp, (g.neumann >> 3) & 1,
-                                                                            g.lift[1], smy, cfy);
+    const E4Face fm(-1.f, hym, (g.neumann >> 2) & 1, g.dxi[1], g.lift[1], smy, cfy),
+        fp(1.f, hyp, (g.neumann >> 3) & 1, g.dxi[1], g.lift[1], smy, cfy);
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
       float2 r[4][2];
@@ -308,10 +295,9 @@ __global__ void __launch_bounds__(BX* BY* BZ, E4Shape<BX, BY, BZ>::PER_SM)
         float2 ge = make_float2(0.f, 0.f);
 #pragma unroll
         for (int l = 0; l < 4; ++l) {
-          const float dd = C::D(dO + 12 + l);
-          ge = __ffma2_rn(make_float2(dd, dd), r[l][p], ge);
+          ge = __ffma2_rn(C::DD(12 + l), r[l][p], ge);
         }
-        G[k][0][p] = fm.apply(U[k][0][p], G[k][0][p], r[3][p], __fmul2_rn(dy2, ge), ACC[k][0][p]);
+        G[k][0][p] = fm.apply(U[k][0][p], G[k][0][p], r[3][p], ge, ACC[k][0][p]);
       }
 #pragma unroll
       for (int l = 0; l < 4; ++l) ld4p(me + DY + k * 16 + l * 4, r[l]);
@@ -320,10 +306,9 @@ __global__ void __launch_bounds__(BX* BY* BZ, E4Shape<BX, BY, BZ>::PER_SM)
         float2 ge = make_float2(0.f, 0.f);
 #pragma unroll
         for (int l = 0; l < 4; ++l) {
-          const float dd = C::D(dO + l);
-          ge = __ffma2_rn(make_float2(dd, dd), r[l][p], ge);
+          ge = __ffma2_rn(C::DD(l), r[l][p], ge);
         }
-        G[k][3][p] = fp.apply(U[k][3][p], G[k][3][p], r[0][p], __fmul2_rn(dy2, ge), ACC[k][3][p]);
+        G[k][3][p] = fp.apply(U[k][3][p], G[k][3][p], r[0][p], ge, ACC[k][3][p]);
       }
     }
   }
@@ -336,8 +321,7 @@ __global__ void __launch_bounds__(BX* BY* BZ, E4Shape<BX, BY, BZ>::PER_SM)
         float2 a = make_float2(0.f, 0.f);
 #pragma unroll
         for (int l = 0; l < 4; ++l) {
-          const float d = C::D(dO + j * 4 + l);
-          a = __ffma2_rn(make_float2(d, d), G[k][l][p], a);
+          a = __ffma2_rn(C::DD(j * 4 + l), G[k][l][p], a);
         }
         ACC[k][j][p] = __ffma2_rn(dy2, a, ACC[k][j][p]);
       }
@@ -351,14 +335,13 @@ __global__ void __launch_bounds__(BX* BY* BZ, E4Shape<BX, BY, BZ>::PER_SM)
         float2 a = make_float2(0.f, 0.f);
 #pragma unroll
         for (int l = 0; l < 4; ++l) {
-          const float d = C::D(dO + k * 4 + l);
-          a = __ffma2_rn(make_float2(d, d), U[l][j][p], a);
+          a = __ffma2_rn(C::DD(k * 4 + l), U[l][j][p], a);
         }
-        G[k][j][p] = __fmul2_rn(dz2, a);
+        G[k][j][p] = a;
       }
   {
-    const E4Face fm(-1.f, hzm, (g.neumann >> 4) & 1, g.lift[2], smz, cfz), fp(1.f, hzp, (g.neumann >> 5) & 1,
-                                                                            g.lift[2], smz, cfz);
+    const E4Face fm(-1.f, hzm, (g.neumann >> 4) & 1, g.dxi[2], g.lift[2], smz, cfz),
+        fp(1.f, hzp, (g.neumann >> 5) & 1, g.dxi[2], g.lift[2], smz, cfz);
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
       float2 r[4][2];
@@ -369,10 +352,9 @@ __global__ void __launch_bounds__(BX* BY* BZ, E4Shape<BX, BY, BZ>::PER_SM)
         float2 ge = make_float2(0.f, 0.f);
 #pragma unroll
         for (int l = 0; l < 4; ++l) {
-          const float dd = C::D(dO + 12 + l);
-          ge = __ffma2_rn(make_float2(dd, dd), r[l][p], ge);
+          ge = __ffma2_rn(C::DD(12 + l), r[l][p], ge);
         }
-        G[0][j][p] = fm.apply(U[0][j][p], G[0][j][p], r[3][p], __fmul2_rn(dz2, ge), ACC[0][j][p]);
+        G[0][j][p] = fm.apply(U[0][j][p], G[0][j][p], r[3][p], ge, ACC[0][j][p]);
       }
 #pragma unroll
       for (int l = 0; l < 4; ++l) ld4p(me + DZ + l * 16 + j * 4, r[l]);
@@ -381,10 +363,9 @@ __global__ void __launch_bounds__(BX* BY* BZ, E4Shape<BX, BY, BZ>::PER_SM)
         float2 ge = make_float2(0.f, 0.f);
 #pragma unroll
         for (int l = 0; l < 4; ++l) {
-          const float dd = C::D(dO + l);
-          ge = __ffma2_rn(make_float2(dd, dd), r[l][p], ge);
+          ge = __ffma2_rn(C::DD(l), r[l][p], ge);
         }
-        G[3][j][p] = fp.apply(U[3][j][p], G[3][j][p], r[0][p], __fmul2_rn(dz2, ge), ACC[3][j][p]);
+        G[3][j][p] = fp.apply(U[3][j][p], G[3][j][p], r[0][p], ge, ACC[3][j][p]);
       }
     }
   }
@@ -397,29 +378,40 @@ __global__ void __launch_bounds__(BX* BY* BZ, E4Shape<BX, BY, BZ>::PER_SM)
         float2 a = make_float2(0.f, 0.f);
 #pragma unroll
         for (int l = 0; l < 4; ++l) {
-          const float d = C::D(dO + k * 4 + l);
-          a = __ffma2_rn(make_float2(d, d), G[l][j][p], a);
+          a = __ffma2_rn(C::DD(k * 4 + l), G[l][j][p], a);
         }
         ACC[k][j][p] = __ffma2_rn(dz2, a, ACC[k][j][p]);
       }
   // A u = -M acc (+ diag u); b - A u with b
   const bool valid = cx < g.nx && cy < g.ny && cz < g.nz;
   const int64_t e = valid ? ((int64_t)cz * g.ny + cy) * g.nx + cx : 0;
+  const float2 w01 = make_float2(C::w(wO), C::w(wO + 1)), w10 = make_float2(w01.y, w01.x);  // weights are symmetric
 #pragma unroll
   for (int k = 0; k < 4; ++k)
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-      float dl[4], bl[4];
-      if (A.diag && valid) row4_g(A.diag + e * 64 + k * 16 + j * 4, dl);
-      if (A.b && valid) row4_g(A.b + e * 64 + k * 16 + j * 4, bl);
-      const float mjk = -g.J * C::w(wO + j) * C::w(wO + k);
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        float res = mjk * C::w(wO + i) * E4(ACC, k, j, i);
-        if (A.diag && valid) res += dl[i] * E4(U, k, j, i);
-        E4(ACC, k, j, i) = (A.b && valid) ? bl[i] - res : res;
-      }
+      const float m = -g.J * (j == 0 || j == 3 ? w01.x : w01.y) * (k == 0 || k == 3 ? w01.x : w01.y);
+      ACC[k][j][0] = __fmul2_rn(__fmul2_rn(make_float2(m, m), w01), ACC[k][j][0]);
+      ACC[k][j][1] = __fmul2_rn(__fmul2_rn(make_float2(m, m), w10), ACC[k][j][1]);
     }
+  if (A.diag && valid) {
+#pragma unroll
+    for (int q = 0; q < 16; ++q) {
+      float dl[4];
+      row4_g(A.diag + e * 64 + q * 4, dl);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) E4(ACC, q >> 2, q & 3, i) += dl[i] * E4(U, q >> 2, q & 3, i);
+    }
+  }
+  if (A.b && valid) {
+#pragma unroll
+    for (int q = 0; q < 16; ++q) {
+      float bl[4];
+      row4_g(A.b + e * 64 + q * 4, bl);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) E4(ACC, q >> 2, q & 3, i) = bl[i] - E4(ACC, q >> 2, q & 3, i);
+    }
+  }
 #undef E4
   __syncthreads();  // every read of the staged box is done: its first slots take the result
   float* o = sm + tid * SL;
@@ -813,7 +805,15 @@ void upload_operator_tables() {
   DG_CUDA(cudaMemcpyToSymbol(cQP32, QP32.data(), sizeof(float2) * kDirPairs));
   DG_CUDA(cudaMemcpyToSymbol(cV64, V.data(), sizeof(double) * kDirVec));
   DG_CUDA(cudaMemcpyToSymbol(cV32, V32.data(), sizeof(float) * kDirVec));
-  DG_CUDA(cudaMemcpyToSymbol(cD4, D4.data(), sizeof(float) * 16));
+  float2 DD4[16], B4[8];
+  for (int o = 0; o < 16; ++o) DD4[o] = make_float2(D4[o], D4[o]);
+  for (int q = 0; q < 4; ++q) {  // output pair q / 2, input pair q % 2
+    const float* d = &D4[q / 2 * 8 + q % 2 * 2];
+    B4[2 * q] = make_float2(d[0], d[5]);
+    B4[2 * q + 1] = make_float2(d[1], d[4]);
+  }
+  DG_CUDA(cudaMemcpyToSymbol(cDD4, DD4, sizeof(DD4)));
+  DG_CUDA(cudaMemcpyToSymbol(cB4, B4, sizeof(B4)));
   DG_CUDA(cudaMemcpyToSymbol(cW64, W.data(), sizeof(double) * kWTab));
   DG_CUDA(cudaMemcpyToSymbol(cW32, W32.data(), sizeof(float) * kWTab));
   done.insert(dev);
