@@ -165,7 +165,7 @@ OpGeom<T> make_geom(const int n[3], const double h[3], int N, double penalty, co
 // ------------------------------------------------------------------ kernels (launchers)
 
 // Optional destination of the apply: instead of `out`, write every result point into the subdomain
-// vectors that contain it (rows from the orientation point maps), i.e. the Schwarz gather fused
+// vectors that contain it (rows from the subdomain records), i.e. the Schwarz gather fused
 // into the residual computation.
 struct SubdomainOut {
   void* rS = nullptr;            // T*: [columns][ld]

@@ -55,7 +55,7 @@ size_t estimate_domain_bytes(const dg_domain_desc& d, int max_iterations, bool l
   const size_t ld = (nS + 31) / 32 * 32;
   const bool mixed = d.precision == DG_PRECISION_MIXED;
   const size_t fb = mixed ? 4 : 8;
-  size_t total = (size_t)48 * (nS + 7 * N * N * N) * 4 + (size_t)64 * N * N * N * 7 * fb;  // point maps, shares
+  size_t total = (size_t)48 * (nS + 7 * N * N * N) * 4 + (size_t)64 * N * N * N * 7 * fb;  // subdomain records, shares
   int n[3] = {d.n[0], d.n[1], d.n[2]};
   size_t build_peak = 0;
   for (int l = 0; l < DG_MAX_LEVELS; ++l) {
