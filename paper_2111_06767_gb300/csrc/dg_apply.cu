@@ -93,9 +93,9 @@ __device__ __forceinline__ void row4_g(const float* __restrict__ p, float (&r)[4
 // What bounds it: the instructions of 8 warps per SM (255 registers a thread), with the wait for the staged box
 // between them; so the gradient stays in reference units (one scaling per direction, squared, at the divergence), a
 // face point is five operations, and Dhat is read from constant memory as pairs. Measured at 96^3 elements (56.6M
-// points): 162 us with scalar constants and scaled gradients, 147 us with the reference units, 129 us with the pairs
-// (0.52 of the HBM copy rate). Bricks staged without their edges (seven boxes): 136 us, 4 x 4 x 4 and
-// 8 x 4 x 2 bricks of that form 127 us, not worth four more tensor maps a launch.
+// points): 162 us with scalar constants and scaled gradients (3190 instructions an element), 147 us with the
+// reference units, 129 us with the pairs (2190; 0.52 of the HBM copy rate). Bricks staged without their edges (seven
+// boxes): 136 us, 4 x 4 x 4 and 8 x 4 x 2 bricks of that form 127 us, not worth four more tensor maps a launch.
 constexpr int kE4Slot = 68;  // words per staged element
 
 struct E4Tab {
