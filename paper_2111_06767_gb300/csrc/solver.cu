@@ -304,9 +304,9 @@ void class_gemm<float>(dg_domain* dom, Level& L, const float* X, float* Y, cudaS
     }
     // Many solves at once: the tuned K split is the one with the shortest launch on an idle GPU, and each
     // further CTA of a cluster costs its fixed part of the others' time. 20 uneven solves in one graph: tuned
-    // splits 21.1 ms, 1 20.7, 2 19.8, 4 22.5.
+    // splits 21.1 ms, 1 20.7, 2 19.8, 4 22.5. A pinned split stays.
     int shape = L.gemm_split;
-    if (gpu_is_shared() && (sw.ld / 32) / 2 >= 4) shape = (shape & kWide) | 2;
+    if (gpu_is_shared() && (sw.ld / 32) / 2 >= 4 && !std::getenv("DG_GEMM_SPLIT")) shape = (shape & kWide) | 2;
     run(shape);
   } else
     simt_class_gemm<float>(L, sw.inv32.get(), X, Y, (float)sw.inv_scale, s);
