@@ -2,10 +2,12 @@
 // (Sec. III.C.3), flexible GMRES (Sec. III.B, Saad Alg. 9.6) and Newton-Raphson with a line
 // search (Sec. III.A). All vector work runs in the library's kernels; the host only keeps the
 // (k+1) x k Hessenberg matrix and its Givens rotations, read back once per Krylov iteration.
+#include <algorithm>
 #include <chrono>
 #include <cmath>
 #include <cstdlib>
 #include <cstring>
+#include <numeric>
 #include <thread>
 #include <type_traits>
 
@@ -1103,11 +1105,19 @@ dg_batch* batch_create(dg_domain* const* doms, const double* const* b, double* c
   DG_CUDA(cudaGraphCreate(&graph, 0));
   try {
     const SharedGpuScope shared(count >= 4);
-    for (int i = 0; i < count; ++i) {
+    // Largest solves first: the branches queue on fewer hardware queues than there are solves, and a long one
+    // that starts late runs on alone. 20 uneven solves: as given 19.7 ms, smallest first 19.4, largest first 19.0.
+    std::vector<int> order(count);
+    std::iota(order.begin(), order.end(), 0);
+    std::stable_sort(order.begin(), order.end(),
+                     [&](int p, int q) { return doms[p]->levels[0].ndof > doms[q]->levels[0].ndof; });
+    bt->fixed.resize(count);
+    bt->body.resize(count);
+    for (int i : order) {
       capture_solve_branch(doms[i], graph, bt->cap, tol, o.relative_to_b != 0, b[i], u[i],
                            bt->reports.get() + 8 * (size_t)i);
-      bt->fixed.push_back(doms[i]->sgraph_fixed_kernels);
-      bt->body.push_back(doms[i]->sgraph_body_kernels);
+      bt->fixed[i] = doms[i]->sgraph_fixed_kernels;
+      bt->body[i] = doms[i]->sgraph_body_kernels;
     }
     DG_CUDA(cudaGraphInstantiate(&bt->exec, graph, 0));
   } catch (...) {
