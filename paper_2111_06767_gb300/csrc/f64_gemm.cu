@@ -116,7 +116,7 @@ __device__ __forceinline__ double combine(int64_t H, int64_t L, int e) {
   return neg ? -v : v;
 }
 
-constexpr int kNonFinite = 1 << 20;  // scale exponent of a column with a NaN or an infinity
+constexpr int kNonFinite = 1 << 20;  // scale exponent of a row or column with a NaN or an infinity
 
 template <int SPLIT>
 __global__ void __launch_bounds__(THREADS, 1)
@@ -284,7 +284,7 @@ __global__ void __launch_bounds__(THREADS, 1)
   auto output = [&](int64_t h, int64_t l, int er, int c) {
     const int ec = col_exp[col0 + c];
     if (zero) return 0.0;
-    return ec == kNonFinite ? __longlong_as_double(0x7FF8000000000000ll) : combine(h, l, er + ec);
+    return ec == kNonFinite || er == kNonFinite ? __longlong_as_double(0x7FF8000000000000ll) : combine(h, l, er + ec);
   };
   if constexpr (SPLIT == 1) {
     if (warp < 8 && row < ld) {
@@ -364,7 +364,7 @@ __global__ void equilibrate_kernel(const double* __restrict__ inv, int ld, int* 
 // dst[group][digit][row][ld], and the row's exponent e, every |x| < 2^e. Values are taken times
 // 2^(sign h_k), h of the row's class (class_of[row], or the group), and times alpha (the inverses, once
 // at set-up). A row with a NaN or an infinity gets the exponent kNonFinite, which the product hands on
-// as NaN to its whole column. Integer arithmetic: the FP64 pipe would take ten times as long.
+// as NaN: for r_S to the whole column, for an inverse to the row of every column of its class. Integer arithmetic: the FP64 pipe would take ten times as long.
 template <bool ALPHA>
 __global__ void __launch_bounds__(256) slice_kernel(const double* __restrict__ src, int ld, double alpha, int sign,
                                                     const int* __restrict__ hexp, const int* __restrict__ class_of,
