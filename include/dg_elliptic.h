@@ -100,9 +100,12 @@ typedef struct dg_domain_desc {
 } dg_domain_desc;
 
 enum dg_subdomain_gemm {
-  DG_GEMM_DEFAULT = 0,      /* MIXED: tensor cores (TF32 inputs, FP32 accumulate); FP64: tensor cores on exact
-                               7-bit digits of the FP64 operands, where the GPU and the memory for the digits
-                               allow it, else (and in served requests) CUDA cores */
+  DG_GEMM_DEFAULT = 0,      /* MIXED: tensor cores (TF32 inputs, FP32 accumulate); FP64: tensor cores on 7-bit
+                               digits of the FP64 operands, whose products and sums are exact, where the GPU and the
+                               memory for the digits allow it, else (and in served requests) CUDA cores. The digits
+                               hold the inverses with all their bits and r_S to 2^-84 or less of a subdomain's
+                               largest value, so that, as with FP64 sums, the error of every component is of the
+                               order of 2^-53 (|A_S^-1| |r_S|) */
   DG_GEMM_SIMT = 1,         /* FP32 (or FP64) CUDA-core GEMM */
   DG_GEMM_TENSOR_TF32 = 2   /* tcgen05 tensor cores, TF32 inputs, FP32 accumulate (MIXED only) */
 };

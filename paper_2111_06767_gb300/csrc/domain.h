@@ -42,9 +42,10 @@ struct SchwarzLevel {
     DevBuf<int4> d;
     int n = 0, widths = 0;  // tiles, mask of their width codes
   } tiles_tc[2];
-  // FP64 domains on the tensor cores: digit slices of the scaled inverses [class][8][ld][ld] with their
-  // row and equilibration exponents [class][ld], tiles of 128 rows x 16..48 columns, K chunks of 64, and the slices of r_S
+  // FP64 domains on the tensor cores: digit slices of the scaled inverses [class][digit][ld][ld] with their
+  // row and equilibration exponents [class][ld], tiles of 128 rows x 16 or 32 columns, K chunks of 64, and the slices of r_S
   bool f64_tc = false;
+  int f64_digits = 0;
   DevBuf<uint16_t> inv_digits, x_digits;
   DevBuf<int> inv_row_exp, inv_hexp, x_exp;
   F64Maps f64_maps;

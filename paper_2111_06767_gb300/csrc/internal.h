@@ -265,22 +265,27 @@ int tc_tile_width(int code);
 // Splits the tensor-core GEMM accepts for this shape (each CTA keeps >= 4 K chunks).
 std::vector<int> tc_gemm_splits(int ld);
 
-// FP64 class GEMM on the tensor cores from digit slices (f64_gemm.cu): the digits of alpha times the
-// inverses [class][8][ld][ld] (BF16), their row exponents and equilibration exponents [class][ld]; the
-// digits [8][column][ld] and exponents of the columns of X.
-void launch_f64_inverse_digits(const double* inv, double alpha, int n_classes, int ld, int* hexp, uint16_t* dst,
-                               int* row_exp, cudaStream_t s);
-void launch_f64_column_digits(const double* X, int n_cols, int ld, const int* hexp, const int* class_of_col,
+// FP64 class GEMM on the tensor cores from digit slices (f64_gemm.cu). Equilibration exponents of the inverses
+// [class][ld] and the largest span of exponents in one row (range); the digits per value that hold such rows
+// exactly (12, 13 or 14; 0: none does).
+void launch_f64_equilibrate(const double* inv, double alpha, int n_classes, int ld, int* hexp, int* range,
+                            cudaStream_t s);
+int f64_digits_for(int range);
+// The digits of alpha times the inverses [class][digit][ld][ld] (BF16) and their row exponents [class][ld]; the digits
+// [digit][column][ld] and exponents of the columns of X.
+void launch_f64_inverse_digits(int digits, const double* inv, double alpha, int n_classes, int ld, const int* hexp,
+                               uint16_t* dst, int* row_exp, cudaStream_t s);
+void launch_f64_column_digits(int digits, const double* X, int n_cols, int ld, const int* hexp, const int* class_of_col,
                               uint16_t* dst, int* col_exp, cudaStream_t s);
 // Tensor maps of a level's digit buffers, encoded once with them: the inverses' (128 x 64 boxes of one
-// digit) and the columns' (16, 32 and 48 columns of every digit).
+// digit) and the columns' (16 and 32 columns of every digit).
 struct F64Maps {
-  CUtensorMap a, x[3];
+  CUtensorMap a, x[2];
 };
-void make_f64_maps(F64Maps& m, const uint16_t* inv, int n_classes, const uint16_t* X, int n_cols, int ld);
+void make_f64_maps(F64Maps& m, int digits, const uint16_t* inv, int n_classes, const uint16_t* X, int n_cols, int ld);
 // Tiles: 128 rows x 16 (width code + 1) columns; d_kchunks as above for chunks of 64, (ld + 63) / 64 + 1
 // ints per class; split as above.
-void launch_f64_gemm(const F64Maps& maps, const int* inv_exp, const int* x_exp, double* Y, int ld,
+void launch_f64_gemm(int digits, const F64Maps& maps, const int* inv_exp, const int* x_exp, double* Y, int ld,
                      const int4* d_tiles, int n_tiles, const int* d_kchunks, int* err, cudaStream_t s, int split = 0);
 
 // Launch-shape autotuning: the first time a kernel shape (key) is seen in the process, time each

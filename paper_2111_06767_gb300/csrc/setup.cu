@@ -251,10 +251,10 @@ void classify_schwarz(dg_domain* dom, Level& L) {
       }
   sw.n_tiles = (int)tiles.size();
   upload(sw.tiles, tiles, s);
-  // FP64 tensor-core tiles: a class's columns in equal parts of at most 48, rounded up to 16
+  // FP64 tensor-core tiles: a class's columns in equal parts of at most 32, rounded up to 16
   std::vector<int4> tiles_f64;
   for (int c = 0; c < (dom->curved || dom->mixed ? 0 : nc); ++c) {
-    const int parts = (sw.class_count[c] + 47) / 48, w = ((sw.class_count[c] + parts - 1) / parts + 15) / 16 * 16;
+    const int parts = (sw.class_count[c] + 31) / 32, w = ((sw.class_count[c] + parts - 1) / parts + 15) / 16 * 16;
     for (int r0 = 0; r0 < sw.ld; r0 += 128)
       for (int c0 = 0; c0 < sw.class_count[c]; c0 += w) tiles_f64.push_back(tile(c, r0, 128, c0, w / 16 - 1));
   }
@@ -730,27 +730,36 @@ void ensure_schwarz(dg_domain* dom, int level) {
     alloc_work(L.w32, L, s);
   } else {
     alloc_work(L.w64, L, s);
-    // Tensor cores except where one or two small subdomains leave the CUDA-core product shorter than
-    // the slicing and the longer kernel (three steps: 1 element at N = 4 61 against 76 us, 2 elements 70
-    // against 76, 1 element at N = 5 78 against 79; 1 at N = 6 83 against 83, at N = 8 126 against 107),
-    // or where the digits (twice the bytes of the inverses) would take more than 8 GiB.
-    sw.f64_tc = dom->desc.subdomain_gemm == DG_GEMM_DEFAULT && tc_gemm_available() && (int64_t)L.E * ld > 512 &&
-                (size_t)16 * nc * ld * ld <= ((size_t)8 << 30);
+    // Tensor cores except at N = 2 above one wave of tiles (columns of 32 values fill half a K chunk and a quarter of
+    // a tile's rows; three steps on 16^3 elements, 130 tiles, 148 us on the CUDA cores and 131 here, on 17 x 17 x 16 151
+    // and 173, on 64^3 3377 and 5464; every size tried from N = 3 on is faster here: 1 element at N = 3 68 and 42, 2
+    // elements at N = 4 75 and 51, 32^3 at N = 3 2334 and 1075, 8^3 at N = 8 4520 and 734), where the digits (24 to 28
+    // bytes an entry) would take more than 8 GiB, or where an inverse's rows span more than 14 digits hold (f64_gemm.cu).
+    sw.f64_tc = dom->desc.subdomain_gemm == DG_GEMM_DEFAULT && tc_gemm_available() && (ld > 32 || sw.n_tiles_f64 <= 152);
     if (sw.f64_tc) {
       try {
-        sw.inv_digits.alloc((size_t)8 * nc * ld * ld);
-        sw.inv_row_exp.alloc((size_t)nc * ld);
+        DevBuf<int> range(1);
         sw.inv_hexp.alloc((size_t)nc * ld);
-        sw.x_digits.alloc((size_t)8 * L.E * ld);
-        sw.x_exp.alloc(L.E);
+        launch_f64_equilibrate(sw.inv64.get(), sw.inv_scale, nc, ld, sw.inv_hexp.get(), range.get(), s);
+        int h_range = 0;
+        DG_CUDA(cudaMemcpyAsync(&h_range, range.get(), sizeof(int), cudaMemcpyDeviceToHost, s));
+        DG_CUDA(cudaStreamSynchronize(s));
+        const size_t S = sw.f64_digits = f64_digits_for(h_range);
+        sw.f64_tc = S > 0 && 2 * S * nc * ld * ld <= ((size_t)8 << 30);
+        if (sw.f64_tc) {
+          sw.inv_digits.alloc(S * nc * ld * ld);
+          sw.inv_row_exp.alloc((size_t)nc * ld);
+          sw.x_digits.alloc(S * L.E * ld);
+          sw.x_exp.alloc(L.E);
+        }
       } catch (const Error& err) {
         if (err.status != DG_ERR_OOM) throw;
         sw.f64_tc = false;  // what fits without the digits still runs, on the CUDA cores
       }
       if (sw.f64_tc) {
-        launch_f64_inverse_digits(sw.inv64.get(), sw.inv_scale, nc, ld, sw.inv_hexp.get(), sw.inv_digits.get(),
-                                  sw.inv_row_exp.get(), s);
-        make_f64_maps(sw.f64_maps, sw.inv_digits.get(), nc, sw.x_digits.get(), L.E, ld);
+        launch_f64_inverse_digits(sw.f64_digits, sw.inv64.get(), sw.inv_scale, nc, ld, sw.inv_hexp.get(),
+                                  sw.inv_digits.get(), sw.inv_row_exp.get(), s);
+        make_f64_maps(sw.f64_maps, sw.f64_digits, sw.inv_digits.get(), nc, sw.x_digits.get(), L.E, ld);
         DG_CUDA(cudaStreamSynchronize(s));
         sw.inv64.release();
       } else {

@@ -235,17 +235,17 @@ void class_gemm<double>(dg_domain* dom, Level& L, const double* X, double* Y, cu
     return;
   }
   if (sw.f64_tc) {
-    launch_f64_column_digits(X, L.E, sw.ld, sw.inv_hexp.get(), sw.class_of_col.get(), sw.x_digits.get(),
+    launch_f64_column_digits(sw.f64_digits, X, L.E, sw.ld, sw.inv_hexp.get(), sw.class_of_col.get(), sw.x_digits.get(),
                              sw.x_exp.get(), s);
     auto run = [&](int split) {
-      launch_f64_gemm(sw.f64_maps, sw.inv_row_exp.get(), sw.x_exp.get(), Y, sw.ld, sw.tiles_f64.get(),
+      launch_f64_gemm(sw.f64_digits, sw.f64_maps, sw.inv_row_exp.get(), sw.x_exp.get(), Y, sw.ld, sw.tiles_f64.get(),
                       sw.n_tiles_f64, sw.kchunks64.get(), dom->err_flag.get(), s, split);
     };
     if (L.f64_split < 0) {  // the K split, tuned per level on first use
       std::vector<int> cand{0, 1};
       for (int sp = 2; sp <= 8; sp *= 2)
         if ((sw.ld + 63) / 64 >= sp) cand.push_back(sp);
-      const int pick = autotune({5, sw.n_classes, sw.ld, sw.n_tiles_f64, L.E}, cand, run, s);
+      const int pick = autotune({5, sw.f64_digits, sw.n_classes, sw.ld, sw.n_tiles_f64, L.E}, cand, run, s);
       cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
       DG_CUDA(cudaStreamIsCapturing(s, &cap));
       if (cap != cudaStreamCaptureStatusNone) {
