@@ -4,6 +4,7 @@
 // timed ones, and the fastest is kept; it replaces hand-picked launch heuristics and has no
 // counterpart in the paper), the stream of this thread's allocations, and the switch for
 // programmatic dependent launch.
+#include <algorithm>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
@@ -12,6 +13,7 @@
 #include <mutex>
 #include <set>
 #include <string>
+#include <utility>
 
 #include "internal.h"
 
@@ -37,6 +39,18 @@ bool tune_log() {
     return v && std::strcmp(v, "1") == 0;
   }();
   return on;
+}
+
+int pinned_shape(const char* name, const std::vector<int>& offered) {
+  const char* e = std::getenv(name);
+  if (!e) return -1;
+  const int v = std::atoi(e);
+  if (std::find(offered.begin(), offered.end(), v) != offered.end()) return v;
+  static std::mutex mu;
+  static std::set<std::pair<std::string, int>> told;
+  std::lock_guard<std::mutex> lk(mu);
+  if (told.emplace(name, v).second) std::fprintf(stderr, "dg %s=%d: no such launch shape here, tuned instead\n", name, v);
+  return -1;
 }
 
 cudaStream_t alloc_stream() { return tl_alloc_stream; }

@@ -293,6 +293,9 @@ void launch_f64_gemm(int digits, const F64Maps& maps, const int* inv_exp, const 
 // kept choice. candidates[0] is the heuristic default, used alone when DG_AUTOTUNE=0 or while s is
 // being captured into a graph.
 bool tune_log();  // DG_TUNE_LOG=1
+// The launch shape that the environment variable `name` pins, -1 where it is not set. A value that is not among `offered`
+// is reported on stderr (once per variable and value) and not pinned.
+int pinned_shape(const char* name, const std::vector<int>& offered);
 int autotune(const std::vector<int64_t>& key, const std::vector<int>& candidates,
              const std::function<void(int)>& run, cudaStream_t s);
 

@@ -191,7 +191,7 @@ void launch_class_gemm_tiles(const T* inv, const T* X, T* Y, int ld, const int4*
 
 namespace {
 // The CUDA-core class GEMM with its K split tuned per level and precision on first use (0, the
-// heuristic, then 1, 2, 4, 8); DG_GEMM_SPLIT pins it as for the tensor-core GEMM.
+// heuristic, then 1, 2, 4, 8); DG_GEMM_SPLIT pins it as for the tensor-core GEMMs.
 template <typename T>
 void simt_class_gemm(Level& L, const T* inv, const T* X, T* Y, T alpha, cudaStream_t s) {
   const SchwarzLevel& sw = L.sw;
@@ -204,9 +204,8 @@ void simt_class_gemm(Level& L, const T* inv, const T* X, T* Y, T alpha, cudaStre
     const int nk = (sw.ld + 15) / 16;
     for (int sp = 1; sp <= 8; sp *= 2)
       if (nk / sp >= 4) cand.push_back(sp);
-    const char* e = std::getenv("DG_GEMM_SPLIT");
-    const int forced = e ? std::atoi(e) : -1;
-    if (forced >= 0 && std::find(cand.begin(), cand.end(), forced) != cand.end()) {
+    const int forced = pinned_shape("DG_GEMM_SPLIT", cand);
+    if (forced >= 0) {
       pick = forced;
     } else {
       const int p = autotune({4, (int64_t)sizeof(T), sw.n_classes, sw.ld, sw.n_tiles, L.E}, cand, run, s);
@@ -245,6 +244,12 @@ void class_gemm<double>(dg_domain* dom, Level& L, const double* X, double* Y, cu
       std::vector<int> cand{0, 1};
       for (int sp = 2; sp <= 8; sp *= 2)
         if ((sw.ld + 63) / 64 >= sp) cand.push_back(sp);
+      const int forced = pinned_shape("DG_GEMM_SPLIT", cand);
+      if (forced >= 0) {
+        L.f64_split = forced;
+        run(forced);
+        return;
+      }
       const int pick = autotune({5, sw.f64_digits, sw.n_classes, sw.ld, sw.n_tiles_f64, L.E}, cand, run, s);
       cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
       DG_CUDA(cudaStreamIsCapturing(s, &cap));
@@ -288,9 +293,11 @@ void class_gemm<float>(dg_domain* dom, Level& L, const float* X, float* Y, cudaS
       }
       // DG_GEMM_SPLIT=k pins one candidate (tests and measurements of each launch shape); read
       // when a level first runs its GEMM, so a process can set it per domain
-      const char* e = std::getenv("DG_GEMM_SPLIT");
-      const int forced = e ? std::atoi(e) : -1;
-      if (forced >= 0 && std::find(cand.begin(), cand.end(), forced) != cand.end()) {
+      std::vector<int> offered = cand;
+      if (sw.tiles_tc[0].n == sw.tiles_tc[1].n)  // the wide list can be pinned where it is the same
+        for (int c : cand) offered.push_back(kWide | c);
+      const int forced = pinned_shape("DG_GEMM_SPLIT", offered);
+      if (forced >= 0) {
         L.gemm_split = forced;
         run(forced);
         return;
