@@ -36,12 +36,11 @@ int apply_variant(dg_domain* dom, Level& L, bool fused, const std::function<void
     for (int v : {2, 3})
       if (apply_bricks(dom->N, v, L.E) >= 76) cand.push_back(v);
     if (!fused && dom->N == 4 && sizeof(T) == 4) cand.push_back(7);
-    // DG_APPLY_VARIANT=v pins one candidate (tests of each launch shape)
-    static const int forced = [] {
-      const char* e = std::getenv("DG_APPLY_VARIANT");
-      return e ? std::atoi(e) : -1;
-    }();
-    if (forced >= 0 && std::find(cand.begin(), cand.end(), forced) != cand.end()) {
+    // DG_APPLY_VARIANT=v pins one shape (tests of each); every shape runs every grid
+    std::vector<int> offered{0, 1, 2, 3, 4};
+    if (cand.back() == 7) offered.push_back(7);
+    const int forced = pinned_shape("DG_APPLY_VARIANT", offered);
+    if (forced >= 0) {
       v = forced;
       return v;
     }

@@ -52,3 +52,24 @@ def test_a_pinned_gemm_split_is_not_tuned(tmp_path, split):
     assert "dg autotune key 1 " in log  # the applies are tuned
     for key in (3, 4, 5):  # the tensor-core products and the CUDA-core one are not
         assert f"dg autotune key {key} " not in log
+
+
+_APPLY = """
+for N in (4, 7):
+    d = dgg.Domain(n=(3, 2, 2), N=N, mg_levels=1, overlap=2)
+    u = torch.ones(d.n_dof, dtype=torch.float64, device="cuda")
+    d.apply(u)
+    d.apply_f32(u.float())
+    d.schwarz_smooth(0, u, u.clone(), 1)
+"""
+
+
+@pytest.mark.parametrize("variant", ["0", "1", "2", "3", "4"])
+def test_a_pinned_apply_shape_is_not_tuned(tmp_path, variant):
+    """Also where the grid is too small for the tuner to be offered the shape."""
+    assert "dg autotune key 1 " not in _log_of(_APPLY, tmp_path, DG_APPLY_VARIANT=variant)
+
+
+def test_a_shape_that_does_not_exist_is_reported_and_tuned(tmp_path):
+    log = _log_of(_APPLY, tmp_path, DG_APPLY_VARIANT="5")
+    assert log.count("dg DG_APPLY_VARIANT=5: no such launch shape here") == 1 and "dg autotune key 1 " in log
