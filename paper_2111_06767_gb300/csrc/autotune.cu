@@ -5,6 +5,7 @@
 // counterpart in the paper), the stream of this thread's allocations, and the switch for
 // programmatic dependent launch.
 #include <algorithm>
+#include <atomic>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
@@ -54,6 +55,15 @@ int pinned_shape(const char* name, const std::vector<int>& offered) {
 }
 
 cudaStream_t alloc_stream() { return tl_alloc_stream; }
+
+namespace {
+std::atomic<int64_t> g_bytes{0};
+}
+void count_bytes(int64_t change) { g_bytes += change; }
+bool within_alloc_limit(size_t more) {
+  const char* e = std::getenv("DG_ALLOC_LIMIT");
+  return !e || g_bytes + (int64_t)more <= std::atoll(e);
+}
 
 void keep_pool_memory() {
   static std::mutex mu;

@@ -368,11 +368,10 @@ dg_status elliptic_solve_host(dg_domain* dom, const double* f_host, double* u_ho
     DG_REQUIRE(u_host != nullptr, "u_host must be a host pointer");
     DG_REQUIRE(f_host != nullptr || dom->desc.problem == DG_PROBLEM_PUNCTURE, "f_host must be a host pointer");
     const int64_t n = dom->levels[0].ndof;
-    if (!dom->host_f.get()) {
-      dom->host_f.alloc(n);
-      dom->host_b.alloc(n);
-      dom->host_u.alloc(n);
-    }
+    dg::with_room(dom, [&] {
+      for (dg::DevBuf<double>* v : {&dom->host_f, &dom->host_b, &dom->host_u})
+        if (!v->get()) v->alloc(n);
+    });
     cudaStream_t s = dom->stream;
     DG_CUDA(cudaMemcpyAsync(dom->host_u.get(), u_host, sizeof(double) * n, cudaMemcpyHostToDevice, s));
     if (f_host) {

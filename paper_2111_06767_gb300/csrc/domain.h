@@ -10,6 +10,21 @@
 
 namespace dg {
 
+// Device bytes taken for digit slices. All of a process together take at most an eighth of the device's memory, so that
+// the problems that fit without them still fit beside them; take() says whether there is room.
+struct DigitBytes {
+  size_t n = 0;
+  DigitBytes() = default;
+  DigitBytes(DigitBytes&& o) noexcept : n(o.n) { o.n = 0; }
+  DigitBytes& operator=(DigitBytes&& o) noexcept {
+    if (this != &o) { give(); n = o.n; o.n = 0; }
+    return *this;
+  }
+  ~DigitBytes() { give(); }
+  bool take(size_t bytes);
+  void give();
+};
+
 struct SchwarzLevel {
   int nS = 0;                      // padded subdomain size N^3 + 6 N_ov N^2
   int ld = 0;                      // storage stride: nS rounded up to 32
@@ -46,6 +61,7 @@ struct SchwarzLevel {
   // row and equilibration exponents [class][ld], tiles of 128 rows x 16 or 32 columns, K chunks of 64, and the slices of r_S
   bool f64_tc = false;
   int f64_digits = 0;
+  DigitBytes digit_bytes;          // their share of what all digits of the process may take
   DevBuf<uint16_t> inv_digits, x_digits;
   DevBuf<int> inv_row_exp, inv_hexp, x_exp;
   F64Maps f64_maps;
@@ -158,6 +174,8 @@ struct dg_domain {
   const std::atomic<bool>* cancel = nullptr;  // set by a serving worker: stop between Krylov iterations
   bool linv_current = false; // per-subdomain inverses built for the current linearization
   bool use_tc = false;       // subdomain GEMM on tcgen05 tensor cores (MIXED)
+  bool no_digits = false;    // FP64 products on the CUDA cores: the digit slices' memory was needed (see drop_digits)
+  bool in_batch = false;     // a batch's graph holds this domain's buffers
   bool coarse_fused = false; // fused cooperative smoother on coarse levels (DG_COARSE_FUSED=1 turns it on)
   int barrier_stall = 0;     // DG_TEST_BARRIER_STALL=1 (read when a solve starts): the fused smoother's
                              // barriers wait for one CTA more than launched, so every wait runs out
@@ -209,6 +227,19 @@ void batch_destroy(dg_batch* bt);
 void profile_read(dg_domain* dom, dg_phase_stats* out);
 void ensure_schwarz(dg_domain* dom, int level);
 size_t domain_device_bytes(const dg_domain* dom);
+// Gives the memory of an FP64 domain's digit slices back: its levels take their inverses as FP64 values and the CUDA-core
+// product from here on. False where there is nothing to give, or a batch's graph holds the slices.
+bool drop_digits(dg_domain* dom);
+// f(), which allocates for dom; once more without the digit slices if the memory does not suffice. f may run twice.
+template <typename F>
+void with_room(dg_domain* dom, F f) {
+  try {
+    f();
+  } catch (const Error& e) {
+    if (e.status != DG_ERR_OOM || !drop_digits(dom)) throw;
+    f();
+  }
+}
 
 // level operators
 void apply_level(dg_domain* dom, int level, const double* u, double* out, const double* b, bool with_lin,

@@ -82,6 +82,11 @@ struct AllocStreamScope {
 // Keep freed memory in this process's default pool of the current device (once per device).
 void keep_pool_memory();
 
+// Device bytes held in buffers of this process, and whether DG_ALLOC_LIMIT (bytes, read at every allocation; unset: no
+// limit) leaves room for more.
+void count_bytes(int64_t change);
+bool within_alloc_limit(size_t more);
+
 // Owning device buffer, move-only. alloc() returns once the memory is usable from any stream
 // (it synchronises the allocation stream); release() is ordered after that stream's work, and
 // the owner makes sure other streams are done with the buffer before (the domain joins its
@@ -103,7 +108,10 @@ struct DevBuf {
   ~DevBuf() { release(); }
   void alloc(size_t n);
   void release() {
-    if (ptr) cudaFreeAsync(ptr, st);
+    if (ptr) {
+      cudaFreeAsync(ptr, st);
+      count_bytes(-(int64_t)bytes());
+    }
     ptr = nullptr;
     count = 0;
   }
@@ -116,7 +124,8 @@ void DevBuf<T>::alloc(size_t n) {
   release();
   if (n == 0) return;
   st = alloc_stream();
-  cudaError_t e = cudaMallocAsync(&ptr, n * sizeof(T), st);
+  cudaError_t e = within_alloc_limit(n * sizeof(T)) ? cudaMallocAsync(&ptr, n * sizeof(T), st)
+                                                    : cudaErrorMemoryAllocation;
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   if (e != cudaSuccess) {
     if (ptr) cudaFreeAsync(ptr, st);
@@ -125,6 +134,7 @@ void DevBuf<T>::alloc(size_t n) {
     fail(DG_ERR_OOM, "allocation of " + std::to_string(n * sizeof(T)) + " bytes failed: " + cudaGetErrorString(e));
   }
   count = n;
+  count_bytes((int64_t)bytes());
 }
 
 // ------------------------------------------------------------------ LGL tables (host)

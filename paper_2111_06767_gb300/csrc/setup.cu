@@ -611,40 +611,38 @@ void build_curved_inverses(dg_domain* dom, Level& L, DevBuf<T>& inv, const T* ge
 }
 }  // namespace
 
-// Explicit inverses and work vectors of one level, built on first use (Sec. III.E: construction
-// cost amortised over all later solves).
-void ensure_schwarz(dg_domain* dom, int level) {
-  Level& L = dom->levels[level];
+namespace {
+std::mutex g_digit_mu;
+size_t g_digit_bytes = 0;
+
+void release_digits(SchwarzLevel& sw) {
+  sw.f64_tc = false;
+  for (auto* p : {&sw.inv_digits, &sw.x_digits}) p->release();
+  for (auto* p : {&sw.inv_row_exp, &sw.inv_hexp, &sw.x_exp}) p->release();
+  sw.digit_bytes.give();
+}
+}  // namespace
+
+bool DigitBytes::take(size_t bytes) {
+  give();
+  size_t free_b = 0, total = 0;
+  DG_CUDA(cudaMemGetInfo(&free_b, &total));
+  std::lock_guard<std::mutex> lk(g_digit_mu);
+  if (g_digit_bytes + bytes > total / 8) return false;
+  g_digit_bytes += bytes;
+  n = bytes;
+  return true;
+}
+void DigitBytes::give() {
+  std::lock_guard<std::mutex> lk(g_digit_mu);
+  g_digit_bytes -= n;
+  n = 0;
+}
+
+namespace {
+// The explicit inverses of a level's classes, from the store or built.
+void build_class_inverses(dg_domain* dom, Level& L) {
   SchwarzLevel& sw = L.sw;
-  if (sw.built) return;
-  sw.rec.alloc((size_t)7 * L.E);
-  launch_subdomain_records(sw.geom, sw.col_of_elem.get(), sw.xform_of_elem.get(), dom->orient_aff.get(), sw.rec.get(),
-                           dom->stream);
-  if (dom->curved) {
-    cudaStream_t s = dom->stream;
-    sw.inv_scale = 1.0;
-    if (dom->mixed) {
-      build_curved_inverses<float>(dom, L, sw.inv32, L.geo32.get(), L.face32.get(), dom->D32.get(), dom->w32.get(), s);
-      if (dom->desc.subdomain_gemm != DG_GEMM_SIMT) {
-        // the smoother streams every inverse once per step: keep them in FP16 (scaled per subdomain),
-        // the input precision of the tensor-core path; "simt" keeps FP32
-        sw.inv16.alloc((size_t)L.E * sw.nS * sw.nS);
-        sw.inv16_scale.alloc(L.E);
-        launch_to_half_scaled(sw.inv32.get(), sw.nS, L.E, sw.inv16.get(), sw.inv16_scale.get(), s);
-        DG_CUDA(cudaStreamSynchronize(s));
-        sw.inv32.release();
-      }
-      alloc_work(L.w32, L, s);
-    } else {
-      build_curved_inverses<double>(dom, L, sw.inv64, L.geo64.get(), L.face64.get(), dom->D64.get(), dom->w64.get(),
-                                    s);
-      alloc_work(L.w64, L, s);
-    }
-    DG_CUDA(cudaStreamSynchronize(s));
-    sw.built = true;
-    dom->bytes = domain_device_bytes(dom);
-    return;
-  }
   const int N = dom->N, ov = dom->desc.overlap, nS = sw.nS, nc = sw.n_classes;
   cudaStream_t s = dom->stream;
   DG_CUDA(cudaStreamSynchronize(s));
@@ -726,6 +724,43 @@ void ensure_schwarz(dg_domain* dom, int level) {
     }
     DG_CUDA(cudaStreamSynchronize(s));
   }
+}
+}  // namespace
+
+namespace {
+void build_schwarz(dg_domain* dom, Level& L) {
+  SchwarzLevel& sw = L.sw;
+  sw.rec.alloc((size_t)7 * L.E);
+  launch_subdomain_records(sw.geom, sw.col_of_elem.get(), sw.xform_of_elem.get(), dom->orient_aff.get(), sw.rec.get(),
+                           dom->stream);
+  if (dom->curved) {
+    cudaStream_t s = dom->stream;
+    sw.inv_scale = 1.0;
+    if (dom->mixed) {
+      build_curved_inverses<float>(dom, L, sw.inv32, L.geo32.get(), L.face32.get(), dom->D32.get(), dom->w32.get(), s);
+      if (dom->desc.subdomain_gemm != DG_GEMM_SIMT) {
+        // the smoother streams every inverse once per step: keep them in FP16 (scaled per subdomain),
+        // the input precision of the tensor-core path; "simt" keeps FP32
+        sw.inv16.alloc((size_t)L.E * sw.nS * sw.nS);
+        sw.inv16_scale.alloc(L.E);
+        launch_to_half_scaled(sw.inv32.get(), sw.nS, L.E, sw.inv16.get(), sw.inv16_scale.get(), s);
+        DG_CUDA(cudaStreamSynchronize(s));
+        sw.inv32.release();
+      }
+      alloc_work(L.w32, L, s);
+    } else {
+      build_curved_inverses<double>(dom, L, sw.inv64, L.geo64.get(), L.face64.get(), dom->D64.get(), dom->w64.get(),
+                                    s);
+      alloc_work(L.w64, L, s);
+    }
+    DG_CUDA(cudaStreamSynchronize(s));
+    sw.built = true;
+    dom->bytes = domain_device_bytes(dom);
+    return;
+  }
+  cudaStream_t s = dom->stream;
+  build_class_inverses(dom, L);
+  const int nc = sw.n_classes, ld = sw.ld;
   if (dom->mixed) {
     alloc_work(L.w32, L, s);
   } else {
@@ -734,8 +769,10 @@ void ensure_schwarz(dg_domain* dom, int level) {
     // a tile's rows; three steps on 16^3 elements, 130 tiles, 148 us on the CUDA cores and 131 here, on 17 x 17 x 16 151
     // and 173, on 64^3 3377 and 5464; every size tried from N = 3 on is faster here: 1 element at N = 3 68 and 42, 2
     // elements at N = 4 75 and 51, 32^3 at N = 3 2334 and 1075, 8^3 at N = 8 4520 and 734), where the digits (24 to 28
-    // bytes an entry) would take more than 8 GiB, or where an inverse's rows span more than 14 digits hold (f64_gemm.cu).
-    sw.f64_tc = dom->desc.subdomain_gemm == DG_GEMM_DEFAULT && tc_gemm_available() && (ld > 32 || sw.n_tiles_f64 <= 152);
+    // bytes an entry of an inverse and a row of r_S) have no room, or where an inverse's rows span more than 14 digits
+    // hold (f64_gemm.cu).
+    sw.f64_tc = dom->desc.subdomain_gemm == DG_GEMM_DEFAULT && !dom->no_digits && tc_gemm_available() &&
+                (ld > 32 || sw.n_tiles_f64 <= 152);
     if (sw.f64_tc) {
       try {
         DevBuf<int> range(1);
@@ -745,7 +782,7 @@ void ensure_schwarz(dg_domain* dom, int level) {
         DG_CUDA(cudaMemcpyAsync(&h_range, range.get(), sizeof(int), cudaMemcpyDeviceToHost, s));
         DG_CUDA(cudaStreamSynchronize(s));
         const size_t S = sw.f64_digits = f64_digits_for(h_range);
-        sw.f64_tc = S > 0 && 2 * S * nc * ld * ld <= ((size_t)8 << 30);
+        sw.f64_tc = S > 0 && sw.digit_bytes.take(2 * S * ((size_t)nc * ld * ld + (size_t)L.E * ld));
         if (sw.f64_tc) {
           sw.inv_digits.alloc(S * nc * ld * ld);
           sw.inv_row_exp.alloc((size_t)nc * ld);
@@ -763,14 +800,45 @@ void ensure_schwarz(dg_domain* dom, int level) {
         DG_CUDA(cudaStreamSynchronize(s));
         sw.inv64.release();
       } else {
-        for (auto* p : {&sw.inv_digits, &sw.x_digits}) p->release();
-        for (auto* p : {&sw.inv_row_exp, &sw.inv_hexp, &sw.x_exp}) p->release();
+        release_digits(sw);
       }
     }
   }
   DG_CUDA(cudaStreamSynchronize(s));
   sw.built = true;
   dom->bytes = domain_device_bytes(dom);
+}
+}  // namespace
+
+// Explicit inverses and work vectors of one level, built on first use (Sec. III.E: construction
+// cost amortised over all later solves).
+void ensure_schwarz(dg_domain* dom, int level) {
+  Level& L = dom->levels[level];
+  if (!L.sw.built) with_room(dom, [&] { build_schwarz(dom, L); });
+}
+
+bool drop_digits(dg_domain* dom) {
+  bool any = false;
+  for (Level& L : dom->levels) any = any || (L.sw.built && L.sw.f64_tc);
+  if (!any || dom->in_batch) return false;
+  DG_CUDA(cudaDeviceSynchronize());  // the slices may be in use on a stream of the caller's
+  for (cudaGraphExec_t* g : {&dom->vgraph, &dom->sgraph}) {  // captured graphs hold the digit product
+    if (*g) cudaGraphExecDestroy(*g);
+    *g = nullptr;
+  }
+  dom->prof.drop_graph_records();
+  dom->vcycle_calls = 0;
+  dom->skey_seen.clear();
+  dom->no_digits = true;
+  for (Level& L : dom->levels) release_digits(L.sw);
+  for (Level& L : dom->levels) {
+    if (!L.sw.built || L.sw.inv64.get()) continue;
+    L.sw.built = false;  // until the inverses are back
+    build_class_inverses(dom, L);
+    L.sw.built = true;
+  }
+  dom->bytes = domain_device_bytes(dom);
+  return true;
 }
 
 size_t domain_device_bytes(const dg_domain* dom) {

@@ -332,7 +332,7 @@ void gather_linearization(dg_domain* dom, cudaStream_t s) {
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   DG_CUDA(cudaStreamIsCapturing(s, &cap));
   if (W.gD.count < (size_t)L.E * L.sw.ld) {
-    W.gD.alloc((size_t)L.E * L.sw.ld);
+    with_room(dom, [&] { W.gD.alloc((size_t)L.E * L.sw.ld); });
     DG_CUDA(cudaMemsetAsync(W.gD.get(), 0, W.gD.bytes(), s));  // rows that no point maps to
   }
   launch_gather<T>(L.sw.geom, lin_diag<T>(dom), L.sw.rec.get(), W.gD.get(), s);
@@ -435,11 +435,12 @@ void schwarz_smooth(dg_domain* dom, int level, const T* b, T* u, int iterations,
     } else {
       // GMRES on (A_S + D_S), right-preconditioned by the Poisson inverse A_S^-1 (Sec. III.E)
       const size_t blk = (size_t)L.E * ld;
-      if (W.gV.count < (size_t)m * blk) {
-        W.gV.alloc(m * blk);
-        W.gZ.alloc(m * blk);
-        W.gH.alloc((size_t)L.E * ((m + 1) * m + 1 + m));
-      }
+      if (W.gV.count < (size_t)m * blk || !W.gZ.get() || !W.gH.get())
+        with_room(dom, [&] {
+          W.gV.alloc(m * blk);
+          W.gZ.alloc(m * blk);
+          W.gH.alloc((size_t)L.E * ((m + 1) * m + 1 + m));
+        });
       gather_linearization<T>(dom, s);
       beta = W.gH.get() + (size_t)L.E * (m + 1) * m;
       y = beta + L.E;
@@ -602,10 +603,10 @@ void precondition(dg_domain* dom, int mode, const double* v, double* z, cudaStre
       DG_CUDA(cudaMemsetAsync(z, 0, sizeof(double) * n, s));
       schwarz_smooth<double>(dom, 0, v, z, steps, true, s);
     } else {
-      if (!dom->vin64.get()) {
-        dom->vin64.alloc(n);
-        dom->vout64.alloc(n);
-      }
+      with_room(dom, [&] {
+        for (DevBuf<double>* v : {&dom->vin64, &dom->vout64})
+          if (!v->get()) v->alloc(n);
+      });
       DG_CUDA(cudaMemcpyAsync(dom->vin64.get(), v, sizeof(double) * n, cudaMemcpyDeviceToDevice, s));
       vcycle_fixed(dom, s);
       DG_CUDA(cudaMemcpyAsync(z, dom->vout64.get(), sizeof(double) * n, cudaMemcpyDeviceToDevice, s));
@@ -634,16 +635,11 @@ double now_s() {
 
 // Krylov workspace for k iterations: V (k + 1 vectors) and Z (k vectors), grown on demand
 // (doubling, contents kept) so that short solves do not hold a basis sized for the iteration cap.
-void ensure_workspace(dg_domain* dom, int k) {
+void ensure_workspace(dg_domain* dom, int k);
+void grow_workspace(dg_domain* dom, int k) {
   const int64_t n = dom->levels[0].ndof;
-  if (!dom->w.get()) {
-    dom->w.alloc(n);
-    dom->r.alloc(n);
-    dom->du.alloc(n);
-    dom->ut.alloc(n);
-    dom->rt.alloc(n);
-    dom->tmp.alloc(n);
-  }
+  for (DevBuf<double>* v : {&dom->w, &dom->r, &dom->du, &dom->ut, &dom->rt, &dom->tmp})
+    if (!v->get()) v->alloc(n);
   if (dom->kcap >= k) return;
   const int cap = std::max(k, std::min(2 * std::max(dom->kcap, 8), 400));
   DevBuf<double> V((size_t)(cap + 1) * n), Z((size_t)cap * n);
@@ -652,11 +648,15 @@ void ensure_workspace(dg_domain* dom, int k) {
     DG_CUDA(cudaMemcpyAsync(Z.get(), dom->Zb.get(), dom->Zb.bytes(), cudaMemcpyDeviceToDevice, dom->stream));
     DG_CUDA(cudaStreamSynchronize(dom->stream));
   }
+  DevBuf<double> partial((size_t)multidot_partial_blocks() * (cap + 2)), dots(3 * (size_t)(cap + 2));
   dom->V = std::move(V);
   dom->Zb = std::move(Z);
-  dom->partial.alloc((size_t)multidot_partial_blocks() * (cap + 2));
-  dom->dots.alloc(3 * (size_t)(cap + 2));
+  dom->partial = std::move(partial);
+  dom->dots = std::move(dots);
   dom->kcap = cap;
+}
+void ensure_workspace(dg_domain* dom, int k) {
+  with_room(dom, [&] { grow_workspace(dom, k); });
 }
 
 double norm2(dg_domain* dom, const double* x, cudaStream_t s) {
@@ -833,17 +833,16 @@ void prepare_solve_graph(dg_domain* dom, int cap) {
     dom->kbuf.alloc(KrylovLayout::size(cap) + 8);  // + the 8-double report
     dom->kr_cap = cap;
   }
-  if (!dom->kb.get()) {
-    dom->kb.alloc(n);
-    dom->kx.alloc(n);
-    dom->zfix.alloc(n);
-  }
-  if (dom->mixed) {
-    if (!dom->vin32.get()) dom->vin32.alloc(2 * n);
-  } else if (!dom->vin64.get()) {
-    dom->vin64.alloc(n);
-    dom->vout64.alloc(n);
-  }
+  with_room(dom, [&] {
+    for (DevBuf<double>* v : {&dom->kb, &dom->kx, &dom->zfix})
+      if (!v->get()) v->alloc(n);
+    if (dom->mixed) {
+      if (!dom->vin32.get()) dom->vin32.alloc(2 * n);
+    } else {
+      for (DevBuf<double>* v : {&dom->vin64, &dom->vout64})
+        if (!v->get()) v->alloc(n);
+    }
+  });
 }
 
 // Run every kernel shape a captured solve uses once, uncaptured, so that launch shapes are tuned
@@ -1107,6 +1106,7 @@ dg_batch* batch_create(dg_domain* const* doms, const double* const* b, double* c
     prepare_solve_graph(dom, bt->cap);
     warm_solve_kernels(dom);
   }
+  for (int i = 0; i < count; ++i) doms[i]->in_batch = true;
   cudaGraph_t graph = nullptr;
   DG_CUDA(cudaGraphCreate(&graph, 0));
   try {
@@ -1247,11 +1247,11 @@ void build_linearized_inverses(dg_domain* dom, cudaStream_t s) {
     DevBuf<int> d_patch(sw.patch.size());
     DG_CUDA(cudaMemcpyAsync(d_patch.get(), sw.patch.data(), sizeof(int) * sw.patch.size(), cudaMemcpyHostToDevice, s));
     const OpGeom<T> g = make_geom<T>(L.n, L.h, N, dom->desc.penalty, dom->lgl);
-    W.linA.alloc((size_t)nc * n2);
+    with_room(dom, [&] { W.linA.alloc((size_t)nc * n2); });
     launch_build_subdomain_matrices<T>(N, dom->desc.overlap, g, Dt, wt, d_patch.get(), nc, nS, W.linA.get(), s);
     DG_CUDA(cudaStreamSynchronize(s));
   }
-  if (W.linv.count < (size_t)E * n2) W.linv.alloc((size_t)E * n2);
+  if (W.linv.count < (size_t)E * n2) with_room(dom, [&] { W.linv.alloc((size_t)E * n2); });
   const double sz = sizeof(T);
   PhaseScope ps(dom->prof, DG_PHASE_SUBDOMAIN_BUILD, s, 3.0 * E * n2 * sz, 2.0 * E * (double)n2 * nS);
   gather_linearization<T>(dom, s);
