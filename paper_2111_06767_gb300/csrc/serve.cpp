@@ -48,14 +48,16 @@ struct Job {
 
 namespace dg {
 
-// Upper bound of a domain's device footprint (bytes) before it is built.
-size_t estimate_domain_bytes(const dg_domain_desc& d, int max_iterations, bool linearized_inverses) {
+// Upper bound of a domain's device footprint (bytes) before it is built, for solves of up to 64 Krylov iterations.
+// FP64 domains hold their inverses as values, not as digit slices (elliptic_serve_submit sees to that).
+size_t estimate_domain_bytes(const dg_domain_desc& d, int max_iterations, bool linearized_inverses,
+                             int subdomain_iterations) {
   const int N = d.N, ov = d.overlap;
   const size_t nS = (size_t)N * N * N + 6 * (size_t)ov * N * N;
   const size_t ld = (nS + 31) / 32 * 32;
   const bool mixed = d.precision == DG_PRECISION_MIXED;
   const size_t fb = mixed ? 4 : 8;
-  size_t total = (size_t)48 * (nS + 7 * N * N * N) * 4 + (size_t)64 * N * N * N * 7 * fb;  // subdomain records, shares
+  size_t total = (size_t)48 * 7 * 16 + (size_t)64 * N * N * N * 7 * fb;  // orientations, weight shares
   int n[3] = {d.n[0], d.n[1], d.n[2]};
   size_t build_peak = 0;
   for (int l = 0; l < DG_MAX_LEVELS; ++l) {
@@ -77,15 +79,24 @@ size_t estimate_domain_bytes(const dg_domain_desc& d, int max_iterations, bool l
     classes = std::min(classes, E);
     if (d.node_xyz || d.coef) {
       // every subdomain has its own inverse, compact; MIXED keeps FP16 copies (FP32 with "simt"),
-      // built in the smoother's precision; plus the nodal metric, face-node penalty and traces
+      // built in the smoother's precision; plus, in both precisions, the metric and coefficient (11 values a
+      // point), the gradient (3), the face sizes (3 a face node) and the traces (1)
       const size_t store = mixed ? (d.subdomain_gemm == DG_GEMM_SIMT ? 4 : 2) : 8;
       build_peak = std::max(build_peak, E * nS * nS * (mixed ? 4 : 8));
-      total += E * nS * nS * store + ndof * (11 * 12 + 8) + E * 6 * N * N * 24;
+      total += E * nS * nS * store + ndof * (11 + 3) * 12 + E * 6 * N * N * (3 + 1) * 12;
     } else {
       build_peak = std::max(build_peak, classes * nS * nS * 8);  // FP64 build, freed after inversion
       total += classes * ld * ld * fb;                            // stored inverses
+      // tile lists (64, and three of 128 rows; columns by 16 at least) and units, and the K chunks of every class
+      total += 16 * ((ld / 64 + 1) * (E / 16 + classes) + 3 * (ld / 128 + 1) * (E / 16 + classes) + (ld / 16) * classes) +
+               4 * classes * (ld / 16 + ld / 32 + ld / 64 + 4);
     }
-    total += 2 * E * ld * fb + 3 * ndof * fb + 4 * E * 4;       // r_S, du_S, b, u, r, tables
+    // r_S, du_S, b, u, r; subdomain records and the three element tables
+    total += 2 * E * ld * fb + 3 * ndof * fb + E * (7 * 16 + 3 * 4);
+    if (l == 0 && d.problem == DG_PROBLEM_PUNCTURE) {  // subdomain GMRES: V, Z, D and the small matrices
+      const size_t m = subdomain_iterations;
+      total += E * fb * ((2 * m + 1) * ld + (m + 1) * m + 1 + m);
+    }
     if ((d.mg_levels && l + 1 == d.mg_levels) || (n[0] % 2 && n[1] % 2 && n[2] % 2)) break;
     for (int i = 0; i < 3; ++i)
       if (n[i] % 2 == 0) n[i] /= 2;
@@ -95,8 +106,10 @@ size_t estimate_domain_bytes(const dg_domain_desc& d, int max_iterations, bool l
     // per-subdomain inverses of the finest level plus its class matrices (at most one per element)
     total += 2 * (size_t)d.n[0] * d.n[1] * d.n[2] * nS * nS * fb;
   }
-  // Krylov basis: grown on demand; admission counts up to 64 iterations
-  total += ndof0 * 8 * (2 * (size_t)std::min(max_iterations, 64) + 16);
+  // Krylov basis: grown on demand, 16 columns at least; admission counts up to 64 iterations. Besides, coordinates and
+  // mass (4), Krylov work (6), a captured solve's vectors (5), the host call's (3), the puncture's fields (4)
+  total += ndof0 * 8 * (2 * (size_t)std::min(std::max(max_iterations, 16), 64) + 1 + 18 +
+                        (d.problem == DG_PROBLEM_PUNCTURE ? 4 : 0));
   return total + build_peak + (8u << 20);
 }
 
@@ -295,7 +308,8 @@ dg_status elliptic_serve_submit(dg_server* srv, const dg_request* req, uint64_t*
   if (d.problem == DG_PROBLEM_POISSON && !req->f_host) return DG_ERR_INVALID_ARG;
   const int max_it = req->opts.max_iterations > 0 ? req->opts.max_iterations : 200;
   if (req->opts.subdomain_solver != 0 && req->opts.subdomain_solver != 1) return DG_ERR_INVALID_ARG;
-  const size_t bytes = dg::estimate_domain_bytes(d, max_it, req->opts.subdomain_solver == 1);
+  const size_t bytes = dg::estimate_domain_bytes(
+      d, max_it, req->opts.subdomain_solver == 1, req->opts.subdomain_iterations > 0 ? req->opts.subdomain_iterations : 3);
   Job* job = new (std::nothrow) Job();
   if (!job) return DG_ERR_OOM;
   job->req = *req;

@@ -849,7 +849,8 @@ size_t domain_device_bytes(const dg_domain* dom) {
              dom->r.bytes() + dom->du.bytes() + dom->ut.bytes() + dom->rt.bytes() + dom->tmp.bytes() +
              dom->partial.bytes() + dom->dots.bytes() + dom->vin32.bytes() + dom->shares64.bytes() +
              dom->shares32.bytes() + dom->orient_aff.bytes() + dom->vin64.bytes() +
-             dom->vout64.bytes() + dom->err_flag.bytes();
+             dom->vout64.bytes() + dom->err_flag.bytes() + dom->kst.bytes() + dom->kbuf.bytes() + dom->kb.bytes() +
+             dom->kx.bytes() + dom->zfix.bytes() + dom->host_f.bytes() + dom->host_b.bytes() + dom->host_u.bytes();
   for (const auto& L : dom->levels) {
     const auto& sw = L.sw;
     b += L.geo64.bytes() + L.geo32.bytes() + L.face64.bytes() + L.face32.bytes() + L.trace64.bytes() +
@@ -859,7 +860,8 @@ size_t domain_device_bytes(const dg_domain* dom) {
          sw.inv32.bytes() + sw.inv16.bytes() + sw.inv16_scale.bytes() + sw.tiles.bytes() + sw.tiles_tc[0].d.bytes() +
          sw.tiles_tc[1].d.bytes() +
          sw.units.bytes() + sw.bar.bytes() + sw.inv_digits.bytes() + sw.inv_row_exp.bytes() + sw.x_digits.bytes() +
-         sw.x_exp.bytes() + sw.inv_hexp.bytes() + sw.tiles_f64.bytes();
+         sw.x_exp.bytes() + sw.inv_hexp.bytes() + sw.tiles_f64.bytes() + sw.kchunks16.bytes() + sw.kchunks32.bytes() +
+         sw.kchunks64.bytes();
     for (auto* p : {&L.w64.b, &L.w64.u, &L.w64.r, &L.w64.rS, &L.w64.duS, &L.w64.gV, &L.w64.gZ, &L.w64.gD,
                     &L.w64.gH, &L.w64.linA, &L.w64.linv})
       b += p->bytes();

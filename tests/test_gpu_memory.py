@@ -1,13 +1,20 @@
-"""Device memory: what a domain takes beyond its vectors is given back when a call needs it."""
+"""Device memory: what a domain takes beyond its vectors is given back when a call needs it, and the server admits a
+request only where all that its domain will hold fits the budget."""
+import ctypes as C
 import os
 import subprocess
 import sys
 
+import numpy as np
 import pytest
+
+import workloads
+from gpu_util import rand
 
 pytestmark = pytest.mark.gpu
 
-pytest.importorskip("paper_2111_06767_gb300")
+dgg = pytest.importorskip("paper_2111_06767_gb300")
+from paper_2111_06767_gb300 import _native as nat  # noqa: E402
 
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
@@ -59,3 +66,42 @@ def test_a_solve_that_needs_the_memory_gets_that_of_the_digit_slices(tmp_path):
     f.write_text(_SCRIPT)
     r = subprocess.run([sys.executable, str(f), ROOT], timeout=600, capture_output=True, text=True)
     assert r.returncode == 0, r.stderr[-2000:]
+
+
+def _held(d):
+    lay = nat.dg_layout()
+    assert dgg._lib.dg_domain_layout(d._h, C.byref(lay)) == nat.DG_OK
+    return int(lay.device_bytes)
+
+
+@pytest.mark.parametrize("kind,n,N,precision,max_it", [
+    ("poisson", (24, 24, 24), 2, "mixed", 1), ("poisson", (24, 24, 24), 2, "fp64", 1), ("poisson", (9, 8, 7), 6, "mixed", 3),
+    ("poisson", (6, 5, 4), 7, "fp64", 64), ("coef", (12, 12, 12), 2, "mixed", 2), ("coef", (4, 4, 4), 5, "fp64", 2),
+    ("puncture", (8, 8, 8), 5, "mixed", 2), ("puncture", (4, 4, 4), 4, "fp64", 20)])
+def test_a_budget_below_what_the_domain_holds_refuses_the_request(kind, n, N, precision, max_it):
+    """The admission estimate is an upper bound: a domain that has solved as the server's do (three times, so that it
+    holds the captured solve as well) holds no more, and a budget one byte below that is refused."""
+    m = n[0] * n[1] * n[2] * N**3
+    more = {}
+    if kind == "coef":
+        more["coef"] = 1.0 + 0.2 * rand(950, (m,))
+    if kind == "puncture":
+        more.update(problem="puncture", punctures=workloads.BINARY_PUNCTURES, lower=(-20.0,) * 3, upper=(20.0,) * 3)
+    box = dict(lower=(-1.0,) * 3, upper=(1.0,) * 3)
+    box.update(more)
+    f = None if kind == "puncture" else rand(951, (m,))
+    opts = dgg.solve_opts(max_iterations=max_it)
+    overlap = min(2, N - 1)
+    d = dgg.Domain(n=n, N=N, precision=precision, overlap=overlap, gemm="simt" if precision == "fp64" else "default", **box)
+    for _ in range(3):
+        try:
+            d.solve_host(f, np.zeros(m), tol=1e-10, opts=opts)
+        except nat.NativeError:
+            pass  # so few iterations need not converge
+    desc = dgg.make_desc(n=n, N=N, precision=precision, overlap=overlap, **box)
+    srv = dgg.Server(max_active=1, n_streams=1, memory_budget_bytes=_held(d) - 1)
+    try:
+        with pytest.raises(nat.NativeError):
+            srv.submit(desc, f, opts=opts)
+    finally:
+        srv.close()
