@@ -406,16 +406,21 @@ void launch_subdomain_records(const SubdomainGeom& g, const int* col_of_elem, co
   DG_LAUNCHED(1);
 }
 
+// One thread per point in CTAs of 256: up to 2^31 - 1 points, so the last CTA's threads go beyond an int.
+constexpr unsigned point_blocks(int points) { return ((unsigned)points + 255u) / 256u; }
+static_assert(point_blocks(std::numeric_limits<int>::max()) == 1u << 23 && (1u << 23) * 256u > (1u << 31) - 1u,
+              "CTAs and thread numbers of the largest problem");
+
 template <int N, typename T>
 __global__ void __launch_bounds__(256) gather_kernel(SubdomainGeom g, const T* __restrict__ r,
                                                      const int4* __restrict__ rec, T* __restrict__ rS) {
   constexpr int N3 = N * N * N;
-  const int t = blockIdx.x * 256 + threadIdx.x;
+  const unsigned t = blockIdx.x * 256u + threadIdx.x;
   pdl_launch_dependents();
   pdl_wait();
-  if (t >= g.E * N3) return;
-  const int e = t / N3;
-  gather_point<N, T>(g, rec, r[t], rS, e, t - e * N3);
+  if (t >= (unsigned)(g.E * N3)) return;
+  const int e = (int)t / N3;
+  gather_point<N, T>(g, rec, r[t], rS, e, (int)t - e * N3);
 }
 
 // u += sum_S R_S^T w_S du_S with du_S = X (m = 0), or du_S = sum_{c < m} y[column][c] X_c, the X_c
@@ -426,14 +431,14 @@ __global__ void __launch_bounds__(256) scatter_kernel(SubdomainGeom g, const T* 
                                                       const int4* __restrict__ rec, const T* __restrict__ shares,
                                                       T* __restrict__ u, int u_zero) {
   constexpr int N3 = N * N * N;
-  const int t = blockIdx.x * 256 + threadIdx.x;
+  const unsigned t = blockIdx.x * 256u + threadIdx.x;
   pdl_launch_dependents();
-  const bool act = t < g.E * N3;
-  const int e = act ? t / N3 : 0;
+  const bool act = t < (unsigned)(g.E * N3);
+  const int e = act ? (int)t / N3 : 0;
   int64_t idx[SL];
   int col[SL];
   T w[SL], v[SL];
-  scatter_look_up<N, SL, T>(g, rec, shares, e, act ? t - e * N3 : 0, idx, col, w);
+  scatter_look_up<N, SL, T>(g, rec, shares, e, act ? (int)t - e * N3 : 0, idx, col, w);
   pdl_wait();
   if (!act) return;
   const T u0 = u_zero ? T(0) : u[t];
@@ -459,7 +464,7 @@ __global__ void __launch_bounds__(256) scatter_kernel(SubdomainGeom g, const T* 
 template <int N, typename T, int SL>
 void launch_scatter_n(const SubdomainGeom& g, const T* X, const T* y, int m, int64_t stride, const int4* rec,
                       const T* shares, T* u, int u_zero, cudaStream_t s) {
-  const dim3 grid((g.E * N * N * N + 255) / 256);
+  const dim3 grid(point_blocks(g.E * N * N * N));
   auto k = m == 0 ? scatter_kernel<N, T, 0, SL> : (m == 3 ? scatter_kernel<N, T, 3, SL> : scatter_kernel<N, T, -1, SL>);
   launch_pdl(k, grid, dim3(256), 0, s, g, X, y, m, stride, rec, shares, u, u_zero);
 }
@@ -467,7 +472,7 @@ void launch_scatter_n(const SubdomainGeom& g, const T* X, const T* y, int m, int
 template <typename T>
 void launch_gather(const SubdomainGeom& g, const T* r, const int4* rec, T* rS, cudaStream_t s) {
   if (g.E == 0) return;
-  const dim3 grid((g.E * g.N * g.N * g.N + 255) / 256);
+  const dim3 grid(point_blocks(g.E * g.N * g.N * g.N));
   switch (g.N) {
 #define DG_CASE(NN) \
   case NN: launch_pdl(gather_kernel<NN, T>, grid, dim3(256), 0, s, g, r, rec, rS); break;
