@@ -42,7 +42,7 @@ constexpr int wtab_off(int N) { return N * (N - 1) / 2 - 1; }  // sum_{m=2}^{N-1
 constexpr int kWTab = wtab_off(DG_MAX_N + 1);
 __constant__ float2 cDD4[16], cB4[8];
 __constant__ double cW64[kWTab];
-__constant__ float cW32[kWTab];
+__constant__ float cW32[kWTab], cWlo32[kWTab];  // value and rounding error
 
 // Tables of the direction-by-direction kernel (dir_apply.cuh)
 __constant__ double2 cPQ64[kDirPairs], cQP64[kDirPairs];
@@ -57,6 +57,7 @@ struct DirTab<N, double> {
   static __device__ __forceinline__ double2 QP(int i) { return cQP64[i]; }
   static __device__ __forceinline__ double vec(int i) { return cV64[i]; }
   static __device__ __forceinline__ double w(int l) { return cW64[wtab_off(N) + l]; }
+  static __device__ __forceinline__ double w_lo(int) { return 0.0; }
 };
 template <int N>
 struct DirTab<N, float> {
@@ -64,6 +65,7 @@ struct DirTab<N, float> {
   static __device__ __forceinline__ float2 QP(int i) { return cQP32[i]; }
   static __device__ __forceinline__ float vec(int i) { return cV32[i]; }
   static __device__ __forceinline__ float w(int l) { return cW32[wtab_off(N) + l]; }
+  static __device__ __forceinline__ float w_lo(int l) { return cWlo32[wtab_off(N) + l]; }
 };
 
 __device__ __forceinline__ void row4_g(const float* __restrict__ p, float (&r)[4]) {
@@ -477,8 +479,8 @@ bool launch_elem4(const ApplyArgs<float>& A, int* err, cudaStream_t s) {
 // What bounds it: in FP64 the FP64 pipe (about 12.5 N + 40 operations per point and direction line of
 // N, two thirds of them the even-odd contractions, at 75-85 % of the probed 0.6 T/s); in FP32 the L1
 // data pipe (81 % busy at N = 8, issue slots 71 %, DRAM 26 %). Measured, 48^3 elements at N = 8: FP32
-// 370 -> 197 us, FP64 7.54 -> 5.13 ms; 37 x 41 x 29 at N = 7: FP32 162 -> 79 us; 43^3 at N = 9: FP64
-// 9.71 -> 5.91 ms; 16^3 at N = 6: FP64 128 -> 94 us (against one x-line per thread with the y- and
+// 370 -> 201 us; 37 x 41 x 29 at N = 7: FP32 162 -> 80 us; 43^3 at N = 9: FP64
+// 9.71 -> 5.66 ms; 16^3 at N = 6: FP64 128 -> 90 us (against one x-line per thread with the y- and
 // z-contractions read from shared memory, and in FP32 against blocks of such lines).
 template <int N, typename T, int EPB>
 __global__ void __launch_bounds__(EPB* N* N) apply_dir_kernel(const ApplyArgs<T> A) {
@@ -565,7 +567,7 @@ template <> struct DirEpb<10> { static constexpr int s = 1, m = 2, l = 4, p = 1;
 // FP64 at N = 8, 8^3 elements, just above: 33.7 us in bricks, 36.4 side by side), else the middle shape
 // once it gives every SM two bricks. The autotuner times them per level.
 template <int N, typename T>
-void launch_apply_n(const OpGeom<T>& g, const T* D, const T* w, const T* u, const T* diag, const T* b, T* out,
+void launch_apply_n(const OpGeom<T>& g, const Pair<T>* wf, const T* u, const T* diag, const T* b, T* out,
                     const SubdomainOut& so, int variant, int* err, cudaStream_t s) {
   const int E = g.nx * g.ny * g.nz;
   if (E == 0) return;
@@ -573,7 +575,7 @@ void launch_apply_n(const OpGeom<T>& g, const T* D, const T* w, const T* u, cons
   DG_REQUIRE(!(((uintptr_t)u | (uintptr_t)diag | (uintptr_t)b | (uintptr_t)out | (uintptr_t)so.rS) & a),
              "DG apply vectors must be aligned to " + std::to_string(a + 1) + " bytes");
   using DE = DirEpb<N>;
-  const ApplyArgs<T> A{g, D, w, u, diag, b, out, E, static_cast<T*>(so.rS), so.ld, so.ov, so.rec};
+  const ApplyArgs<T> A{g, wf, u, diag, b, out, E, static_cast<T*>(so.rS), so.ld, so.ov, so.rec};
   if constexpr (N == 4 && std::is_same<T, float>::value) {
     if (variant == 7 && !so.rS && launch_elem4<8, 4, 4>(A, err, s)) return;
   }
@@ -771,9 +773,13 @@ void upload_operator_tables() {
   std::lock_guard<std::mutex> lk(mu);
   if (done.count(dev)) return;
   std::vector<double> W(kWTab);
+  std::vector<float> Wlo32(kWTab);
   for (int N = 2; N <= DG_MAX_N; ++N) {
     const LglTables t = make_lgl(N);
-    std::copy(t.w, t.w + N, W.begin() + wtab_off(N));
+    for (int l = 0; l < N; ++l) {
+      W[wtab_off(N) + l] = t.w[l];
+      Wlo32[wtab_off(N) + l] = (float)(t.w[l] - (float)t.w[l]);
+    }
   }
   const LglTables t4 = make_lgl(4);
   const std::vector<float> D4(t4.D, t4.D + 16), W32(W.begin(), W.end());
@@ -785,12 +791,14 @@ void upload_operator_tables() {
     const int h = N / 2, po = dir_pair_off(N), vo = dir_vec_off(N);
     for (int i = 0; i < h; ++i)
       for (int l = 0; l < h; ++l) {
-        const double a = t.D[i * N + l], b = t.D[i * N + N - 1 - l];
-        const int q = po + i * h + l;
-        PQ[q] = make_double2(a - b, a + b);
-        QP[q] = make_double2(a + b, a - b);
-        PQ32[q] = make_float2((float)(a - b), (float)(a + b));
-        QP32[q] = make_float2((float)(a + b), (float)(a - b));
+        const int m = i * N + l, n = i * N + N - 1 - l;  // each sum rounded once
+        const double p = (double)((long double)t.D[m] - t.D[n] + ((long double)t.D_lo[m] - t.D_lo[n]));
+        const double q = (double)((long double)t.D[m] + t.D[n] + ((long double)t.D_lo[m] + t.D_lo[n]));
+        const int at = po + i * h + l;
+        PQ[at] = make_double2(p, q);
+        QP[at] = make_double2(q, p);
+        PQ32[at] = make_float2((float)p, (float)q);
+        QP32[at] = make_float2((float)q, (float)p);
       }
     for (int l = 0; l < N; ++l) V[vo + l] = 2.0 * t.D[(N - 1) * N + l];
     for (int l = 0; l < h && N % 2; ++l) {
@@ -816,23 +824,24 @@ void upload_operator_tables() {
   DG_CUDA(cudaMemcpyToSymbol(cB4, B4, sizeof(B4)));
   DG_CUDA(cudaMemcpyToSymbol(cW64, W.data(), sizeof(double) * kWTab));
   DG_CUDA(cudaMemcpyToSymbol(cW32, W32.data(), sizeof(float) * kWTab));
+  DG_CUDA(cudaMemcpyToSymbol(cWlo32, Wlo32.data(), sizeof(float) * kWTab));
   done.insert(dev);
 }
 
 template <typename T>
-void launch_apply(int N, const OpGeom<T>& g, const T* D, const T* w, const T* u, const T* diag, const T* b, T* out,
+void launch_apply(int N, const OpGeom<T>& g, const Pair<T>* wf, const T* u, const T* diag, const T* b, T* out,
                   cudaStream_t s, const SubdomainOut* so_ptr, int variant, int* err) {
   const SubdomainOut so = so_ptr ? *so_ptr : SubdomainOut{};
   switch (N) {
-    case 2: launch_apply_n<2, T>(g, D, w, u, diag, b, out, so, variant, err, s); break;
-    case 3: launch_apply_n<3, T>(g, D, w, u, diag, b, out, so, variant, err, s); break;
-    case 4: launch_apply_n<4, T>(g, D, w, u, diag, b, out, so, variant, err, s); break;
-    case 5: launch_apply_n<5, T>(g, D, w, u, diag, b, out, so, variant, err, s); break;
-    case 6: launch_apply_n<6, T>(g, D, w, u, diag, b, out, so, variant, err, s); break;
-    case 7: launch_apply_n<7, T>(g, D, w, u, diag, b, out, so, variant, err, s); break;
-    case 8: launch_apply_n<8, T>(g, D, w, u, diag, b, out, so, variant, err, s); break;
-    case 9: launch_apply_n<9, T>(g, D, w, u, diag, b, out, so, variant, err, s); break;
-    case 10: launch_apply_n<10, T>(g, D, w, u, diag, b, out, so, variant, err, s); break;
+    case 2: launch_apply_n<2, T>(g, wf, u, diag, b, out, so, variant, err, s); break;
+    case 3: launch_apply_n<3, T>(g, wf, u, diag, b, out, so, variant, err, s); break;
+    case 4: launch_apply_n<4, T>(g, wf, u, diag, b, out, so, variant, err, s); break;
+    case 5: launch_apply_n<5, T>(g, wf, u, diag, b, out, so, variant, err, s); break;
+    case 6: launch_apply_n<6, T>(g, wf, u, diag, b, out, so, variant, err, s); break;
+    case 7: launch_apply_n<7, T>(g, wf, u, diag, b, out, so, variant, err, s); break;
+    case 8: launch_apply_n<8, T>(g, wf, u, diag, b, out, so, variant, err, s); break;
+    case 9: launch_apply_n<9, T>(g, wf, u, diag, b, out, so, variant, err, s); break;
+    case 10: launch_apply_n<10, T>(g, wf, u, diag, b, out, so, variant, err, s); break;
     default: fail(DG_ERR_INVALID_ARG, "unsupported N");
   }
   DG_LAUNCHED(1);
@@ -846,10 +855,10 @@ int apply_bricks(int N, int variant, int E) {
   return E / (variant == 2 ? m : l)[N - 2];
 }
 
-template void launch_apply<double>(int, const OpGeom<double>&, const double*, const double*, const double*,
-                                   const double*, const double*, double*, cudaStream_t, const SubdomainOut*, int, int*);
-template void launch_apply<float>(int, const OpGeom<float>&, const float*, const float*, const float*, const float*,
-                                  const float*, float*, cudaStream_t, const SubdomainOut*, int, int*);
+template void launch_apply<double>(int, const OpGeom<double>&, const double2*, const double*, const double*,
+                                   const double*, double*, cudaStream_t, const SubdomainOut*, int, int*);
+template void launch_apply<float>(int, const OpGeom<float>&, const float2*, const float*, const float*, const float*,
+                                  float*, cudaStream_t, const SubdomainOut*, int, int*);
 
 // static shared memory of the fused kernel stays within 48 KiB up to N = 8
 bool coarse_smooth_available(int N) { return N >= 2 && N <= 8; }

@@ -114,11 +114,12 @@ struct DirLine {
   __device__ __forceinline__ T upper2() const { return st[0].x - st[0].y; }
 
   // Lifting into (S, T) with the interior and exterior values lo, hi, u0, u1 at the ends and twice the
-  // exterior derivatives G0, G1, then acc = f2 (Dhat vhat + face terms) (FIRST), or acc += it;
-  // f2 = J (2/h_d)^2 / 2. The face terms join after the even and odd parts are recombined: they are
-  // the largest terms of the operator, and through S and T each end would carry the other's rounding.
+  // exterior derivatives G0, G1, then acc = 2 (Dhat vhat + face terms) (FIRST), or acc += q times it;
+  // q = (h_x / h_d)^2, and J (2/h_x)^2 / 2 comes with the weights. The face terms join after the even and odd parts
+  // are recombined, the larger last: they are the largest terms of the operator, and through S and T each
+  // end would carry the other's rounding.
   template <bool FIRST>
-  __device__ __forceinline__ void divergence(T lo, T hi, T u0, T G0, T u1, T G1, T lam, T pen, T f2, T (&acc)[N]) {
+  __device__ __forceinline__ void divergence(T lo, T hi, T u0, T G0, T u1, T G1, T lam, T pen, T q, T (&acc)[N]) {
     const T j0 = u0 - lo, j1 = u1 - hi, d0 = G0 - lower2(), d1 = G1 - upper2();
     st[0].x += lam * (j1 - j0);
     st[0].y -= lam * (j0 + j1);
@@ -135,20 +136,34 @@ struct DirLine {
     for (int i = 0; i < h; ++i) {
       T a = r[i].y + r[i].x, b = r[i].y - r[i].x;
       if (i == 0) {
-        a += pen * j0 - lam * d0;
-        b += pen * j1 + lam * d1;
+        a -= lam * d0;
+        b += lam * d1;
+        a += pen * j0;
+        b += pen * j1;
       }
-      acc[i] = FIRST ? f2 * a : acc[i] + f2 * a;
-      acc[N - 1 - i] = FIRST ? f2 * b : acc[N - 1 - i] + f2 * b;
+      acc[i] = FIRST ? a : acc[i] + q * a;
+      acc[N - 1 - i] = FIRST ? b : acc[N - 1 - i] + q * b;
     }
     if constexpr (odd) {
       T mid = CT::vec(vo + N + h) * st[0].y;
 #pragma unroll
       for (int l = 1; l < h; ++l) mid += CT::vec(vo + N + h + l) * st[l].y;
-      acc[h] = FIRST ? (T(2) * f2) * mid : acc[h] + (T(2) * f2) * mid;
+      acc[h] = FIRST ? T(2) * mid : acc[h] + (T(2) * q) * mid;
     }
   }
 };
+
+// -(wa wk) acc. In FP32 the weights come as value and rounding error: one rounding where the plain products have three
+// and the weights' own. Against 64 bits, N = 4..10, in units of rounding in norm: 0.45-0.55; plain products and the
+// factors J (2/h_d)^2 / 2 inside the sums 0.58-0.96 (an x-line's fluxes weighted and summed one by one: 0.47-0.85).
+// 48^3 at N = 8 199.5 -> 200.7 us, error 9.7e-8 -> 6.1e-8. In FP64, whose pipe the two extra operations a point would load
+// (43^3 at N = 9 5660 -> 6060 us), the values alone: 0.47-0.87 units (before the factors moved 0.58-1.12 and 5900 us).
+__device__ __forceinline__ float weighted(float2 wa, float wk, float wk_lo, float acc) {
+  const float p = wa.x * wk;
+  const float e = fmaf(wa.y, wk, fmaf(wa.x, wk_lo, fmaf(wa.x, wk, -p)));
+  return -fmaf(p, acc, e * acc);
+}
+__device__ __forceinline__ double weighted(double2 wa, double wk, double, double acc) { return -(wa.x * wk) * acc; }
 
 template <typename T, bool L2ONLY>
 __device__ __forceinline__ T gld1(const T* __restrict__ p) {
@@ -194,7 +209,7 @@ __device__ __forceinline__ void apply_dir_block(const ApplyArgs<T>& A, int blk, 
         s_rec[el2][q - el2 * 7] = __ldg(A.rec + (int64_t)(c0 + nx * (c1 + ny * c2)) * 7 + (q - el2 * 7));
     }
   }
-  const T wa = __ldg(A.w + t0) * __ldg(A.w + t1);
+  const typename PairOf<T>::V wa = __ldg(A.wf + t);
   if constexpr (PDL) pdl_wait();
   T v[N];
   if (valid) gld_line<N, T, L2ONLY>(u + (int64_t)e * N3 + t * N, v);
@@ -270,7 +285,7 @@ __device__ __forceinline__ void apply_dir_block(const ApplyArgs<T>& A, int blk, 
   __syncthreads();
   if (valid) {
     take(0, ln, lo, hi, u0, G0, u1, G1);
-    ln.template divergence<true>(lo, hi, u0, G0, u1, G1, g.lam, g.pen, g.f2[0], acc);
+    ln.template divergence<true>(lo, hi, u0, G0, u1, G1, g.lam, g.pen, T(1), acc);
     sst_line<N>(ax + t1 * P + t0 * N, acc);
     // y
 #pragma unroll
@@ -285,7 +300,7 @@ __device__ __forceinline__ void apply_dir_block(const ApplyArgs<T>& A, int blk, 
     take(1, ln, lo, hi, u0, G0, u1, G1);
 #pragma unroll
     for (int l = 0; l < N; ++l) acc[l] = ax[t1 * P + l * N + t0];
-    ln.template divergence<false>(lo, hi, u0, G0, u1, G1, g.lam, g.pen, g.f2[1], acc);
+    ln.template divergence<false>(lo, hi, u0, G0, u1, G1, g.lam, g.pen, g.q[1], acc);
 #pragma unroll
     for (int l = 0; l < N; ++l) ax[t1 * P + l * N + t0] = acc[l];
     // z
@@ -307,11 +322,12 @@ __device__ __forceinline__ void apply_dir_block(const ApplyArgs<T>& A, int blk, 
   take(2, ln, lo, hi, u0, G0, u1, G1);
 #pragma unroll
   for (int l = 0; l < N; ++l) acc[l] = ax[l * P + t];
-  ln.template divergence<false>(lo, hi, u0, G0, u1, G1, g.lam, g.pen, g.f2[2], acc);
-  // A u = -w_i w_j w_k acc (+ diag u): J is in f2
+  ln.template divergence<false>(lo, hi, u0, G0, u1, G1, g.lam, g.pen, g.q[2], acc);
+  // A u = -w_i w_j w_k acc (+ diag u): J (2/h_x)^2 / 2 is in wa
 #pragma unroll
   for (int l = 0; l < N; ++l) {
-    T r = -(wa * CT::w(l)) * acc[l];
+    const int m = l < N - 1 - l ? l : N - 1 - l;  // the weights are symmetric
+    T r = weighted(wa, CT::w(m), CT::w_lo(m), acc[l]);
     if (A.diag) r += __ldg(A.diag + base + l * N2) * v[l];
     acc[l] = A.b ? bl[l] - r : r;
   }
@@ -449,9 +465,8 @@ __device__ __forceinline__ void apply_par_block(const ApplyArgs<T>& A, int blk, 
       u1 = neu ? hi : -hi;
       G1 = neu ? -ln.upper2() : ln.upper2();
     }
-    const T f2 = d == 0 ? g.f2[0] : (d == 1 ? g.f2[1] : g.f2[2]);
     T acc[N];
-    ln.template divergence<true>(lo, hi, u0, G0, u1, G1, g.lam, g.pen, f2, acc);
+    ln.template divergence<true>(lo, hi, u0, G0, u1, G1, g.lam, g.pen, T(1), acc);
     // point (k N + j) N + i at (k N + j) LN + i
     T* dst = sm + d * PS + el * N2 * LN + (d == 0 ? t * LN : (d == 1 ? t1 * N * LN + t0 : t1 * LN + t0));
     const int ds = d == 0 ? 1 : (d == 1 ? LN : N * LN);
@@ -470,8 +485,9 @@ __device__ __forceinline__ void apply_par_block(const ApplyArgs<T>& A, int blk, 
     const int kj = p / N, i = p - kj * N, k = kj / N, j = kj - k * N;
     const int64_t at = (int64_t)e2 * N3 + p;
     const int o = (el2 * N2 + kj) * LN + i;
-    const T acc = sm[o] + sm[PS + o] + sm[2 * PS + o];
-    T val = -(__ldg(A.w + i) * __ldg(A.w + j) * __ldg(A.w + k)) * acc;
+    const T acc = fma(g.q[2], sm[2 * PS + o], fma(g.q[1], sm[PS + o], sm[o]));
+    const typename PairOf<T>::V wk = __ldg(A.wf + N2 + k);
+    T val = weighted(__ldg(A.wf + j * N + i), wk.x, wk.y, acc);
     if (A.diag) val += __ldg(A.diag + at) * __ldg(u + at);
     if (A.b) val = __ldg(A.b + at) - val;
     if (!A.rS) {

@@ -91,6 +91,8 @@ struct Level {
   double h[3] = {0, 0, 0};
   OpGeom<double> g64{};
   OpGeom<float> g32{};
+  DevBuf<double2> wf64;  // the apply's weights (make_weight_pairs)
+  DevBuf<float2> wf32;
   // curved elements: metric, face-node sizes and penalty; face-node normal fluxes and gradient (scratch of
   // every apply)
   DevBuf<double> geo64, face64, trace64, grad64;

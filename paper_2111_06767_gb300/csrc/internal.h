@@ -9,6 +9,7 @@
 #include <functional>
 #include <memory>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "../../include/dg_elliptic.h"
@@ -144,6 +145,7 @@ struct LglTables {
   double x[DG_MAX_N] = {};
   double w[DG_MAX_N] = {};
   double D[DG_MAX_N * DG_MAX_N] = {};        // D[k*N + l] = l_l'(x_k)
+  double D_lo[DG_MAX_N * DG_MAX_N] = {};     // what the rounding to double left of D
   double I_lo[DG_MAX_N * DG_MAX_N] = {};     // child on the lower half: l_j((x_t - 1)/2), [t*N + j]
   double I_hi[DG_MAX_N * DG_MAX_N] = {};     // upper half: l_j((x_t + 1)/2)
 };
@@ -163,11 +165,18 @@ struct OpGeom {
   T sigma[3];    // penalty C N^2 / h_d (Eq. penalty, equal neighbours)
   T lift[3];     // 1 / (w_0 h_d): L = M^-1 ML at a face node is 2 lift[d]
   // constants of the direction-by-direction apply (dir_apply.cuh), rounded once from double
-  T f2[3];       // J (2 / h_d)^2 / 2
+  T q[3];        // (h_x / h_d)^2: weight of direction d's term beside x's
   T lam;         // 1 / (2 w_0)
   T pen;         // 2 Jf_d (sigma_d - lift_d) / (J w_0 (2 / h_d)^2) = (C N^2 - 1 / w_0) / w_0, the same for every d
   int neumann;   // bit f: box face f (= 2 d + side) is homogeneous Neumann, else Dirichlet
 };
+
+template <typename T>
+using Pair = typename std::conditional<sizeof(T) == 4, float2, double2>::type;
+// Weights of the direction-by-direction apply as a value and its rounding error: [N^2] J (2 / h_x)^2 / 2 w_a w_b at b N + a,
+// then [N] w_l (see weighted() in dir_apply.cuh).
+template <typename T>
+std::vector<Pair<T>> make_weight_pairs(const double h[3], const LglTables& t);
 
 template <typename T>
 OpGeom<T> make_geom(const int n[3], const double h[3], int N, double penalty, const LglTables& t, int neumann = 0);
@@ -188,8 +197,7 @@ struct SubdomainOut {
 template <typename T>
 struct ApplyArgs {
   OpGeom<T> g;
-  const T* D;
-  const T* w;
+  const Pair<T>* wf;  // make_weight_pairs
   const T* u;
   const T* diag;
   const T* b;
@@ -208,7 +216,7 @@ struct ApplyArgs {
 // gives up; a variant that cannot serve the call runs as 0).
 int apply_bricks(int N, int variant, int E);  // full bricks of E elements in shape 2 or 3
 template <typename T>
-void launch_apply(int N, const OpGeom<T>& g, const T* D, const T* w, const T* u, const T* diag, const T* b, T* out,
+void launch_apply(int N, const OpGeom<T>& g, const Pair<T>* wf, const T* u, const T* diag, const T* b, T* out,
                   cudaStream_t s, const SubdomainOut* so = nullptr, int variant = 0, int* err = nullptr);
 
 // Build explicit subdomain matrices A_S for a set of classes (column-major == row-major by symmetry).

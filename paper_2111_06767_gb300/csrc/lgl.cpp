@@ -87,9 +87,11 @@ LglTables make_lgl(int N) {
       if (l == k) continue;
       long double v = (b[l] / b[k]) / (x[k] - x[l]);
       t.D[k * N + l] = (double)v;
+      t.D_lo[k * N + l] = (double)(v - t.D[k * N + l]);
       diag -= v;
     }
     t.D[k * N + k] = (double)diag;
+    t.D_lo[k * N + k] = (double)(diag - t.D[k * N + k]);
   }
   for (int tt = 0; tt < N; ++tt) {
     long double lo = 0.5L * (x[tt] - 1.0L), hi = 0.5L * (x[tt] + 1.0L);
@@ -117,14 +119,28 @@ OpGeom<T> make_geom(const int n[3], const double h[3], int N, double penalty, co
     g.Jf[d] = (T)jf;
     g.sigma[d] = (T)(penalty * (double)N * (double)N / h[d]);
     g.lift[d] = (T)(1.0 / (t.w[0] * h[d]));
-    g.f2[d] = (T)(0.5 * (h[0] * h[1] * h[2] / 8.0) * (2.0 / h[d]) * (2.0 / h[d]));
+    g.q[d] = (T)((h[0] / h[d]) * (h[0] / h[d]));
   }
   g.lam = (T)(0.5 / t.w[0]);
-  // the penalty term is the largest of the operator and is multiplied by the rounded w_0 at the end:
-  // divided by that value, so that its weight is exact
-  g.pen = (T)((penalty * (double)N * (double)N - 1.0 / t.w[0]) / (double)(T)t.w[0]);
+  g.pen = (T)((penalty * (double)N * (double)N - 1.0 / t.w[0]) / t.w[0]);
   return g;
 }
+
+template <typename T>
+std::vector<Pair<T>> make_weight_pairs(const double h[3], const LglTables& t) {
+  std::vector<Pair<T>> v;
+  auto push = [&](long double x) {
+    const T hi = (T)x;
+    v.push_back(Pair<T>{hi, (T)(x - hi)});
+  };
+  const long double f = (long double)h[1] * h[2] / (4.0L * h[0]);  // J (2 / h_x)^2 / 2
+  for (int b = 0; b < t.N; ++b)
+    for (int a = 0; a < t.N; ++a) push(f * t.w[a] * t.w[b]);
+  for (int l = 0; l < t.N; ++l) push(t.w[l]);
+  return v;
+}
+template std::vector<Pair<double>> make_weight_pairs<double>(const double*, const LglTables&);
+template std::vector<Pair<float>> make_weight_pairs<float>(const double*, const LglTables&);
 
 template OpGeom<double> make_geom<double>(const int*, const double*, int, double, const LglTables&, int);
 template OpGeom<float> make_geom<float>(const int*, const double*, int, double, const LglTables&, int);

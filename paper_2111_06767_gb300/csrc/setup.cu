@@ -525,6 +525,8 @@ void domain_setup(dg_domain* dom) {
     L.ndof = (int64_t)L.E * N * N * N;
     L.g64 = make_geom<double>(L.n, L.h, N, d.penalty, t, d.neumann_faces);
     L.g32 = make_geom<float>(L.n, L.h, N, d.penalty, t, d.neumann_faces);
+    upload(L.wf64, make_weight_pairs<double>(L.h, t), s);
+    upload(L.wf32, make_weight_pairs<float>(L.h, t), s);
     dom->levels.push_back(std::move(L));
     if ((int)dom->levels.size() == (d.mg_levels ? d.mg_levels : DG_MAX_LEVELS)) break;
     if (n[0] % 2 && n[1] % 2 && n[2] % 2) break;
@@ -853,7 +855,7 @@ size_t domain_device_bytes(const dg_domain* dom) {
              dom->kx.bytes() + dom->zfix.bytes() + dom->host_f.bytes() + dom->host_b.bytes() + dom->host_u.bytes();
   for (const auto& L : dom->levels) {
     const auto& sw = L.sw;
-    b += L.geo64.bytes() + L.geo32.bytes() + L.face64.bytes() + L.face32.bytes() + L.trace64.bytes() +
+    b += L.wf64.bytes() + L.wf32.bytes() + L.geo64.bytes() + L.geo32.bytes() + L.face64.bytes() + L.face32.bytes() + L.trace64.bytes() +
          L.trace32.bytes() + L.grad64.bytes() + L.grad32.bytes();
     b += sw.rec.bytes() + sw.col_of_elem.bytes() + sw.class_of_col.bytes() + sw.xform_of_elem.bytes() +
          sw.inv64.bytes() +

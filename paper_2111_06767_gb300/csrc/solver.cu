@@ -93,7 +93,7 @@ void apply_level(dg_domain* dom, int level, const double* u, double* out, const 
   const double* diag = (with_lin && level == 0 && dom->lin_set) ? dom->lin64.get() : nullptr;
   PhaseScope ps(dom->prof, DG_PHASE_APPLY_FP64, s, apply_bytes(L.ndof, 8, b, diag), apply_flops(L.ndof, dom->N));
   auto run = [&](int v) {
-    launch_apply<double>(dom->N, L.g64, dom->D64.get(), dom->w64.get(), u, diag, b, out, s, so, v,
+    launch_apply<double>(dom->N, L.g64, L.wf64.get(), u, diag, b, out, s, so, v,
                          dom->err_flag.get());
   };
   run(apply_variant<double>(dom, L, so != nullptr, run, s));
@@ -111,7 +111,7 @@ void apply_level_f32(dg_domain* dom, int level, const float* u, float* out, cons
   const float* diag = (with_lin && level == 0 && dom->lin_set && dom->lin32.get()) ? dom->lin32.get() : nullptr;
   PhaseScope ps(dom->prof, DG_PHASE_APPLY_FP32, s, apply_bytes(L.ndof, 4, b, diag), apply_flops(L.ndof, dom->N));
   auto run = [&](int v) {
-    launch_apply<float>(dom->N, L.g32, dom->D32.get(), dom->w32.get(), u, diag, b, out, s, so, v,
+    launch_apply<float>(dom->N, L.g32, L.wf32.get(), u, diag, b, out, s, so, v,
                         dom->err_flag.get());
   };
   run(apply_variant<float>(dom, L, so != nullptr, run, s));
@@ -376,7 +376,7 @@ void schwarz_smooth(dg_domain* dom, int level, const T* b, T* u, int iterations,
       // all steps of this call in one cooperative launch
       CoarseArgs a{};
       const float* diag = (level == 0 && dom->lin_set && dom->lin32.get()) ? dom->lin32.get() : nullptr;
-      a.ap = ApplyArgs<float>{L.g32, dom->D32.get(), dom->w32.get(), u, diag, b, nullptr, L.E, W.rS.get(), sw.ld,
+      a.ap = ApplyArgs<float>{L.g32, L.wf32.get(), u, diag, b, nullptr, L.E, W.rS.get(), sw.ld,
                               dom->desc.overlap, sw.rec.get()};
       a.sg = sw.geom;
       a.shares = dom->shares32.get();
