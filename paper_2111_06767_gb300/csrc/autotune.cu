@@ -85,7 +85,7 @@ AllocStreamScope::~AllocStreamScope() { tl_alloc_stream = prev; }
 
 // Off by default for every launch: on levels with long kernels the dependent CTAs only hold SMs that
 // other work would use. DG_PDL=1 turns it on everywhere; a PdlScope turns it on for the launches made
-// inside it on this thread (levels small enough to gain, see level_pdl in solver.cu).
+// inside it on this thread (the levels that gain, see level_pdl in solver.cu).
 namespace {
 thread_local int tl_pdl_scope = 0;
 }

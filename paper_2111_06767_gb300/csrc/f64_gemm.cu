@@ -545,6 +545,12 @@ void launch_column_digits(const double* X, int n_cols, int ld, const int* hexp, 
 
 }  // namespace
 
+int f64_default_split(int n_tiles, int ld) {
+  int split = 1;
+  while (split < 8 && n_tiles * split * 2 <= 152 && (ld + BK - 1) / BK / (split * 2) >= 1) split *= 2;
+  return split;
+}
+
 int f64_digits_for(int range) {
   for (int S : {12, 13, 14})
     if (range <= 7 * S - 54) return S;
@@ -587,11 +593,7 @@ void make_f64_maps(F64Maps& m, int digits, const uint16_t* inv, int n_classes, c
 void launch_f64_gemm(int digits, const F64Maps& maps, const int* inv_exp, const int* x_exp, double* Y, int ld,
                      const int4* d_tiles, int n_tiles, const int* d_kchunks, int* err, cudaStream_t s, int split) {
   if (n_tiles == 0) return;
-  const int nk = (ld + BK - 1) / BK;
-  if (split == 0) {
-    split = 1;
-    while (split < 8 && n_tiles * split * 2 <= 152 && nk / (split * 2) >= 1) split *= 2;
-  }
+  if (split == 0) split = f64_default_split(n_tiles, ld);
   DG_REQUIRE(split == 1 || split == 2 || split == 4 || split == 8, "GEMM split must be 1, 2, 4 or 8");
   auto run = digits == 12 ? launch_gemm<12> : (digits == 13 ? launch_gemm<13> : launch_gemm<14>);
   run(maps, inv_exp, x_exp, Y, ld, d_tiles, n_tiles, d_kchunks, err, s, split);

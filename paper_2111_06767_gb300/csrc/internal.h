@@ -280,6 +280,7 @@ void launch_class_gemm_tc(const float* inv, int n_classes, const float* X, float
                           float alpha, cudaStream_t s, int split = 0);
 int tc_tile_width_code(int columns);  // smallest width that holds that many columns (at most 128)
 int tc_tile_width(int code);
+int tc_default_split(int n_tiles, int ld);  // what split 0 stands for
 // Splits the tensor-core GEMM accepts for this shape (each CTA keeps >= 4 K chunks).
 std::vector<int> tc_gemm_splits(int ld);
 
@@ -289,6 +290,7 @@ std::vector<int> tc_gemm_splits(int ld);
 void launch_f64_equilibrate(const double* inv, double alpha, int n_classes, int ld, int* hexp, int* range,
                             cudaStream_t s);
 int f64_digits_for(int range);
+int f64_default_split(int n_tiles, int ld);  // what split 0 stands for
 // The digits of alpha times the inverses [class][digit][ld][ld] (BF16) and their row exponents [class][ld]; the digits
 // [digit][column][ld] and exponents of the columns of X.
 void launch_f64_inverse_digits(int digits, const double* inv, double alpha, int n_classes, int ld, const int* hexp,

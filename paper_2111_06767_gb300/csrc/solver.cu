@@ -311,10 +311,14 @@ void class_gemm<float>(dg_domain* dom, Level& L, const float* X, float* Y, cudaS
       L.gemm_split = pick;
     }
     // Many solves at once: the tuned K split is the one with the shortest launch on an idle GPU, and each
-    // further CTA of a cluster costs its fixed part of the others' time. 20 uneven solves in one graph: tuned
-    // splits 21.1 ms, 1 20.7, 2 19.8, 4 22.5. A pinned split stays.
+    // further CTA of a cluster costs its fixed part of the others' time, so it is at most 2 there (20 uneven solves:
+    // 15.0 -> 14.0 ms; a level that fills the GPU by itself stays unsplit: 8 of 12^3, N = 6 15.9 ms tuned, 15.0
+    // capped, 17.5 with 2 everywhere). A pinned split stays.
     int shape = L.gemm_split;
-    if (gpu_is_shared() && (sw.ld / 32) / 2 >= 4 && !std::getenv("DG_GEMM_SPLIT")) shape = (shape & kWide) | 2;
+    if (gpu_is_shared() && !std::getenv("DG_GEMM_SPLIT")) {
+      const int split = shape & 15 ? shape & 15 : tc_default_split(sw.tiles_tc[shape & kWide ? 1 : 0].n, sw.ld);
+      shape = (shape & kWide) | std::min(split, 2);
+    }
     run(shape);
   } else
     simt_class_gemm<float>(L, sw.inv32.get(), X, Y, (float)sw.inv_scale, s);
@@ -343,17 +347,19 @@ void gather_linearization(dg_domain* dom, cudaStream_t s) {
 // Levels with at most this many elements are smoothed by the fused cooperative kernel (MIXED).
 constexpr int kCoarseFusedElems = 64;
 
-// Levels whose kernels are launched with programmatic dependent launch: those where each kernel is a
-// short latency chain, so that the next one's launch, set-up and first tiles of the inverse overlap it.
-// Above these sizes the waiting CTAs cost more than they hide. Mixed solve, 8^3 elements at N = 8: coarse
-// levels only 4.03 ms, all three levels 3.96; 20 uneven solves in one graph 23.2 and 22.5 ms; punctures with
-// 16^3 elements on the finest level 14.74 and 14.79. FP64 steps (tensor-core product, one CTA per SM): at 8
-// elements of N = 8 29.4 -> 27.0 us, at 64 elements 44.7 -> 67.8. DG_PDL_COARSE: 0 none, 2 every level.
+// Levels whose kernels are launched with programmatic dependent launch, so that a kernel's launch, set-up and first
+// tiles of the inverse overlap the one before it. FP32: every level (a V-cycle of one level with and without it,
+// 512 to 64,000 elements, N = 4..8: 0.81-0.98 of the time, 32^3 at N = 6 1169 and 1193 us). FP64 on the tensor
+// cores, whose product takes an SM per CTA: while its CTAs and the slicing's (one per element) are at most 100, since more
+// wait for each other's SMs (64 + 27 CTAs 0.88 of the time without, 80 + 12 0.92, 32 + 64 0.93, 96 + 18 1.01, 96 +
+// 27 1.21, 64 + 64 1.40, 96 + 36 1.76). FP64 on the CUDA cores: none. DG_PDL_COARSE: 0 none, 2 every level.
 template <typename T>
 bool level_pdl(const Level& L) {
   const int mode = pdl_vcycle_mode();
   if (mode == 0 || (sizeof(T) == 8 && !L.sw.f64_tc)) return false;
-  return mode >= 2 || L.E <= (sizeof(T) == 4 ? 1024 : 32);
+  if (mode >= 2 || sizeof(T) == 4) return true;
+  const int split = L.f64_split > 0 ? L.f64_split : f64_default_split(L.sw.n_tiles_f64, L.sw.ld);
+  return L.sw.n_tiles_f64 * split + L.E <= 100;
 }
 
 // gathered: r_S holds R_S b already (u_is_zero).
@@ -1110,7 +1116,10 @@ dg_batch* batch_create(dg_domain* const* doms, const double* const* b, double* c
   cudaGraph_t graph = nullptr;
   DG_CUDA(cudaGraphCreate(&graph, 0));
   try {
-    const SharedGpuScope shared(count >= 4);
+    // From 5 solves on, where capped splits gain for all but the smallest solves (equal solves of 2^3 to 12^3 elements,
+    // N = 5..8, against tuned splits: 4 solves 0.95-1.06 of the time, 5 0.91-1.05, 8 0.85-1.02, 16 0.87-1.03; the
+    // largest figure of each row is 2^3 at N = 6).
+    const SharedGpuScope shared(count >= 5);
     // Largest solves first: the branches queue on fewer hardware queues than there are solves, and a long one
     // that starts late runs on alone. 20 uneven solves: as given 19.7 ms, smallest first 19.4, largest first 19.0.
     std::vector<int> order(count);

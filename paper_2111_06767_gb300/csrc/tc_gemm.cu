@@ -262,6 +262,14 @@ int tc_tile_width_code(int columns) {
 }
 int tc_tile_width(int code) { return tile_width(code); }
 
+// Split K over a cluster of `split` CTAs so that the launch fills one wave of the co-resident CTAs, keeping >= 4 K
+// chunks each.
+int tc_default_split(int n_tiles, int ld) {
+  int split = 1;
+  while (split < 8 && n_tiles * split * 2 <= 2 * 152 && ld / BK / (split * 2) >= 4) split *= 2;
+  return split;
+}
+
 void launch_class_gemm_tc(const float* inv, int n_classes, const float* X, float* Y, int ld, int n_cols,
                           const int4* d_tiles, int n_tiles, int width_mask, const int* d_kchunks, int* err,
                           float alpha, cudaStream_t s, int split) {
@@ -292,13 +300,8 @@ void launch_class_gemm_tc(const float* inv, int n_classes, const float* X, float
       done.insert(dev);
     }
   }
-  // Default: split K over a cluster of `split` CTAs so that the launch fills one wave of the
-  // co-resident CTAs, keeping >= 4 K chunks each.
   const int nk = ld / BK;
-  if (split == 0) {
-    split = 1;
-    while (split < 8 && n_tiles * split * 2 <= 2 * 152 && nk / (split * 2) >= 4) split *= 2;
-  }
+  if (split == 0) split = tc_default_split(n_tiles, ld);
   DG_REQUIRE(split == 1 || split == 2 || split == 4 || split == 8, "GEMM split must be 1, 2, 4 or 8");
   DG_REQUIRE(split == 1 || nk / split >= 1, "GEMM split larger than the K chunks");
   cudaLaunchConfig_t cfg = {};
