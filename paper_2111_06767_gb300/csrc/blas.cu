@@ -58,10 +58,6 @@ __global__ void f2d_kernel(int64_t n, const float* __restrict__ x, double* __res
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
     y[i] = (double)x[i];
 }
-__global__ void addf2d_kernel(int64_t n, const float* __restrict__ x, double* __restrict__ y) {
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-    y[i] += (double)x[i];
-}
 __global__ void mul_kernel(int64_t n, const double* __restrict__ a, const double* __restrict__ b, double* __restrict__ y) {
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
     y[i] = a[i] * b[i];
@@ -75,11 +71,6 @@ void launch_convert_d2f(int64_t n, const double* x, float* y, cudaStream_t s) {
 void launch_convert_f2d(int64_t n, const float* x, double* y, cudaStream_t s) {
   if (n == 0) return;
   f2d_kernel<<<grid_for(n), kThreads, 0, s>>>(n, x, y);
-  DG_LAUNCHED(1);
-}
-void launch_add_f2d(int64_t n, const float* x, double* y, cudaStream_t s) {
-  if (n == 0) return;
-  addf2d_kernel<<<grid_for(n), kThreads, 0, s>>>(n, x, y);
   DG_LAUNCHED(1);
 }
 void launch_scale_mul(int64_t n, const double* a, const double* b, double* y, cudaStream_t s) {

@@ -390,7 +390,6 @@ template <typename T>
 void launch_fill(int64_t n, T v, T* y, cudaStream_t s);  // y = v
 void launch_convert_d2f(int64_t n, const double* x, float* y, cudaStream_t s);
 void launch_convert_f2d(int64_t n, const float* x, double* y, cudaStream_t s);
-void launch_add_f2d(int64_t n, const float* x, double* y, cudaStream_t s);  // y += x
 void launch_scale_mul(int64_t n, const double* a, const double* b, double* y, cudaStream_t s);  // y = a .* b
 // Deterministic multi-dot: out[k] = sum_i V[k*ld + i] * w[i] for k < m (two-pass reduction).
 void launch_multidot(int64_t n, int m, const double* V, int64_t ld, const double* w, double* partial, double* out,

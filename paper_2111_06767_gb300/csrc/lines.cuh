@@ -21,12 +21,6 @@ template <>
 struct VT<double, 16> { using type = double2; };
 template <>
 struct VT<double, 8> { using type = double; };
-template <>
-struct VT<int, 16> { using type = int4; };
-template <>
-struct VT<int, 8> { using type = int2; };
-template <>
-struct VT<int, 4> { using type = int; };
 
 template <int N, typename T>
 struct LineVec {
@@ -46,31 +40,6 @@ __device__ __forceinline__ void gld_line(const T* __restrict__ p, T (&v)[N]) {
   for (int q = 0; q < L::n; ++q) {
     const typename L::V* vp = reinterpret_cast<const typename L::V*>(p) + q;
     const typename L::V x = L2ONLY ? __ldcg(vp) : __ldg(vp);
-    const T* xs = reinterpret_cast<const T*>(&x);
-#pragma unroll
-    for (int r = 0; r < L::per; ++r) v[q * L::per + r] = xs[r];
-  }
-}
-
-template <int N, typename T>
-__device__ __forceinline__ void gst_line(T* __restrict__ p, const T (&v)[N]) {
-  using L = LineVec<N, T>;
-#pragma unroll
-  for (int q = 0; q < L::n; ++q) {
-    typename L::V x;
-    T* xs = reinterpret_cast<T*>(&x);
-#pragma unroll
-    for (int r = 0; r < L::per; ++r) xs[r] = v[q * L::per + r];
-    reinterpret_cast<typename L::V*>(p)[q] = x;
-  }
-}
-
-template <int N, typename T>
-__device__ __forceinline__ void sld_line(const T* p, T (&v)[N]) {
-  using L = LineVec<N, T>;
-#pragma unroll
-  for (int q = 0; q < L::n; ++q) {
-    const typename L::V x = reinterpret_cast<const typename L::V*>(p)[q];
     const T* xs = reinterpret_cast<const T*>(&x);
 #pragma unroll
     for (int r = 0; r < L::per; ++r) v[q * L::per + r] = xs[r];

@@ -314,7 +314,7 @@ dg_status elliptic_serve_submit(dg_server* srv, const dg_request* req, uint64_t*
   if (!job) return DG_ERR_OOM;
   job->req = *req;
   // FP64 domains of the pool keep the CUDA-core product: requests are admitted, and idle domains kept,
-  // by footprint, and the tensor-core product's digit slices take twice the bytes of the inverses
+  // by footprint, and the tensor-core product's digit slices take three times the bytes of the inverses
   if (d.precision == DG_PRECISION_FP64 && d.subdomain_gemm == DG_GEMM_DEFAULT)
     job->req.domain.subdomain_gemm = DG_GEMM_SIMT;
   job->bytes = bytes;

@@ -155,13 +155,9 @@ void classify_schwarz(dg_domain* dom, Level& L) {
   sw.class_first.assign(nc, 0);
   for (int c = 1; c < nc; ++c) sw.class_first[c] = sw.class_first[c - 1] + sw.class_count[c - 1];
   sw.position.resize(E);
-  std::vector<int> elem_of_col(E);
   {
     std::vector<int> fill = sw.class_first;
-    for (int e = 0; e < E; ++e) {
-      sw.position[e] = fill[sw.class_of[e]]++;
-      elem_of_col[sw.position[e]] = e;
-    }
+    for (int e = 0; e < E; ++e) sw.position[e] = fill[sw.class_of[e]]++;
   }
   // canonical patch of every class (slot 0 centre, 1 + f neighbour across canonical face f)
   sw.patch.assign((size_t)nc * 49, -2);
@@ -284,10 +280,9 @@ void classify_schwarz(dg_domain* dom, Level& L) {
   DG_CUDA(cudaMemsetAsync(sw.bar.get(), 0, sw.bar.bytes(), s));
 }
 
-// Point maps of the 48 subdomain orientations (orientation o = 8 perm + flips: canonical axis a is
-// actual axis kPerms[perm][a], reflected if bit a of flips): map[o][q] = (actual slot << 16) |
-// actual point of canonical subdomain row q; inv[o][slot][p] = canonical row of point p of that
-// actual slot, -1 outside the subdomain.
+// Rows of the 48 subdomain orientations (orientation o = 8 perm + flips: canonical axis a is
+// actual axis kPerms[perm][a], reflected if bit a of flips): inv[o][slot][p] = canonical row of point p of that
+// actual slot, -1 outside the subdomain, and from it the row's affine form per orientation and slot.
 void build_orientation_tables(dg_domain* dom) {
   const int N = dom->N, N2 = N * N, N3 = N2 * N, ov = dom->desc.overlap;
   const int nS = N3 + 6 * ov * N2;
