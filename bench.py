@@ -826,8 +826,8 @@ def run_ours(args):
                  "mixed_vs_fp64_solution_rel_diff": sol_diff, "mixed_speedup": value / value64 / world,
                  "phases_ms": {k: round(v["ms"], 3) for k, v in prof64.items() if v["launches"]},
                  "subdomain_gemm_tflops": fp64_gemm_tflops,
-                 "subdomain_gemm_frac_of_fp64_pipe": fp64_gemm_tflops / FP64_PEAK_TFLOPS,
-                 "subdomain_gemm_unit": "tensor cores: exact digit products, FP64 flops of the product they stand for",
+                 "subdomain_gemm_unit": "tensor cores: 7-bit digits with exact products and sums, FP64 flops of the "
+                                        "product they stand for",
                  "fp64_peak": f"{FP64_PEAK_TFLOPS} TFLOP/s, FP64 FMA rate probed on this pool's GB300"},
         "fcg": fcg,
         "dg_apply": apply,

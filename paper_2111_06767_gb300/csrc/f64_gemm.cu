@@ -27,10 +27,12 @@
 // integer partial sums are added through distributed shared memory, so the result does not depend on
 // the split.
 //
-// What bounds it: the inverses' digits on their way from L2 (24 to 28 bytes an entry; 266 KB a chunk per CTA at 13
-// digits, 4.9 TB/s over all SMs at 8^3 elements, N = 8; the MMAs alone would take 84 us at the cuBLAS rate). 8^3, N = 8
-// (13 digits): 187 us a launch against 1450 us on the CUDA cores; 6 x 8 x 4, N = 5: 26 and 4 us of slicing against 111.
-// With 8 digits, in tiles of up to 48 columns, these took 93 and 20 us: the price of every component's accuracy.
+// What bounds it: the chain inside a CTA. S digit tiles a chunk go through the ring and the MMAs in series, the MMAs wait
+// for the drain of all levels every 256 terms, and a cluster's CTAs for each other: at 8^3 elements, N = 8 (13 digits,
+// split 4, 760 CTAs) the tensor pipe is 36 % busy (43 % on the busiest SM), L2 19 %, DRAM 25 % from cold caches; unsplit
+// (190 CTAs on 152 SMs) 46 % with 81 % on the busiest and 230 us. 8^3, N = 8: 187 us a launch against 1450 us on the CUDA
+// cores; 6 x 8 x 4, N = 5: 26 and 4 us of slicing against 111. With 8 digits, in tiles of up to 48 columns, these took 93
+// and 20 us: the price of every component's accuracy. Tiles ordered longest first: 185 us, no change.
 #include <mutex>
 #include <set>
 
