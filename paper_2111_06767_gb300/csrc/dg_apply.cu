@@ -480,7 +480,7 @@ bool launch_elem4(const ApplyArgs<float>& A, int* err, cudaStream_t s) {
 // N, two thirds of them the even-odd contractions, at 75-85 % of the probed 0.6 T/s); in FP32 the L1
 // data pipe (81 % busy at N = 8, issue slots 71 %, DRAM 26 %). Measured, 48^3 elements at N = 8: FP32
 // 370 -> 201 us; 37 x 41 x 29 at N = 7: FP32 162 -> 80 us; 43^3 at N = 9: FP64
-// 9.71 -> 5.66 ms; 16^3 at N = 6: FP64 128 -> 90 us (against one x-line per thread with the y- and
+// 9.71 -> 5.67 ms; 16^3 at N = 6: FP64 128 -> 92 us (against one x-line per thread with the y- and
 // z-contractions read from shared memory, and in FP32 against blocks of such lines).
 template <int N, typename T, int EPB>
 __global__ void __launch_bounds__(EPB* N* N) apply_dir_kernel(const ApplyArgs<T> A) {

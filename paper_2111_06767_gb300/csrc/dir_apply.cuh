@@ -157,7 +157,7 @@ struct DirLine {
 // and the weights' own. Against 64 bits, N = 4..10, in units of rounding in norm: 0.45-0.55; plain products and the
 // factors J (2/h_d)^2 / 2 inside the sums 0.58-0.96 (an x-line's fluxes weighted and summed one by one: 0.47-0.85).
 // 48^3 at N = 8 199.5 -> 200.7 us, error 9.7e-8 -> 6.1e-8. In FP64, whose pipe the two extra operations a point would load
-// (43^3 at N = 9 5660 -> 6060 us), the values alone: 0.47-0.87 units (before the factors moved 0.58-1.12 and 5900 us).
+// (43^3 at N = 9 5670 -> 6070 us), the values alone: 0.47-0.87 units (before the factors moved 0.58-1.12 and 5900 us).
 __device__ __forceinline__ float weighted(float2 wa, float wk, float wk_lo, float acc) {
   const float p = wa.x * wk;
   const float e = fmaf(wa.y, wk, fmaf(wa.x, wk_lo, fmaf(wa.x, wk, -p)));
@@ -286,6 +286,10 @@ __device__ __forceinline__ void apply_dir_block(const ApplyArgs<T>& A, int blk, 
   if (valid) {
     take(0, ln, lo, hi, u0, G0, u1, G1);
     ln.template divergence<true>(lo, hi, u0, G0, u1, G1, g.lam, g.pen, T(1), acc);
+    if (g.q[0] != T(1)) {
+#pragma unroll
+      for (int l = 0; l < N; ++l) acc[l] *= g.q[0];
+    }
     sst_line<N>(ax + t1 * P + t0 * N, acc);
     // y
 #pragma unroll
@@ -485,7 +489,7 @@ __device__ __forceinline__ void apply_par_block(const ApplyArgs<T>& A, int blk, 
     const int kj = p / N, i = p - kj * N, k = kj / N, j = kj - k * N;
     const int64_t at = (int64_t)e2 * N3 + p;
     const int o = (el2 * N2 + kj) * LN + i;
-    const T acc = fma(g.q[2], sm[2 * PS + o], fma(g.q[1], sm[PS + o], sm[o]));
+    const T acc = fma(g.q[2], sm[2 * PS + o], fma(g.q[1], sm[PS + o], g.q[0] * sm[o]));
     const typename PairOf<T>::V wk = __ldg(A.wf + N2 + k);
     T val = weighted(__ldg(A.wf + j * N + i), wk.x, wk.y, acc);
     if (A.diag) val += __ldg(A.diag + at) * __ldg(u + at);

@@ -165,7 +165,7 @@ struct OpGeom {
   T sigma[3];    // penalty C N^2 / h_d (Eq. penalty, equal neighbours)
   T lift[3];     // 1 / (w_0 h_d): L = M^-1 ML at a face node is 2 lift[d]
   // constants of the direction-by-direction apply (dir_apply.cuh), rounded once from double
-  T q[3];        // (h_x / h_d)^2: weight of direction d's term beside x's
+  T q[3];        // (h_x / h_d)^2, the weight of direction d's term beside x's (so q[0] = 1; very thin elements: see lgl.cpp)
   T lam;         // 1 / (2 w_0)
   T pen;         // 2 Jf_d (sigma_d - lift_d) / (J w_0 (2 / h_d)^2) = (C N^2 - 1 / w_0) / w_0, the same for every d
   int neumann;   // bit f: box face f (= 2 d + side) is homogeneous Neumann, else Dirichlet
@@ -173,7 +173,8 @@ struct OpGeom {
 
 template <typename T>
 using Pair = typename std::conditional<sizeof(T) == 4, float2, double2>::type;
-// Weights of the direction-by-direction apply as a value and its rounding error: [N^2] J (2 / h_x)^2 / 2 w_a w_b at b N + a,
+// Weights of the direction-by-direction apply as a value and its rounding error: [N^2] w_a w_b times x's factor J (2 / h_x)^2 / 2
+// at b N + a (the factor is 1 for very thin elements),
 // then [N] w_l (see weighted() in dir_apply.cuh).
 template <typename T>
 std::vector<Pair<T>> make_weight_pairs(const double h[3], const LglTables& t);

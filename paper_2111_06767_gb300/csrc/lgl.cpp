@@ -103,6 +103,19 @@ LglTables make_lgl(int N) {
   return t;
 }
 
+namespace {
+// J (2 / h_d)^2 / 2, which the apply takes as x's beside the weights and the other directions' ratio to it; where a ratio
+// would leave FP32's range (elements thinner than 1 : 2^60), as 1 beside the weights and each direction's own.
+long double direction_factor(const double h[3], int d) {
+  return (long double)h[0] * h[1] * h[2] / (4.0L * h[d] * h[d]);
+}
+bool far_apart(const double h[3]) {
+  for (int d = 1; d < 3; ++d)
+    if (fabsl(log2l((long double)h[0] / h[d])) > 60.0L) return true;
+  return false;
+}
+}  // namespace
+
 template <typename T>
 OpGeom<T> make_geom(const int n[3], const double h[3], int N, double penalty, const LglTables& t, int neumann) {
   OpGeom<T> g;
@@ -119,7 +132,7 @@ OpGeom<T> make_geom(const int n[3], const double h[3], int N, double penalty, co
     g.Jf[d] = (T)jf;
     g.sigma[d] = (T)(penalty * (double)N * (double)N / h[d]);
     g.lift[d] = (T)(1.0 / (t.w[0] * h[d]));
-    g.q[d] = (T)((h[0] / h[d]) * (h[0] / h[d]));
+    g.q[d] = (T)(far_apart(h) ? direction_factor(h, d) : (long double)(h[0] / h[d]) * (h[0] / h[d]));
   }
   g.lam = (T)(0.5 / t.w[0]);
   g.pen = (T)((penalty * (double)N * (double)N - 1.0 / t.w[0]) / t.w[0]);
@@ -133,7 +146,7 @@ std::vector<Pair<T>> make_weight_pairs(const double h[3], const LglTables& t) {
     const T hi = (T)x;
     v.push_back(Pair<T>{hi, (T)(x - hi)});
   };
-  const long double f = (long double)h[1] * h[2] / (4.0L * h[0]);  // J (2 / h_x)^2 / 2
+  const long double f = far_apart(h) ? 1.0L : direction_factor(h, 0);
   for (int b = 0; b < t.N; ++b)
     for (int a = 0; a < t.N; ++a) push(f * t.w[a] * t.w[b]);
   for (int l = 0; l < t.N; ++l) push(t.w[l]);
