@@ -1109,8 +1109,20 @@ dg_batch* batch_create(dg_domain* const* doms, const double* const* b, double* c
     for (int j = 0; j < i; ++j) DG_REQUIRE(doms[j] != dom, "a domain appears twice in the batch");
     dom->lin_set = false;
     dom->barrier_stall = 0;
-    prepare_solve_graph(dom, bt->cap);
-    warm_solve_kernels(dom);
+  }
+  auto ready = [&] {
+    for (int i = 0; i < count; ++i) {
+      prepare_solve_graph(doms[i], bt->cap);
+      warm_solve_kernels(doms[i]);
+    }
+  };
+  try {
+    ready();
+  } catch (const Error& e) {  // one domain's vectors may need the memory of another's digit slices
+    bool dropped = false;
+    for (int i = 0; i < count && e.status == DG_ERR_OOM; ++i) dropped |= drop_digits(doms[i]);
+    if (!dropped) throw;
+    ready();
   }
   for (int i = 0; i < count; ++i) doms[i]->in_batch = true;
   cudaGraph_t graph = nullptr;

@@ -68,6 +68,41 @@ def test_a_solve_that_needs_the_memory_gets_that_of_the_digit_slices(tmp_path):
     assert r.returncode == 0, r.stderr[-2000:]
 
 
+_BATCH_SCRIPT = r"""
+import ctypes as C, os, sys, torch
+sys.path.insert(0, sys.argv[1]); sys.path.insert(0, sys.argv[1] + "/tests")
+import paper_2111_06767_gb300 as dgg
+from test_gpu_memory import _held
+from gpu_util import rand, rel
+
+shapes = [((8, 8, 8), 4), ((4, 4, 4), 6)]  # the first needs more than its own slices take, the second holds the larger ones
+doms, bs, us, ref = [], [], [], []
+for i, (n, N) in enumerate(shapes):
+    d = dgg.Domain(n=n, N=N)
+    b = torch.from_numpy(rand(941 + i, (d.n_dof,))).cuda()
+    s = dgg.Domain(n=n, N=N, gemm="simt")
+    r = torch.zeros_like(b)
+    s.solve(b, r, tol=1e-10)
+    ref.append(r.cpu().numpy())
+    s.close()
+    d.vcycle(b)
+    doms.append(d); bs.append(b); us.append(torch.zeros_like(b))
+os.environ["DG_ALLOC_LIMIT"] = str(sum(_held(d) for d in doms) + (1 << 20))
+batch = dgg.Batch(doms, bs, us, tol=1e-10)
+for r in batch.run():
+    assert r.relative_residual <= 1e-10
+for u, r in zip(us, ref):
+    assert rel(u.cpu().numpy(), r) < 1e-9
+"""
+
+
+def test_a_batch_takes_the_memory_of_its_other_domains_slices(tmp_path):
+    f = tmp_path / "run.py"
+    f.write_text(_BATCH_SCRIPT)
+    r = subprocess.run([sys.executable, str(f), ROOT], timeout=600, capture_output=True, text=True)
+    assert r.returncode == 0, r.stderr[-2000:]
+
+
 def _held(d):
     lay = nat.dg_layout()
     assert dgg._lib.dg_domain_layout(d._h, C.byref(lay)) == nat.DG_OK
