@@ -622,9 +622,10 @@ void release_digits(SchwarzLevel& sw) {
 
 bool DigitBytes::take(size_t bytes) {
   give();
-  size_t free_b = 0, total = 0;
-  DG_CUDA(cudaMemGetInfo(&free_b, &total));
   std::lock_guard<std::mutex> lk(g_digit_mu);
+  static size_t total = 0;  // asked for once: the call takes as long as several launches
+  size_t free_b = 0;
+  if (total == 0) DG_CUDA(cudaMemGetInfo(&free_b, &total));
   if (g_digit_bytes + bytes > total / 8) return false;
   g_digit_bytes += bytes;
   n = bytes;
@@ -772,11 +773,11 @@ void build_schwarz(dg_domain* dom, Level& L) {
                 (ld > 32 || sw.n_tiles_f64 <= 152);
     if (sw.f64_tc) {
       try {
-        DevBuf<int> range(1);
-        sw.inv_hexp.alloc((size_t)nc * ld);
-        launch_f64_equilibrate(sw.inv64.get(), sw.inv_scale, nc, ld, sw.inv_hexp.get(), range.get(), s);
+        sw.inv_hexp.alloc((size_t)nc * ld + 1);
+        int* range = sw.inv_hexp.get() + (size_t)nc * ld;
+        launch_f64_equilibrate(sw.inv64.get(), sw.inv_scale, nc, ld, sw.inv_hexp.get(), range, s);
         int h_range = 0;
-        DG_CUDA(cudaMemcpyAsync(&h_range, range.get(), sizeof(int), cudaMemcpyDeviceToHost, s));
+        DG_CUDA(cudaMemcpyAsync(&h_range, range, sizeof(int), cudaMemcpyDeviceToHost, s));
         DG_CUDA(cudaStreamSynchronize(s));
         const size_t S = sw.f64_digits = f64_digits_for(h_range);
         sw.f64_tc = S > 0 && sw.digit_bytes.take(2 * S * ((size_t)nc * ld * ld + (size_t)L.E * ld));

@@ -641,7 +641,6 @@ double now_s() {
 
 // Krylov workspace for k iterations: V (k + 1 vectors) and Z (k vectors), grown on demand
 // (doubling, contents kept) so that short solves do not hold a basis sized for the iteration cap.
-void ensure_workspace(dg_domain* dom, int k);
 void grow_workspace(dg_domain* dom, int k) {
   const int64_t n = dom->levels[0].ndof;
   for (DevBuf<double>* v : {&dom->w, &dom->r, &dom->du, &dom->ut, &dom->rt, &dom->tmp})
